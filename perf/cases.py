@@ -269,7 +269,7 @@ def _widths(case):
 
 def _cand_cap(case):
     """Room for every candidate the inputs give, as a program leaves it."""
-    return {"beam": 1 << 17, "beam_host": 1 << 13, "stream": 1 << 14}.get(case["kind"], 1 << 15)
+    return {"beam": 1 << 17, "beam_host": 1 << 13, "stream": 1 << 14, "search": 1 << 16}.get(case["kind"], 1 << 15)
 
 
 # ---------------------------------------------------------------- prepare --
