@@ -121,7 +121,7 @@ int sp_compute_delays(const double *freqs_mhz, int32_t nchan, double tsamp_s,
                       const double *dms, int32_t ndm, int32_t *h_out, int32_t *max_delay);
 
 /* ------------------------------------------- kernel shapes, autotuner --
- * The dedispersion kernel is compiled for SP_DEDISP_NUM_SHAPES tile shapes,
+ * The direct dedispersion kernel is compiled for SP_DEDISP_NUM_SHAPES tile shapes,
  * each a (DM tile, time tile, channel chunk) triple: shape 0 = 32 trial DMs
  * x 512 samples x 8 channels (the shape of sp_plan_create), 1 = 32 x 256 x 8,
  * 2 = 16 x 512 x 4.  A plan is built for one shape (its DM tiles and staging
@@ -129,7 +129,9 @@ int sp_compute_delays(const double *freqs_mhz, int32_t nchan, double tsamp_s,
  * the same DM transform, bit for bit.  Choosing it by measurement has no
  * counterpart in the paper (whose kernels come from its dedispersion
  * library); it exists because the best tile shape depends on the channel
- * count, the DM list and the GPU.
+ * count, the DM list and the GPU.  A plan of shape 0 also holds the tables of
+ * the shared-sum kernel where its trials share enough of their sums, and its
+ * launches then run that kernel (the same transform, bit for bit).
  * sp_dedisp_shape_info: the triple of a shape (out pointers may be NULL).
  * sp_plan_create_shaped: sp_plan_create for a given shape, or for
  *   SP_SHAPE_AUTO: the shape sp_autotune_dedisperse picks with
@@ -163,7 +165,8 @@ int sp_plan_shape(const sp_plan *plan, int32_t *shape, int32_t *ntiles, int32_t 
  * bounds of the bulk copies (inside the staged row of pitch
  * sp_staged_pitch(n_out + max_delay) and inside the raw slot), the four
  * shifted copies inside the copies buffer, and every shared load of the
- * sums inside its channel's copy.  h_report [8] (host): DM tiles, channel
+ * sums inside its channel's copy; for shape 0 also every access of the
+ * shared-sum kernel, and that each trial's rows start at its delays.  h_report [8] (host): DM tiles, channel
  * chunks, copies bytes, raw bytes, dynamic shared memory bytes of the
  * kernel, number of violated conditions (0 for a sound plan), max delay,
  * staged pitch.  Errors: SP_EINVAL (the sp_plan_create argument checks,

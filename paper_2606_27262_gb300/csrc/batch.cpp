@@ -32,9 +32,10 @@ int64_t table_bytes(int32_t nbeams) {
            align256((int64_t)(nbeams + 1) * 8);
 }
 
-// Checks one beam and fills its kernel descriptor; *items = its work items.
+// Checks one beam and fills its kernel descriptor for the direct or the
+// shared-sum kernel; *items = its work items.
 int describe(const sp_plan *p, const uint8_t *staged, int64_t pitch, int64_t n_in, int32_t *out, int64_t n_out,
-             BatchBeamDev &d, int64_t *items) {
+             bool sums, BatchBeamDev &d, int64_t *items) {
     if (!p || !staged || !out || n_in <= 0 || n_out <= 0) return SP_EINVAL;
     if (!on_plan_device(p)) return SP_EINVAL;
     if ((reinterpret_cast<uintptr_t>(staged) & 255) || pitch < dedisp_pitch(n_in) || (pitch & 63)) return SP_EINVAL;
@@ -55,6 +56,11 @@ int describe(const sp_plan *p, const uint8_t *staged, int64_t pitch, int64_t n_i
     d.ntiles = p->ntiles;
     d.ntime = (int32_t)nt;
     *items = (int64_t)p->ntiles * nt;
+    if (sums) {
+        d.sums = p->d_sums;
+        d.ntime = (int32_t)((n_out + kSumTime - 1) / kSumTime);
+        *items = sums_items(p, n_out);
+    }
     return SP_OK;
 }
 
@@ -96,17 +102,30 @@ extern "C" int sp_dedisperse_batch(const sp_batch_beam *h_beams, int32_t nbeams,
     std::vector<BatchBeamDev> dev((size_t)nbeams);
     std::vector<int64_t> begin((size_t)nbeams + 1, 0);
     std::vector<const sp_plan *> plans;
-    for (int32_t b = 0; b < nbeams; ++b) {
-        const sp_batch_beam &x = h_beams[b];
-        int64_t items = 0;
-        const int rc = describe(x.plan, x.d_staged, x.pitch, x.n_in, x.d_out, x.n_out, dev[b], &items);
-        if (rc) return rc;
-        begin[b + 1] = begin[b] + items;
-        plans.push_back(x.plan);
-    }
-    BatchLaunch L{};
-    int rc = launch_geometry(plans, L);
+    std::vector<int64_t> n_outs;
+    auto describe_all = [&](bool sums) {
+        for (int32_t b = 0; b < nbeams; ++b) {
+            const sp_batch_beam &x = h_beams[b];
+            int64_t items = 0;
+            const int rc = describe(x.plan, x.d_staged, x.pitch, x.n_in, x.d_out, x.n_out, sums, dev[b], &items);
+            if (rc) return rc;
+            begin[b + 1] = begin[b] + items;
+        }
+        return (int)SP_OK;
+    };
+    int rc = describe_all(false);
     if (rc) return rc;
+    for (int32_t b = 0; b < nbeams; ++b) {
+        plans.push_back(h_beams[b].plan);
+        n_outs.push_back(h_beams[b].n_out);
+    }
+    const bool sums = sums_pay(plans.data(), n_outs.data(), nbeams);
+    if (sums) rc = describe_all(true);
+    if (rc) return rc;
+    BatchLaunch L{};
+    rc = launch_geometry(plans, L);
+    if (rc) return rc;
+    L.sums = sums;
     uint8_t *w = reinterpret_cast<uint8_t *>(d_work);
     L.nbeams = nbeams;
     L.nitems = begin[nbeams];
@@ -402,16 +421,19 @@ extern "C" int sp_batch_create(const sp_plan *const *plans, int32_t nplans, cons
         std::vector<BatchBeamDev> dev((size_t)n);
         std::vector<int64_t> begin((size_t)n + 1, 0);
         std::vector<const sp_plan *> gp;
+        for (int32_t i = 0; i < n; ++i) gp.push_back(plan_of(b, G.first + i));
+        const bool sums = sums_pay(gp.data(), b->n_out.data() + G.first, n);
         for (int32_t i = 0; i < n && !rc; ++i) {
             const int32_t beam = G.first + i;
             int64_t items = 0;
             rc = describe(plan_of(b, beam), b->d_staged[slot] + b->staged_off[beam], b->pitch[beam], b->n_in[beam],
-                          b->d_dmt[slot] + b->dmt_off[beam], b->n_out[beam], dev[i], &items);
+                          b->d_dmt[slot] + b->dmt_off[beam], b->n_out[beam], sums, dev[i], &items);
             begin[i + 1] = begin[i] + items;
-            gp.push_back(plan_of(b, beam));
         }
         if (!rc) rc = launch_geometry(gp, G.launch);
+        if (!rc && sums) rc = sums_configure();
         if (rc) break;
+        G.launch.sums = sums;
         uint8_t *w = b->d_tables + toff;
         G.launch.nbeams = n;
         G.launch.nitems = begin[n];

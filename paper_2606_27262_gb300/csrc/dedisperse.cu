@@ -1,4 +1,7 @@
-// dedisperse.cu -- brute-force incoherent dedispersion on sm_103a
+// dedisperse.cu -- incoherent dedispersion on sm_103a: staging, the direct
+// kernel, and the choice between it and the shared-sum kernel of
+// dedisp_sums.cu, which forms sums that several trials share once and takes
+// the DM lists where that pays (sums_pay in plan_sums.cpp)
 // (arXiv 2606.27262, Sec. 3.1.1: shift every channel by its Eq.-1 delay and
 // sum, for every trial DM; the result is the DM transform).
 //
@@ -708,7 +711,7 @@ int set_staging_fault(uint32_t extra_bytes, long long wait_limit) {
         cudaGetLastError();
         return SP_ECUDA;
     }
-    return SP_OK;
+    return set_sums_fault(extra_bytes, wait_limit);
 }
 
 int launch_stage_input(const uint8_t *d_in, int64_t n_in, int32_t nchan, uint8_t *d_staged, int64_t pitch,
@@ -729,6 +732,7 @@ int dedisp_configure(const sp_plan *plan) { return configure_shape(plan->shape, 
 
 int launch_dedisperse(const sp_plan *plan, const uint8_t *d_xt, int64_t pitch, int64_t n_out, int32_t *d_out,
                       cudaStream_t stream, int32_t *status) {
+    if (sums_pay(&plan, &n_out, 1)) return launch_dedisperse_sums(plan, d_xt, pitch, n_out, d_out, stream, status);
     int rc = dedisp_configure(plan);
     if (rc) return rc;
     const ShapeKernels &k = kShapes[plan->shape];
@@ -761,6 +765,7 @@ int batch_grid(BatchLaunch &b) {
 }
 
 int launch_dedisperse_batch(const BatchLaunch &b, cudaStream_t stream, bool persistent) {
+    if (b.sums) return launch_dedisperse_sums_batch(b, stream);
     if (b.shape < 0 || b.shape >= kDedispNumShapes || b.grid < 1) return SP_EINVAL;
     const ShapeKernels &k = kShapes[b.shape];
     int64_t grid = std::max<int64_t>(b.nitems, 1);

@@ -3,6 +3,7 @@
 // the binary64 expression is evaluated exactly as written (no fused
 // multiply-add), left to right.
 #include <algorithm>
+#include <atomic>
 #include <climits>
 #include <cmath>
 #include <cstring>
@@ -30,19 +31,33 @@ int compute_delays(const double *freqs, int32_t nchan, double tsamp, const doubl
     if ((int64_t)ndm * nchan > (int64_t)INT32_MAX) return SP_ELIMIT;
     out.resize((size_t)ndm * nchan);
     const double ftop = freqs[0];
-    int32_t mx = 0;
-    for (int32_t d = 0; d < ndm; ++d) {
-        const double dm = dms[d];
-        for (int32_t c = 0; c < nchan; ++c) {
-            const double f = freqs[c];
-            const double x = kDispersionConstant * dm * (1.0 / (f * f) - 1.0 / (ftop * ftop)) / tsamp;
-            const double r = std::floor(x + 0.5);
-            if (!(r < 1.0e9)) return SP_ELIMIT;
-            const int32_t v = (int32_t)r;
-            out[(size_t)d * nchan + c] = v;
-            mx = std::max(mx, v);
+    // Trials are independent: blocks of them on the host's cores.
+    std::atomic<int32_t> next{0}, mx{0};
+    std::atomic<bool> beyond{false};
+    constexpr int32_t kBlock = 64;
+    auto work = [&]() {
+        int32_t most = 0;
+        for (int32_t d0; (d0 = next.fetch_add(kBlock)) < ndm && !beyond;) {
+            for (int32_t d = d0; d < std::min(ndm, d0 + kBlock); ++d) {
+                const double dm = dms[d];
+                for (int32_t c = 0; c < nchan; ++c) {
+                    const double f = freqs[c];
+                    const double x = kDispersionConstant * dm * (1.0 / (f * f) - 1.0 / (ftop * ftop)) / tsamp;
+                    const double r = std::floor(x + 0.5);
+                    if (!(r < 1.0e9)) {
+                        beyond = true;
+                        return;
+                    }
+                    const int32_t v = (int32_t)r;
+                    out[(size_t)d * nchan + c] = v;
+                    most = std::max(most, v);
+                }
+            }
         }
-    }
+        for (int32_t seen = mx.load(); most > seen && !mx.compare_exchange_weak(seen, most);) {}
+    };
+    run_on_cores(work, (ndm + kBlock - 1) / kBlock);
+    if (beyond) return SP_ELIMIT;
     *max_delay = mx;
     return SP_OK;
 }
@@ -111,6 +126,9 @@ static void free_plan_device(sp_plan *p) {
     cudaFree(p->d_chunk_geo);
     cudaFree(p->d_chunk_off);
     cudaFree(p->d_status);
+    cudaFree(p->d_sums_mem);
+    p->d_sums_mem = nullptr;
+    p->d_sums = nullptr;
     p->d_delays = p->d_tile_first = p->d_tile_count = p->d_chunk_off = p->d_status = nullptr;
     p->d_chunk_geo = nullptr;
 }
@@ -122,6 +140,48 @@ static int upload(T **dst, const T *src, size_t n) {
         return SP_ENOMEM;
     }
     if (cudaMemcpy(*dst, src, n * sizeof(T), cudaMemcpyHostToDevice) != cudaSuccess) return SP_ECUDA;
+    return SP_OK;
+}
+
+// Uploads the shared-sum tables in one allocation: the descriptor, then each
+// array at a multiple of 256 bytes.
+static int upload_sums(sp_plan *p, const SumTables &t) {
+    const void *src[] = {t.tile_first.data(), t.tile_count.data(), t.tile_chunk.data(), t.tile_group.data(),
+                         t.tile_job.data(),   t.jobs.data(),       t.chunks.data(),     t.prog_bytes.data(), t.geo.data(),        t.prog.data(),
+                         t.off.data()};
+    const size_t n[] = {t.tile_first.size(), t.tile_count.size(), t.tile_chunk.size(), t.tile_group.size(),
+                        t.tile_job.size(),   t.jobs.size(),       t.chunks.size(),     t.prog_bytes.size(), t.geo.size(),        t.prog.size(),
+                        t.off.size()};
+    constexpr int kArrays = 11;
+    int64_t at[kArrays + 1] = {align256(sizeof(SumTablesDev))};
+    for (int i = 0; i < kArrays; ++i) at[i + 1] = align256(at[i] + (int64_t)n[i] * 4);
+    std::vector<uint8_t> h((size_t)at[kArrays], 0);
+    uint8_t *d = nullptr;
+    if (cudaMalloc((void **)&d, h.size()) != cudaSuccess) {
+        cudaGetLastError();
+        return SP_ENOMEM;
+    }
+    p->d_sums_mem = d;
+    SumTablesDev v{};
+    v.tile_first = reinterpret_cast<const int32_t *>(d + at[0]);
+    v.tile_count = reinterpret_cast<const int32_t *>(d + at[1]);
+    v.tile_chunk = reinterpret_cast<const int32_t *>(d + at[2]);
+    v.tile_group = reinterpret_cast<const int32_t *>(d + at[3]);
+    v.tile_job = reinterpret_cast<const int32_t *>(d + at[4]);
+    v.jobs = reinterpret_cast<const uint2 *>(d + at[5]);
+    v.chunks = reinterpret_cast<const int4 *>(d + at[6]);
+    v.prog_bytes = reinterpret_cast<const int32_t *>(d + at[7]);
+    v.geo = reinterpret_cast<const int4 *>(d + at[8]);
+    v.prog = reinterpret_cast<const uint4 *>(d + at[9]);
+    v.off = reinterpret_cast<const int32_t *>(d + at[10]);
+    v.ntiles = (int32_t)t.tile_first.size();
+    v.nchan = p->nchan;
+    std::memcpy(h.data(), &v, sizeof v);
+    for (int i = 0; i < kArrays; ++i) std::memcpy(h.data() + at[i], src[i], n[i] * 4);
+    if (cudaMemcpy(d, h.data(), h.size(), cudaMemcpyHostToDevice) != cudaSuccess) return SP_ECUDA;
+    p->d_sums = reinterpret_cast<SumTablesDev *>(d);
+    p->sums_ntiles = v.ntiles;
+    p->sums_tile_clocks = t.tile_clocks;
     return SP_OK;
 }
 
@@ -215,6 +275,17 @@ static int create_plan(const double *freqs_mhz, int32_t nchan, double tsamp_s, c
     if (!rc) rc = upload(&p->d_chunk_off, off.data(), off.size());
     const int32_t zero = 0;
     if (!rc) rc = upload(&p->d_status, &zero, 1);
+    if (!rc && shape == 0) {  // the default shape's plans; the others stay the direct kernel's
+        try {
+            SumTables t;
+            if (build_sum_tables(*p, t) == SP_OK && sum_tables_pay(*p, t)) {
+                rc = upload_sums(p, t);
+                if (!rc) rc = sums_configure();
+            }
+        } catch (const std::bad_alloc &) {
+            rc = SP_ENOMEM;
+        }
+    }
     if (!rc) rc = dedisp_configure(p);
     if (rc) {
         free_plan_device(p);
@@ -338,6 +409,12 @@ extern "C" int sp_plan_check_tables(const double *freqs_mhz, int32_t nchan, doub
                 }
             }
         }
+    }
+    if (shape == 0) {
+        SumTables t;
+        const int src = build_sum_tables(p, t);
+        if (src == SP_OK) bad += check_sum_tables(p, t, n_out);
+        else bad += src != SP_ELIMIT;
     }
     h_report[0] = p.ntiles;
     h_report[1] = p.nchunks;

@@ -2,7 +2,9 @@
 // Not installed; the public interface is include/spotlight.h.
 #pragma once
 
+#include <algorithm>
 #include <cstdint>
+#include <thread>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -55,6 +57,54 @@ __host__ __device__ inline int32_t dedisp_row_bytes(int32_t span, int32_t time_t
     return ((15 + span + time_tile + 15) / 16) * 16;
 }
 
+// Shared-sum dedispersion (dedisp_sums.cu, tables in plan_sums.cpp).  One
+// CTA = up to kSumDms consecutive trial DMs x kSumTime output samples.
+// Channels go in groups of up to kSumMaxGroup; the DMs of a tile see a group's
+// channels at few distinct relative delays, so the group's sum is formed once
+// per distinct pattern (a "row" of 16-bit sums) and added to every DM that
+// has it.  A chunk is a run of groups whose rows fill one row slot.
+constexpr int kSumDms = 64;
+constexpr int kSumTime = 1024;
+constexpr int kSumHalf = kSumTime / 2;    // a row word holds samples j and j + kSumHalf
+constexpr int kSumMaxGroup = 16;          // channels per group
+constexpr int kSumMaxChunk = 16;          // channels per chunk
+constexpr int kSumSlots = 3;              // chunks in flight (raw windows, rows)
+constexpr int kSumRowBytes = 52 * 1024;   // one row slot
+constexpr int kSumRawBytes = 23 * 1024;   // one raw slot: program, then channel windows
+constexpr int kSumHeader = 1024;
+constexpr int kSumSmem = kSumHeader + kSumSlots * (kSumRowBytes + kSumRawBytes);
+static_assert(kSumSmem <= 227 * 1024, "one CTA per SM");
+// 16-bit lanes: 255 left by a carry extraction plus 256 channels of bytes.
+constexpr int kSumCarryChannels = 256;
+constexpr int kSumMaxChan = 65536;        // 16-bit carries
+
+// Device view of a plan's shared-sum tables.
+struct SumTablesDev {
+    const int32_t *tile_first, *tile_count;  // [ntiles]
+    const int32_t *tile_chunk, *tile_group, *tile_job;  // [ntiles + 1] first chunk / group / job of a tile
+    const int4 *chunks;                      // [nchunks] {channels, first channel, first geo entry, program offset / 16}
+    const int32_t *prog_bytes;               // [nchunks]
+    const int4 *geo;                         // per channel of a chunk {window start, window bytes, raw slot offset, 0}
+    const uint4 *prog;                       // producers' programs
+    const uint2 *jobs;                       // [njobs], see kSumJob*
+    const int32_t *off;                      // [ngroups][kSumDms] byte offset in the row slot | flags
+    int32_t ntiles, nchan;
+};
+// Flags in the low bits of off[g][8 w] (offsets are multiples of 4).
+constexpr int kSumLastOfChunk = 1, kSumCarryAfter = 2;
+// A job (32 quads of one segment): x = slot | phase parity << 2 | first use of
+// the slot | arrivals on full[slot] << 8 (a chunk's jobs arrive kSumJobArrivals
+// times in all), y = segment's offset in the raw slot / 16 | first quad << 16.
+constexpr uint32_t kSumJobFirstUse = 8u;
+constexpr int kSumJobArrivals = 64;
+constexpr int kSumMinJobs = kSumHalf / 128;  // of a chunk: a row has at least kSumHalf / 4 quads
+// Host tables.
+struct SumTables {
+    std::vector<int32_t> tile_first, tile_count, tile_chunk, tile_group, tile_job, chunks, prog_bytes, geo, off;
+    std::vector<uint32_t> prog, jobs;
+    double tile_clocks = 0.0;  // modelled SM clocks of an average work item
+};
+
 }  // namespace sp
 
 struct sp_plan {
@@ -86,6 +136,12 @@ struct sp_plan {
     // the chunk's copies (copy (shift & 3), word shift >> 2).
     int32_t *d_chunk_off = nullptr;   // [ntiles][nchunks][chan_chunk][dm_tile]
     int32_t *d_status = nullptr;      // device status word (bit 0: a staging wait timed out)
+    // Shared-sum tables (nullptr: this plan's DMs share too little; the
+    // kernel above runs).  One allocation behind d_sums_mem.
+    sp::SumTablesDev *d_sums = nullptr;
+    void *d_sums_mem = nullptr;
+    int32_t sums_ntiles = 0;
+    double sums_tile_clocks = 0.0;
 };
 
 namespace sp {
@@ -108,7 +164,10 @@ struct BatchBeamDev {
     int64_t pitch;
     int64_t n_out;
     int32_t *out;                  // [ndm][n_out]
-    const int32_t *tile_first;
+    union {
+        const int32_t *tile_first;
+        const SumTablesDev *sums;  // of a shared-sum launch (the other tables are then unused)
+    };
     const int32_t *tile_count;
     const int4 *geo;
     const int32_t *off;
@@ -116,6 +175,7 @@ struct BatchBeamDev {
 };
 // Host view of a batch launch: every beam's plan must have the same shape.
 struct BatchLaunch {
+    bool sums;                     // shared-sum kernel (every plan has its tables)
     int32_t shape;
     int32_t nbeams;
     int64_t nitems;                // sum over beams of ntiles * ntime
@@ -132,6 +192,18 @@ int batch_grid(BatchLaunch &b);
 // persistent: a resident grid draining the work queue; else one CTA per item.
 int launch_dedisperse_batch(const BatchLaunch &b, cudaStream_t stream, bool persistent = true);
 int64_t dedisp_time_tiles(const sp_plan *plan, int64_t n_out);
+// Shared-sum kernel: whether a launch over these beams goes to it
+// (plan_sums.cpp), its tables, its launches.
+bool sums_pay(const sp_plan *const *plans, const int64_t *n_out, int32_t nbeams);
+int build_sum_tables(const sp_plan &p, SumTables &t);
+bool sum_tables_pay(const sp_plan &p, const SumTables &t);
+int64_t check_sum_tables(const sp_plan &p, const SumTables &t, int64_t n_out);
+int64_t sums_items(const sp_plan *plan, int64_t n_out);
+int sums_configure();
+int launch_dedisperse_sums(const sp_plan *plan, const uint8_t *d_xt, int64_t pitch, int64_t n_out, int32_t *d_out,
+                           cudaStream_t stream, int32_t *status);
+int launch_dedisperse_sums_batch(const BatchLaunch &b, cudaStream_t stream);
+int set_sums_fault(uint32_t extra_bytes, long long wait_limit);
 // Test hook of the dedispersion kernel's bounded waits on the current device.
 int set_staging_fault(uint32_t extra_bytes, long long wait_limit);
 // Sets the dynamic shared-memory limit of the plan's kernels on the current
@@ -167,6 +239,21 @@ int launch_sps_window(SpsArgs a, int32_t radius, cudaStream_t stream);
 // Sets the boxcar kernels' shared-memory limit for widths up to maxw on the
 // current device (launch_sps does it on first use otherwise).
 int sps_configure(int32_t maxw);
+
+// Runs work() on this thread and on as many more as the host has cores for, up
+// to 16 in all and no more than there are pieces; work takes pieces until none
+// is left, so threads that cannot be started only leave more to the others.
+template <class F>
+inline void run_on_cores(F &work, int64_t pieces) {
+    const int64_t n = std::min<int64_t>({(int64_t)std::thread::hardware_concurrency(), 16, pieces});
+    std::vector<std::thread> pool;
+    try {
+        for (int64_t k = 1; k < n; ++k) pool.emplace_back([&work]() { work(); });
+    } catch (...) {
+    }
+    work();
+    for (std::thread &t : pool) t.join();
+}
 
 inline int64_t align256(int64_t x) { return (x + 255) & ~int64_t(255); }
 

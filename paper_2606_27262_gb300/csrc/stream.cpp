@@ -150,6 +150,7 @@ struct sp_stream {
     // SP_STREAM_ONE_STREAM keeps all of a batch on its launch stream.
     cudaStream_t search_stream = nullptr;
     BatchLaunch geometry{};
+    bool sums = false;  // the batched launches go to the shared-sum kernel
     std::deque<Gulp> pending;
     std::deque<Searched> searched;
     std::deque<Result> results;
@@ -327,7 +328,8 @@ int launch_batch(sp_stream *s, int li) {
             rc = launch_dedisperse(p, sl.d_staged, s->pitch, s->gulp, sl.d_dmt, st, L.d_status);
         }
     } else if (!rc) {
-        const int64_t items = (int64_t)p->ntiles * dedisp_time_tiles(p, s->gulp);
+        const bool sums = s->sums;
+        const int64_t items = sums ? sums_items(p, s->gulp) : (int64_t)p->ntiles * dedisp_time_tiles(p, s->gulp);
         L.h_begin[0] = 0;
         for (int i = 0; i < n; ++i) {
             const Slot &sl = s->slots[L.slots[i]];
@@ -344,6 +346,10 @@ int launch_batch(sp_stream *s, int li) {
             d.nchunks = p->nchunks;
             d.ntiles = p->ntiles;
             d.ntime = (int32_t)dedisp_time_tiles(p, s->gulp);
+            if (sums) {
+                d.sums = p->d_sums;
+                d.ntime = (int32_t)((s->gulp + kSumTime - 1) / kSumTime);
+            }
             L.h_begin[i + 1] = L.h_begin[i] + items;
         }
         // Pinned sources: the copies are asynchronous; the buffers are
@@ -354,6 +360,7 @@ int launch_batch(sp_stream *s, int li) {
                 cudaSuccess)
             rc = SP_ECUDA;
         BatchLaunch B = s->geometry;
+        B.sums = sums;
         B.nbeams = n;
         B.nitems = L.h_begin[n];
         B.d_beams = L.d_table;
@@ -687,6 +694,12 @@ extern "C" int sp_stream_create(const sp_plan *plan, int32_t nbeams, int64_t gul
         G.raw_max = plan->raw_max;
         G.smem_bytes = plan->smem_bytes;
         rc = batch_grid(G);
+    }
+    if (!rc) {  // a full batch decides: every batch then runs the same kernel
+        const std::vector<const sp_plan *> plans((size_t)max_batch, plan);
+        const std::vector<int64_t> n_outs((size_t)max_batch, gulp);
+        s->sums = sums_pay(plans.data(), n_outs.data(), max_batch);
+        if (s->sums) rc = sums_configure();
     }
     if (!rc) rc = dedisp_configure(plan);
     if (!rc) rc = sps_configure(h_widths[nw - 1]);
