@@ -423,7 +423,7 @@ extern "C" int sp_cnn_train_step(sp_cnn *c, const void *d_ft, const void *d_dmt,
 }
 
 extern "C" int64_t sp_cnn_features_workspace_bytes(int32_t batch) {
-    // both raw fp32 images and 8 blocks x 4 sums per candidate
+    // a reserved block, the raw fp32 DM-time images, and 8 blocks x 4 sums per candidate
     return batch > 0 ? 2 * align256((int64_t)batch * kImg * kImg * 4) + align256((int64_t)batch * 8 * 16) : -1;
 }
 
@@ -433,12 +433,11 @@ extern "C" int sp_cnn_features(const float *d_sub, int32_t batch, int32_t nsub, 
     if (!d_work || work_bytes < sp_cnn_features_workspace_bytes(batch) ||
         (reinterpret_cast<uintptr_t>(d_work) & 255))
         return SP_EWORKSPACE;
-    float *ft_raw = static_cast<float *>(d_work);
     float *dmt_raw = reinterpret_cast<float *>(static_cast<uint8_t *>(d_work) +
                                                align256((int64_t)batch * kImg * kImg * 4));
     float *part = reinterpret_cast<float *>(static_cast<uint8_t *>(d_work) +
                                             2 * align256((int64_t)batch * kImg * kImg * 4));
-    return cnn_features(d_sub, batch, nsub, t_in, d_shift, ft_raw, dmt_raw, part, static_cast<__nv_bfloat16 *>(d_ft),
+    return cnn_features(d_sub, batch, nsub, t_in, d_shift, dmt_raw, part, static_cast<__nv_bfloat16 *>(d_ft),
                         static_cast<__nv_bfloat16 *>(d_dmt), reinterpret_cast<cudaStream_t>(stream));
 }
 

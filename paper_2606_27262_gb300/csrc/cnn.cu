@@ -15,9 +15,9 @@
 //   col2im_relu_kernel  the adjoint of im2col (a gather, no atomics) fused
 //                       with the ReLU derivative of the layer below.
 //   transpose_kernel    bf16 [R][C] -> [C][R] (operands of the backward GEMMs).
-//   features_raw_kernel frequency-time and DM-time images of a subband
-//   normalise_kernel    dynamic spectrum, then each normalised to zero mean
-//                       and unit variance, as bf16.
+//   features_raw_kernel DM-time images of subband dynamic spectra
+//   normalise_kernel    frequency-time and DM-time images normalised to zero
+//                       mean and unit variance, as bf16.
 //   plus average pooling, the linear heads, the fused loss and Adam.
 #include <cuda_bf16.h>
 
@@ -512,115 +512,198 @@ __global__ void to_bf16_kernel(const float *__restrict__ a, int64_t n, __nv_bflo
 // (already dedispersed at the candidate DM within each subband; time bins):
 //   ft[s][u]  = sub[s][u0 + u]                         (S x 256)
 //   dmt[j][u] = sum_s sub[s][u0 + u + shift[j][s]]     (256 trial-DM offsets)
-// u0 = (T_in - 256) / 2.  Each image is then set to zero mean and unit
-// variance (computed in fp32 over its 65536 values) and stored as bf16.
-// One CTA (256 threads) per (candidate, image row); a second pass normalises.
-// Raw images of candidate b: ft_raw[b][s][u] = sub[b][s][u0 + u] and
-// dmt_raw[b][j][u] = sum over subbands k (in order) of sub[b][k][u0 + u +
-// shift[j][k]] (bins outside the spectrum count 0), u0 = (T_in - 256) / 2.
-// One CTA per (block of kFeatRows rows j, candidate), one thread per bin u:
-// subband k's whole row of T_in bins is staged in shared memory (double
-// buffered) between kImg zero bins on each side and serves the CTA's
-// kFeatRows shifted sums at once.  Each shift is clamped once, when the
-// block's shift table is staged, to [-u0 - kImg, T_in - u0]: a row whose
-// window lies wholly outside the spectrum then reads only zeros, so the sum
-// loop needs no bounds test; per subband a thread takes its kFeatRows shifts
-// with 16-byte broadcast loads; the next subband's row is fetched by
-// asynchronous copies (cp.async) while the current one is summed.  (A third
-// buffer with the next row prefetched into registers ran at half the speed:
-// fewer CTAs per SM.)
+// u0 = (T_in - 256) / 2, bins outside the spectrum count 0, subbands added in
+// order.  Each image is then set to zero mean and unit variance (computed in
+// fp32 over its 65536 values) and stored as bf16.
+//
+// DM-time rows: one CTA per (32 rows j, candidate), one warp per R rows of
+// 256 bins (a lane's bins are lane + 32 i).  The sum is bound by shared-memory
+// reads and instruction issue.  Neighbouring rows read most subbands at the
+// same shift (the shifts of a 255-bin sweep differ by at most one bin from
+// row to row, at the band's bottom), so a warp keeps the bins it has loaded
+// and loads again only where the shift changes: about 0.4 loads per row and
+// subband; one address serves a lane's eight bins, and two bins are added per
+// instruction (add.f32x2, the same rounding as two adds).  Windows of
+// [smallest, largest shift of the 32 rows] + 256 bins arrive by 16-byte
+// asynchronous copies, several subbands to a stage, two stages.  The shifts
+// are any integers: wide ones take fewer subbands per stage, and where not even
+// one window fits a stage the bins are read from global memory.
+// 512-bin spectra: 1.00 -> 0.35 ms at batch 256 and 0.175 -> 0.046 ms at batch 5
+// against one load, one address and one add per bin and row.
 constexpr int kFeatRows = 32;
-__global__ void __launch_bounds__(kImg) features_raw_kernel(const float *__restrict__ sub, int T_in,
-                                                            const int32_t *__restrict__ shift,
-                                                            float *__restrict__ ft_raw, float *__restrict__ dmt_raw,
-                                                            float4 *__restrict__ part) {
-    extern __shared__ __align__(16) float fsm[];
-    // staged row: kImg zeros, T_in bins, kImg zeros (stride a multiple of 4 floats, so that the shift
-    // table after the two rows is 16-byte aligned for its int4 loads)
-    const int RW = (T_in + 2 * kImg + 3) & ~3;
-    float *rows = fsm;                                          // [2][RW]
-    int32_t *sh = reinterpret_cast<int32_t *>(fsm + 2 * RW);    // [kImg subbands][kFeatRows]
-    const int b = blockIdx.y, j0 = blockIdx.x * kFeatRows, u = threadIdx.x;
+constexpr int kFeatStage = 8 * 336;  // floats of one stage
+
+__device__ __forceinline__ void add2(unsigned long long &a, unsigned long long b) {
+    asm("add.rn.f32x2 %0, %0, %1;" : "+l"(a) : "l"(b));
+}
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+
+template <int R>
+__global__ void __launch_bounds__(32 * kFeatRows / R) features_raw_kernel(const float *__restrict__ sub, int T_in,
+                                                                        const int32_t *__restrict__ shift, bool vec,
+                                                                        float *__restrict__ dmt_raw,
+                                                                        float4 *__restrict__ part) {
+    constexpr int NW = kFeatRows / R, NT = 32 * NW, NI = kImg / 32;
+    __shared__ __align__(16) float win[2][kFeatStage];
+    __shared__ __align__(16) uint16_t rel[kImg][kFeatRows];  // bin of a row's u = 0 in its subband's window
+    __shared__ int base[kImg];                               // first bin of the window (a multiple of 4)
+    __shared__ float4 row_sum[kFeatRows];
+    __shared__ int widest;
+    const int b = blockIdx.y, j0 = blockIdx.x * kFeatRows, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int u0 = (T_in - kImg) / 2;
     const float *sb = sub + (size_t)b * kImg * T_in;
-    float fs = 0.f, fs2 = 0.f;  // this thread's share of the block's frequency-time sums
-    for (int r = 0; r < kFeatRows; ++r) {
-        const float v = sb[(size_t)(j0 + r) * T_in + u0 + u];
-        ft_raw[((size_t)b * kImg + j0 + r) * kImg + u] = v;
-        fs += v;
-        fs2 += v * v;
-    }
-    for (int i = threadIdx.x; i < kImg * kFeatRows; i += blockDim.x) {
-        const int r = i / kImg, k = i - r * kImg;
-        sh[k * kFeatRows + r] = min(max(shift[(size_t)(j0 + r) * kImg + k], -u0 - kImg), T_in - u0);
-    }
-    for (int i = threadIdx.x; i < kImg; i += blockDim.x) {  // the zero margins of both buffers
-        rows[i] = rows[kImg + T_in + i] = 0.f;
-        rows[RW + i] = rows[RW + kImg + T_in + i] = 0.f;
-    }
-    for (int i = 2 * kImg + T_in + threadIdx.x; i < RW; i += blockDim.x) rows[i] = rows[RW + i] = 0.f;
-    for (int i = threadIdx.x; i < T_in; i += blockDim.x) rows[kImg + i] = sb[i];
+    if (threadIdx.x == 0) widest = 0;
     __syncthreads();
-    float acc[kFeatRows];
-#pragma unroll
-    for (int r = 0; r < kFeatRows; ++r) acc[r] = 0.f;
-    for (int k = 0; k < kImg; ++k) {
-        // bin u + shift of the row lies at index kImg + u0 + u + shift
-        const float *cur = rows + (k & 1) * RW + kImg + u0 + u;
-        float *nxt = rows + ((k + 1) & 1) * RW + kImg;  // read last in step k - 1, before its barrier
-        // the next row arrives by asynchronous copies while this one is summed
-        if (k + 1 < kImg) {
-            for (int i = threadIdx.x; i < T_in; i += blockDim.x) cp_async4(nxt + i, sb + (size_t)(k + 1) * T_in + i);
-            cp_async_commit();
+    for (int k = threadIdx.x; k < kImg; k += NT) {
+        // A shift that leaves the spectrum altogether reads zeros only: clamped to the first that does.
+        auto at = [&](int r) { return u0 + min(max(shift[(size_t)(j0 + r) * kImg + k], -u0 - kImg), T_in - u0); };
+        int lo = at(0), hi = lo;
+        for (int r = 1; r < kFeatRows; ++r) {
+            const int v = at(r);
+            lo = min(lo, v);
+            hi = max(hi, v);
         }
-        const int4 *shk = reinterpret_cast<const int4 *>(sh + k * kFeatRows);
-#pragma unroll
-        for (int q = 0; q < kFeatRows / 4; ++q) {
-            const int4 s4 = shk[q];
-            acc[4 * q] += cur[s4.x];
-            acc[4 * q + 1] += cur[s4.y];
-            acc[4 * q + 2] += cur[s4.z];
-            acc[4 * q + 3] += cur[s4.w];
-        }
-        cp_async_wait<0>();
-        __syncthreads();
+        lo &= ~3;
+        base[k] = lo;
+        for (int r = 0; r < kFeatRows; ++r) rel[k][r] = (uint16_t)(at(r) - lo);
+        atomicMax(&widest, hi - lo);
     }
-    float ds = 0.f, ds2 = 0.f;
-#pragma unroll
-    for (int r = 0; r < kFeatRows; ++r) {
-        dmt_raw[((size_t)b * kImg + j0 + r) * kImg + u] = acc[r];
-        ds += acc[r];
-        ds2 += acc[r] * acc[r];
-    }
-    // The block's sums of both images, in a fixed order: warp trees, then
-    // the warps in turn (the normalisation adds the blocks in turn).
-    float4 t4 = make_float4(fs, fs2, ds, ds2);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        t4.x += __shfl_xor_sync(0xffffffffu, t4.x, o);
-        t4.y += __shfl_xor_sync(0xffffffffu, t4.y, o);
-        t4.z += __shfl_xor_sync(0xffffffffu, t4.z, o);
-        t4.w += __shfl_xor_sync(0xffffffffu, t4.w, o);
-    }
-    __shared__ float4 wsum[kImg / 32];
-    if ((u & 31) == 0) wsum[u >> 5] = t4;
     __syncthreads();
-    if (u == 0) {
-        float4 a = wsum[0];
-        for (int w = 1; w < kImg / 32; ++w) {
-            a.x += wsum[w].x;
-            a.y += wsum[w].y;
-            a.z += wsum[w].z;
-            a.w += wsum[w].w;
+    const int stride = (kImg + widest + 3) & ~3;        // floats of a window
+    const int per = min(8, kFeatStage / stride);        // subbands of a stage (0: straight from global memory)
+    auto stage = [&](int k0, int buf) {
+        for (int kk = warp; kk < per && k0 + kk < kImg; kk += NW) {
+            const int e0 = base[k0 + kk];
+            const float *src = sb + (size_t)(k0 + kk) * T_in;
+            float *dst = &win[buf][kk * stride];
+            if (vec) {  // rows start at 16-byte boundaries: a group of four bins is inside or outside as one
+                for (int c = 4 * lane; c < stride; c += 128) {
+                    const bool ok = e0 + c >= 0 && e0 + c < T_in;
+                    cp_async16(dst + c, src + (ok ? e0 + c : 0), ok);
+                }
+            } else {
+                for (int c = lane; c < stride; c += 32) {
+                    if (e0 + c >= 0 && e0 + c < T_in) cp_async4(dst + c, src + e0 + c);
+                    else dst[c] = 0.f;
+                }
+            }
         }
-        part[(size_t)b * (kImg / kFeatRows) + blockIdx.x] = a;
+        cp_async_commit();
+    };
+    unsigned long long acc[R][NI / 2];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int i = 0; i < NI / 2; ++i) acc[r][i] = 0ull;
+    unsigned long long v[NI / 2];
+    auto rows_of = [&](int k, uint32_t (&o)[R]) {
+        const uint16_t *p = &rel[k][warp * R];
+        if constexpr (R == 8) {
+            const uint4 w = *reinterpret_cast<const uint4 *>(p);
+            const uint32_t x[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+            for (int r = 0; r < 8; ++r) o[r] = (x[r >> 1] >> (16 * (r & 1))) & 0xFFFFu;
+        } else if constexpr (R == 4) {
+            const uint2 w = *reinterpret_cast<const uint2 *>(p);
+            o[0] = w.x & 0xFFFFu, o[1] = w.x >> 16, o[2] = w.y & 0xFFFFu, o[3] = w.y >> 16;
+        } else {
+#pragma unroll
+            for (int r = 0; r < R; ++r) o[r] = p[r];
+        }
+    };
+    if (per > 0) {
+        stage(0, 0);
+        for (int k0 = 0, buf = 0; k0 < kImg; k0 += per, buf ^= 1) {
+            stage(k0 + per, buf ^ 1);
+            cp_async_wait<1>();
+            __syncthreads();
+            const int nk = min(per, kImg - k0);
+            for (int kk = 0; kk < nk; ++kk) {
+                const float *p = &win[buf][kk * stride + lane];
+                uint32_t o[R];
+                rows_of(k0 + kk, o);
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    if (r == 0 || o[r] != o[r - 1]) {
+#pragma unroll
+                        for (int i = 0; i < NI / 2; ++i) v[i] = pack2(p[o[r] + 64 * i], p[o[r] + 64 * i + 32]);
+                    }
+#pragma unroll
+                    for (int i = 0; i < NI / 2; ++i) add2(acc[r][i], v[i]);
+                }
+            }
+            __syncthreads();
+        }
+    } else {
+        for (int k = 0; k < kImg; ++k) {
+            uint32_t o[R];
+            rows_of(k, o);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int e = base[k] + (int)o[r] + lane;
+                auto bin = [&](int i) {
+                    const int x = e + 32 * i;
+                    return x >= 0 && x < T_in ? __ldg(sb + (size_t)k * T_in + x) : 0.f;
+                };
+#pragma unroll
+                for (int i = 0; i < NI / 2; ++i) add2(acc[r][i], pack2(bin(2 * i), bin(2 * i + 1)));
+            }
+        }
+    }
+    // Sums of each row of both images: a lane's bins in order, then a warp
+    // tree; of the block's rows: another (the same for every R).
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int j = j0 + warp * R + r;
+        float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < NI; ++i) {
+            const float f = sb[(size_t)j * T_in + u0 + 32 * i + lane];
+            const float2 d2 = unpack2(acc[r][i >> 1]);
+            const float d = i & 1 ? d2.y : d2.x;
+            dmt_raw[((size_t)b * kImg + j) * kImg + 32 * i + lane] = d;
+            t.x += f;
+            t.y += f * f;
+            t.z += d;
+            t.w += d * d;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            t.x += __shfl_xor_sync(0xffffffffu, t.x, o);
+            t.y += __shfl_xor_sync(0xffffffffu, t.y, o);
+            t.z += __shfl_xor_sync(0xffffffffu, t.z, o);
+            t.w += __shfl_xor_sync(0xffffffffu, t.w, o);
+        }
+        if (lane == 0) row_sum[warp * R + r] = t;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        float4 t = row_sum[lane];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            t.x += __shfl_xor_sync(0xffffffffu, t.x, o);
+            t.y += __shfl_xor_sync(0xffffffffu, t.y, o);
+            t.z += __shfl_xor_sync(0xffffffffu, t.z, o);
+            t.w += __shfl_xor_sync(0xffffffffu, t.w, o);
+        }
+        if (lane == 0) part[(size_t)b * (kImg / kFeatRows) + blockIdx.x] = t;
     }
 }
 
 // One CTA per (block of kFeatRows rows, candidate, image): the image's mean
 // and population variance from the feature kernel's per-block sums (added
-// in block order), then the block's rows scaled and stored as bf16.
-__global__ void __launch_bounds__(kImg) normalise_kernel(const float *__restrict__ ft_raw,
+// in block order), then the block's rows scaled and stored as bf16.  The
+// frequency-time rows come straight from the spectrum.
+__global__ void __launch_bounds__(kImg) normalise_kernel(const float *__restrict__ sub, int T_in,
                                                          const float *__restrict__ dmt_raw,
                                                          const float4 *__restrict__ part, __nv_bfloat16 *__restrict__ ft,
                                                          __nv_bfloat16 *__restrict__ dmt) {
@@ -635,12 +718,12 @@ __global__ void __launch_bounds__(kImg) normalise_kernel(const float *__restrict
     const float mean = s / n;
     const float var = fmaxf(s2 / n - mean * mean, 0.f);
     const float inv = var > 0.f ? rsqrtf(var) : 0.f;
-    const float *raw = img ? dmt_raw : ft_raw;
-    __nv_bfloat16 *out = img ? dmt : ft;
-    for (int r = 0; r < kFeatRows; ++r) {
-        const size_t i = ((size_t)b * kImg + j0 + r) * kImg + u;
-        out[i] = __float2bfloat16((raw[i] - mean) * inv);
-    }
+    const float *raw = img ? dmt_raw + (size_t)b * kImg * kImg : sub + (size_t)b * kImg * T_in + (T_in - kImg) / 2;
+    const int row = img ? kImg : T_in;
+    __nv_bfloat16 *out = (img ? dmt : ft) + (size_t)b * kImg * kImg;
+#pragma unroll 8
+    for (int r = 0; r < kFeatRows; ++r)
+        out[(j0 + r) * kImg + u] = __float2bfloat16((raw[(size_t)(j0 + r) * row + u] - mean) * inv);
 }
 
 // Subband dynamic spectrum of candidate q from the staged beam xt
@@ -825,19 +908,19 @@ int cnn_extract(const uint8_t *xt, int64_t pitch, int64_t n_in, int32_t nchan, c
     return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
 }
 
-int cnn_features(const float *sub, int Nb, int S, int T_in, const int32_t *shift, float *ft_raw, float *dmt_raw,
-                 float *part, __nv_bfloat16 *ft, __nv_bfloat16 *dmt, cudaStream_t st) {
+int cnn_features(const float *sub, int Nb, int S, int T_in, const int32_t *shift, float *dmt_raw, float *part,
+                 __nv_bfloat16 *ft, __nv_bfloat16 *dmt, cudaStream_t st) {
     if (S != kImg || T_in < kImg || T_in > 4096) return SP_EINVAL;
-    const size_t smem = (size_t)2 * ((T_in + 2 * kImg + 3) & ~3) * 4 + (size_t)kImg * kFeatRows * 4;  // <= 36 KB + 32 KB
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(features_raw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-            cudaSuccess)
-        return SP_ECUDA;
     float4 *p4 = reinterpret_cast<float4 *>(part);
-    features_raw_kernel<<<dim3(kImg / kFeatRows, Nb), kImg, smem, st>>>(sub, T_in, shift, ft_raw, dmt_raw, p4);
+    const bool vec = T_in % 4 == 0 && (reinterpret_cast<uintptr_t>(sub) & 15) == 0;
+    // Rows per warp: more share more loads, fewer give more warps.
+    const dim3 grid(kImg / kFeatRows, Nb);
+    if (Nb >= 48) features_raw_kernel<8><<<grid, 32 * kFeatRows / 8, 0, st>>>(sub, T_in, shift, vec, dmt_raw, p4);
+    else if (Nb >= 16) features_raw_kernel<4><<<grid, 32 * kFeatRows / 4, 0, st>>>(sub, T_in, shift, vec, dmt_raw, p4);
+    else features_raw_kernel<2><<<grid, 32 * kFeatRows / 2, 0, st>>>(sub, T_in, shift, vec, dmt_raw, p4);
     note_launch();
     if (cudaGetLastError() != cudaSuccess) return SP_ECUDA;
-    normalise_kernel<<<dim3(kImg / kFeatRows, Nb, 2), kImg, 0, st>>>(ft_raw, dmt_raw, p4, ft, dmt);
+    normalise_kernel<<<dim3(kImg / kFeatRows, Nb, 2), kImg, 0, st>>>(sub, T_in, dmt_raw, p4, ft, dmt);
     note_launch();
     return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
 }

@@ -70,7 +70,7 @@ int cnn_extract(const uint8_t *xt, int64_t pitch, int64_t n_in, int32_t nchan, c
                 const sp_cand *cands, int32_t ncand, const ExtractWidths &wt, int32_t nsub, int32_t t_in, float *sub,
                 cudaStream_t st);
 // part: Nb * 8 float4 of workspace (per-block image sums, 16-byte aligned).
-int cnn_features(const float *sub, int Nb, int S, int T_in, const int32_t *shift, float *ft_raw, float *dmt_raw,
-                 float *part, __nv_bfloat16 *ft, __nv_bfloat16 *dmt, cudaStream_t st);
+int cnn_features(const float *sub, int Nb, int S, int T_in, const int32_t *shift, float *dmt_raw, float *part,
+                 __nv_bfloat16 *ft, __nv_bfloat16 *dmt, cudaStream_t st);
 
 }  // namespace sp
