@@ -169,35 +169,49 @@ int upload_params(sp_cnn *c, int br, const std::vector<float> &h) {
 
 int forward(sp_cnn *c, const __nv_bfloat16 *ft, const __nv_bfloat16 *dmt, int B, const float *labels, float *prob,
             cudaStream_t st) {
+    // Both branches' layers go in one launch each: with a few candidates a
+    // layer is bound by its latency, not by its work.  No patch matrix in the
+    // forward pass (the backward pass builds the patches it needs for the
+    // weight gradients), the same in training and inference: the first layer
+    // directly, the others as implicit GEMMs on the tensor cores, or im2col +
+    // GEMM where a shape does not suit those.
     int rc = SP_OK;
-    for (int bi = 0; bi < 2 && !rc; ++bi) {
-        Branch &b = c->br[bi];
-        const __nv_bfloat16 *x = bi == 0 ? ft : dmt;
-        for (int l = 0; l < kLayers && !rc; ++l) {
-            const int H = kHin[l], Ho = ho_of(l), Kp = kp_of(l);
-            const int P = B * Ho * Ho;
-            // No patch matrix in the forward pass (the backward pass builds the
-            // patches it needs for the weight gradients), the same in training
-            // and inference: the first layer directly, the others as implicit
-            // GEMMs on the tensor cores, or im2col + GEMM where a shape does not
-            // suit those.
-            if (l == 0)
-                rc = cnn_conv0(x, B, H, H, Ho, Ho, b.pb + b.off_w[0], Kp, b.params + b.off_b[0], b.y[0], st);
-            else
-                rc = cnn_conv_tc(x, B, H, H, kCin[l], Ho, Ho, b.pb + b.off_w[l], Kp, kCout[l], b.params + b.off_b[l],
-                                 b.y[l], st);
-            if (rc != SP_ELIMIT) {
-                x = b.y[l];
-                continue;
-            }
-            rc = cnn_im2col(x, B, H, H, kCin[l], 2, Ho, Ho, Kp, b.cols[l], st);
-            if (!rc)
-                rc = cnn_gemm(kEpiBiasRelu, b.cols[l], Kp, b.pb + b.off_w[l], Kp, P, kCout[l], Kp, nullptr, b.y[l],
-                              kCout[l], b.params + b.off_b[l], 1, st);
-            x = b.y[l];
+    ConvPair p;
+    p.x[0] = ft;
+    p.x[1] = dmt;
+    for (int l = 0; l < kLayers && !rc; ++l) {
+        const int H = kHin[l], Ho = ho_of(l), Kp = kp_of(l);
+        for (int bi = 0; bi < 2; ++bi) {
+            Branch &b = c->br[bi];
+            p.w[bi] = b.pb + b.off_w[l];
+            p.bias[bi] = b.params + b.off_b[l];
+            p.y[bi] = b.y[l];
         }
-        if (!rc) rc = cnn_avgpool(b.y[kLayers - 1], B, ho_of(kLayers - 1) * ho_of(kLayers - 1), kFeat, b.feat, st);
-        if (!rc) rc = cnn_head(b.feat, B, kFeat, b.params + b.off_hw, b.params + b.off_hb, b.logit, st);
+        rc = l == 0 ? cnn_conv0(p, B, H, Kp, st) : cnn_conv_tc(p, B, H, kCin[l], kCout[l], Kp, st);
+        if (rc == SP_ELIMIT) {
+            rc = SP_OK;
+            for (int bi = 0; bi < 2 && !rc; ++bi) {
+                __nv_bfloat16 *cols = c->br[bi].cols[l];
+                rc = cnn_im2col(p.x[bi], B, H, H, kCin[l], 2, Ho, Ho, Kp, cols, st);
+                if (!rc)
+                    rc = cnn_gemm(kEpiBiasRelu, cols, Kp, p.w[bi], Kp, B * Ho * Ho, kCout[l], Kp, nullptr, p.y[bi],
+                                  kCout[l], p.bias[bi], 1, st);
+            }
+        }
+        p.x[0] = p.y[0];
+        p.x[1] = p.y[1];
+    }
+    if (!rc) {
+        HeadPair h;
+        for (int bi = 0; bi < 2; ++bi) {
+            Branch &b = c->br[bi];
+            h.y[bi] = b.y[kLayers - 1];
+            h.w[bi] = b.params + b.off_hw;
+            h.b[bi] = b.params + b.off_hb;
+            h.feat[bi] = b.feat;
+            h.logit[bi] = b.logit;
+        }
+        rc = cnn_pool_head(h, B, ho_of(kLayers - 1) * ho_of(kLayers - 1), st);
     }
     if (!rc && labels && cudaMemsetAsync(c->loss, 0, sizeof(float), st) != cudaSuccess) rc = SP_ECUDA;
     if (!rc)

@@ -59,6 +59,21 @@ __device__ __forceinline__ void mma_bf16(float *c, const uint32_t *a, uint32_t b
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// Two fp32 lanes of a 64-bit register (one instruction, each lane rounded as by the scalar one).
+__device__ __forceinline__ void add2(unsigned long long &a, unsigned long long b) {
+    asm("add.rn.f32x2 %0, %0, %1;" : "+l"(a) : "l"(b));
+}
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+
 // 256 threads: warp (wm, wn) = (warp % 4, warp / 4) owns a 32 x 32 block of
 // the 128 x 64 tile: 2 x 4 mma tiles of 16 x 8.  blockIdx.z = K split.
 template <int EPI>
@@ -208,45 +223,99 @@ __global__ void im2col_c1_kernel(const __nv_bfloat16 *__restrict__ x, int H, int
     }
 }
 
-// Layer 0 of the inference forward (one input channel, 3x3, stride 2, zero
-// padding 1) as a direct convolution: one thread per output pixel gathers
-// its nine taps and accumulates the sixteen outputs in fp32 from the bf16
-// weights (every product exact), then adds the bias, applies the ReLU and
-// rounds once to bf16 -- the im2col + GEMM path's result up to the order of
-// its fp32 accumulation, without writing and reading the patch matrix.
+// Layer 0 (one input channel, 3x3, stride 2, zero padding 1) of both branches
+// (blockIdx.y) as a direct convolution: a thread computes the sixteen outputs
+// of four neighbouring pixels in fp32 from the bf16 weights (every product
+// exact), then adds the bias, applies the ReLU and rounds once to bf16.  Its
+// floor is the write of the output (134 MB a branch at batch 256: 20 us).  Four
+// pixels share each read of the weights, two outputs go to one fma.f32x2, and a
+// warp's output leaves in contiguous stores: 68 us a branch with one pixel and
+// 32 scattered bytes per thread, 51 us now.
 constexpr int kConv0Out = 16;
-__global__ void __launch_bounds__(256) conv0_kernel(const __nv_bfloat16 *__restrict__ x, int H, int W, int Ho,
-                                                    int Wo, uint32_t P, const __nv_bfloat16 *__restrict__ w, int Kp,
-                                                    const float *__restrict__ bias, __nv_bfloat16 *__restrict__ y) {
-    __shared__ float ws[kConv0Out][9];
+__device__ __forceinline__ void fma2(unsigned long long &d, unsigned long long a, unsigned long long b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__global__ void __launch_bounds__(256) conv0_kernel(const ConvPair p, int H, int lwo4, uint32_t quads, int Kp) {
+    __shared__ __align__(16) float ws[9][kConv0Out];
     __shared__ float bs[kConv0Out];
+    __shared__ __align__(16) uint4 out_s[256][8];
+    const bool br = blockIdx.y;
+    const __nv_bfloat16 *w = br ? p.w[1] : p.w[0];
     if (threadIdx.x < kConv0Out * 9) {
         const int co = threadIdx.x / 9, k = threadIdx.x - co * 9;
-        ws[co][k] = __bfloat162float(w[co * Kp + k]);
+        ws[k][co] = __bfloat162float(w[co * Kp + k]);
     }
-    if (threadIdx.x < kConv0Out) bs[threadIdx.x] = bias[threadIdx.x];
+    if (threadIdx.x < kConv0Out) bs[threadIdx.x] = (br ? p.bias[1] : p.bias[0])[threadIdx.x];
     __syncthreads();
-    const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;  // one pixel per thread (the grid covers P)
-    if (p < P) {
-        const uint32_t t = p / (uint32_t)Wo, wo = p - t * (uint32_t)Wo;
-        const uint32_t n = t / (uint32_t)Ho, ho = t - n * (uint32_t)Ho;
+    const uint32_t g = blockIdx.x * blockDim.x + threadIdx.x;  // pixels 4g .. 4g + 3
+    const uint32_t gc = min(g, quads - 1);                     // threads past the end repeat the last
+    const int Ho = H / 2;
+    const int wq = (int)(gc & ((1u << lwo4) - 1)), ho = (int)((gc >> lwo4) % (uint32_t)Ho);
+    const size_t n = (gc >> lwo4) / (uint32_t)Ho;
+    const __nv_bfloat16 *img = (br ? p.x[1] : p.x[0]) + n * H * H;
+    unsigned long long acc[4][kConv0Out / 2];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int j = 0; j < kConv0Out / 2; ++j) acc[q][j] = 0ull;
+#pragma unroll
+    for (int ky = 0; ky < 3; ++ky) {
+        const int h = 2 * ho - 1 + ky;  // < H: only the row above the image is missing
         float v[9];
+        if (h >= 0) {  // columns 8 wq - 1 .. 8 wq + 7
+            const __nv_bfloat16 *row = img + (size_t)h * H + 8 * wq;
+            const uint4 x = __ldg(reinterpret_cast<const uint4 *>(row));
+            const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
+            v[0] = wq > 0 ? __bfloat162float(row[-1]) : 0.f;
 #pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            const int h = 2 * (int)ho - 1 + k / 3, ww = 2 * (int)wo - 1 + k % 3;
-            v[k] = (h >= 0 && h < H && ww >= 0 && ww < W) ? __bfloat162float(x[((size_t)n * H + h) * W + ww]) : 0.f;
+            for (int i = 0; i < 4; ++i) {  // bf16 = the upper half of an fp32
+                v[2 * i + 1] = __uint_as_float(xs[i] << 16);
+                v[2 * i + 2] = __uint_as_float(xs[i] & 0xFFFF0000u);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) v[i] = 0.f;
         }
-        __align__(16) __nv_bfloat16 o[kConv0Out];
 #pragma unroll
-        for (int co = 0; co < kConv0Out; ++co) {
-            float acc = 0.f;
+        for (int kx = 0; kx < 3; ++kx) {
+            const ulonglong2 *w4 = reinterpret_cast<const ulonglong2 *>(ws[3 * ky + kx]);
+            unsigned long long vv[4];
 #pragma unroll
-            for (int k = 0; k < 9; ++k) acc = fmaf(v[k], ws[co][k], acc);
-            o[co] = __float2bfloat16(fmaxf(acc + bs[co], 0.f));
+            for (int q = 0; q < 4; ++q) vv[q] = pack2(v[2 * q + kx], v[2 * q + kx]);
+#pragma unroll
+            for (int j = 0; j < kConv0Out / 4; ++j) {
+                const ulonglong2 wj = w4[j];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    fma2(acc[q][2 * j], vv[q], wj.x);
+                    fma2(acc[q][2 * j + 1], vv[q], wj.y);
+                }
+            }
         }
-        uint4 *dst = reinterpret_cast<uint4 *>(y + (size_t)p * kConv0Out);
-        dst[0] = *reinterpret_cast<const uint4 *>(&o[0]);
-        dst[1] = *reinterpret_cast<const uint4 *>(&o[8]);
+    }
+    // A warp's 4 KB of output goes through shared memory (16-byte pieces
+    // swizzled by lane), so that its stores are contiguous.
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        uint32_t o[kConv0Out / 2];
+#pragma unroll
+        for (int j = 0; j < kConv0Out / 2; ++j) {
+            const float2 a = unpack2(acc[q][j]);
+            const __nv_bfloat162 h =
+                __floats2bfloat162_rn(fmaxf(a.x + bs[2 * j], 0.f), fmaxf(a.y + bs[2 * j + 1], 0.f));
+            o[j] = *reinterpret_cast<const uint32_t *>(&h);
+        }
+        out_s[threadIdx.x][(2 * q) ^ (lane & 7)] = make_uint4(o[0], o[1], o[2], o[3]);
+        out_s[threadIdx.x][(2 * q + 1) ^ (lane & 7)] = make_uint4(o[4], o[5], o[6], o[7]);
+    }
+    __syncwarp();
+    const uint32_t g0 = g - lane;
+    uint4 *dst = reinterpret_cast<uint4 *>((br ? p.y[1] : p.y[0]) + (size_t)g0 * 4 * kConv0Out);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int id = 32 * i + lane, from = id >> 3;
+        if (g0 + from < quads) dst[id] = out_s[threadIdx.x - lane + from][(id & 7) ^ (from & 7)];
     }
 }
 
@@ -374,16 +443,28 @@ __global__ void transpose_kernel(const __nv_bfloat16 *__restrict__ in, int64_t R
     }
 }
 
-// feat[n][c] = mean over the H*W positions of y[n][.][.][c].
-__global__ void avgpool_kernel(const __nv_bfloat16 *__restrict__ y, int Nb, int HW, int C, float *__restrict__ feat) {
-    const int64_t total = (int64_t)Nb * C;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int c = (int)(idx % C);
-        const int64_t n = idx / C;
-        float s = 0.f;
-        for (int i = 0; i < HW; ++i) s += __bfloat162float(y[(n * HW + i) * C + c]);
-        feat[idx] = s / (float)HW;
+// Average pooling and linear head of both branches (blockIdx.y), one CTA of
+// 256 threads (one per channel) per example.
+__global__ void __launch_bounds__(256) pool_head_kernel(const HeadPair p, int HW) {
+    constexpr int C = 256;
+    __shared__ float warp_sum[C / 32];
+    const int n = blockIdx.x, c = threadIdx.x;
+    const bool br = blockIdx.y;
+    const __nv_bfloat16 *y = (br ? p.y[1] : p.y[0]) + (size_t)n * HW * C + c;
+    float s = 0.f;
+#pragma unroll 8
+    for (int i = 0; i < HW; ++i) s += __bfloat162float(y[(size_t)i * C]);
+    s /= (float)HW;
+    (br ? p.feat[1] : p.feat[0])[(size_t)n * C + c] = s;
+    float d = s * (br ? p.w[1] : p.w[0])[c];
+#pragma unroll
+    for (int o = 16; o; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+    if ((c & 31) == 0) warp_sum[c >> 5] = d;
+    __syncthreads();
+    if (c == 0) {
+        float t = 0.f;
+        for (int w = 0; w < C / 32; ++w) t += warp_sum[w];
+        (br ? p.logit[1] : p.logit[0])[n] = t + (br ? p.b[1] : p.b[0])[0];
     }
 }
 
@@ -398,17 +479,6 @@ __global__ void avgpool_back_kernel(const float *__restrict__ dfeat, const __nv_
         const float g = __bfloat162float(y[idx]) > 0.f ? dfeat[n * C + c] / (float)HW : 0.f;
         dz[idx] = __float2bfloat16(g);
     }
-}
-
-// logit[n] = feat[n] . w + b, one warp per example.
-__global__ void head_kernel(const float *__restrict__ feat, int Nb, int C, const float *__restrict__ w,
-                            const float *__restrict__ b, float *__restrict__ logit) {
-    const int n = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32, lane = threadIdx.x & 31;
-    if (n >= Nb) return;
-    float s = 0.f;
-    for (int c = lane; c < C; c += 32) s += feat[(int64_t)n * C + c] * w[c];
-    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) logit[n] = s + b[0];
 }
 
 __device__ __forceinline__ float sigmoidf(float x) { return 1.f / (1.f + expf(-x)); }
@@ -532,20 +602,6 @@ __global__ void to_bf16_kernel(const float *__restrict__ a, int64_t n, __nv_bflo
 // against one load, one address and one add per bin and row.
 constexpr int kFeatRows = 32;
 constexpr int kFeatStage = 8 * 336;  // floats of one stage
-
-__device__ __forceinline__ void add2(unsigned long long &a, unsigned long long b) {
-    asm("add.rn.f32x2 %0, %0, %1;" : "+l"(a) : "l"(b));
-}
-__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ float2 unpack2(unsigned long long v) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
 
 template <int R>
 __global__ void __launch_bounds__(32 * kFeatRows / R) features_raw_kernel(const float *__restrict__ sub, int T_in,
@@ -810,11 +866,16 @@ int cnn_im2col(const __nv_bfloat16 *x, int Nb, int H, int W, int C, int stride, 
     return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
 }
 
-int cnn_conv0(const __nv_bfloat16 *x, int Nb, int H, int W, int Ho, int Wo, const __nv_bfloat16 *w, int Kp,
-              const float *bias, __nv_bfloat16 *y, cudaStream_t st) {
-    const int64_t P = (int64_t)Nb * Ho * Wo;
-    if (P >= ((int64_t)1 << 31) || Kp < 9 || (reinterpret_cast<uintptr_t>(y) & 15)) return SP_ELIMIT;
-    conv0_kernel<<<(unsigned)((P + 255) / 256), 256, 0, st>>>(x, H, W, Ho, Wo, (uint32_t)P, w, Kp, bias, y);
+int cnn_conv0(const ConvPair &p, int Nb, int H, int Kp, cudaStream_t st) {
+    const int Ho = H / 2;
+    const int64_t P = (int64_t)Nb * Ho * Ho;
+    uintptr_t all = 0;
+    for (int b = 0; b < 2; ++b) all |= reinterpret_cast<uintptr_t>(p.x[b]) | reinterpret_cast<uintptr_t>(p.y[b]);
+    int lwo4 = 0;
+    while ((4 << lwo4) < Ho) ++lwo4;
+    if (P >= ((int64_t)1 << 31) || Kp < 9 || (all & 15) || (4 << lwo4) != Ho) return SP_ELIMIT;
+    const uint32_t quads = (uint32_t)(P / 4);
+    conv0_kernel<<<dim3((quads + 255) / 256, 2), 256, 0, st>>>(p, H, lwo4, quads, Kp);
     note_launch();
     return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
 }
@@ -842,8 +903,8 @@ int cnn_transpose(const __nv_bfloat16 *in, int64_t R, int64_t C, __nv_bfloat16 *
     return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
 }
 
-int cnn_avgpool(const __nv_bfloat16 *y, int Nb, int HW, int C, float *feat, cudaStream_t st) {
-    avgpool_kernel<<<grid_for((int64_t)Nb * C), 256, 0, st>>>(y, Nb, HW, C, feat);
+int cnn_pool_head(const HeadPair &p, int Nb, int HW, cudaStream_t st) {
+    pool_head_kernel<<<dim3((unsigned)Nb, 2), 256, 0, st>>>(p, HW);
     note_launch();
     return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
 }
@@ -851,12 +912,6 @@ int cnn_avgpool(const __nv_bfloat16 *y, int Nb, int HW, int C, float *feat, cuda
 int cnn_avgpool_back(const float *dfeat, const __nv_bfloat16 *y, int Nb, int HW, int C, __nv_bfloat16 *dz,
                      cudaStream_t st) {
     avgpool_back_kernel<<<grid_for((int64_t)Nb * HW * C), 256, 0, st>>>(dfeat, y, Nb, HW, C, dz);
-    note_launch();
-    return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
-}
-
-int cnn_head(const float *feat, int Nb, int C, const float *w, const float *b, float *logit, cudaStream_t st) {
-    head_kernel<<<(Nb + 7) / 8, 256, 0, st>>>(feat, Nb, C, w, b, logit);
     note_launch();
     return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
 }

@@ -17,14 +17,15 @@
 // (tcgen05.ld) and apply the epilogue.  Every wait is bounded; a wait that
 // runs out skips the epilogue and sets the status word.
 //
-// Convolutions with short K (cnn_conv_tc) run as implicit GEMMs: A's rows are
-// output pixels' 3x3 patches, gathered by warps 2 and 3 from the NHWC input
-// straight into the swizzled shared-memory layout (two stages, so that more
-// CTAs share an SM), and no patch matrix is written to global memory.
+// Convolutions (cnn_conv_tc) run as implicit GEMMs in a kernel of their own:
+// a tap's 128 x C operand is a strided box of the NHWC input, fetched by one
+// tensor-memory-access copy per 64 channels.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
+#include <climits>
 #include <mutex>
 
 #include "sp_cnn_internal.h"
@@ -73,53 +74,14 @@ __device__ __forceinline__ bool mbar_wait_tc(uint32_t bar, uint32_t parity) {
     return true;
 }
 
-// Implicit-GEMM convolution geometry (3x3, stride 2, zero padding 1): A's
-// row p is output pixel p = (n, ho, wo) of an NHWC bf16 input x [Nb][H][W][C],
-// column k = tap * C + c with tap = 3 * ky + kx -- the layout of the im2col
-// matrix, never written out.  C, Ho and Wo are powers of two (shifts).
-struct ConvGeom {
-    const __nv_bfloat16 *x;
-    int H, W;
-    int lc, lwo, lho;  // log2 of C, Wo, Ho
-};
-
-// One stage's A tile (128 rows x 64 columns of K) gathered by the 64 threads
-// of warps 2 and 3 into the 128-byte-swizzled K-major layout that the TMA
-// copies produce: 16-byte chunk j of row r at chunk j ^ (r & 7) of the
-// row's 128 bytes.  Taps past the ninth and pixels outside the image are
-// zeros.
-__device__ __forceinline__ void gather_a(const ConvGeom &g, int M, int m0, int k0, uint8_t *sa, int t) {
-    const int C = 1 << g.lc;
-    uint4 v[16];  // all sixteen loads in flight before the first store
-#pragma unroll
-    for (int q = 0; q < 16; ++q) {
-        const int cid = t + 64 * q, r = cid >> 3, j = cid & 7;
-        const int k = k0 + 8 * j, tap = k >> g.lc, c0 = k & (C - 1), p = m0 + r;
-        v[q] = make_uint4(0u, 0u, 0u, 0u);
-        if (p < M && tap < 9) {
-            const int wo = p & ((1 << g.lwo) - 1), t2 = p >> g.lwo;
-            const int ho = t2 & ((1 << g.lho) - 1), n = t2 >> g.lho;
-            const int h = 2 * ho - 1 + tap / 3, w = 2 * wo - 1 + tap % 3;
-            if (h >= 0 && h < g.H && w >= 0 && w < g.W)
-                v[q] = __ldg(reinterpret_cast<const uint4 *>(g.x + (((int64_t)n * g.H + h) * g.W + w) * C + c0));
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < 16; ++q) {
-        const int cid = t + 64 * q, r = cid >> 3, j = cid & 7;
-        *reinterpret_cast<uint4 *>(sa + r * 128 + ((j ^ (r & 7)) << 4)) = v[q];
-    }
-}
-
-template <int EPI, int BN, bool GATHER = false>
+template <int EPI, int BN>
 __global__ void __launch_bounds__(128) gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA,
                                                       const __grid_constant__ CUtensorMap tmB, int M, int N,
                                                       int kb_per_split, int kb_total, float *__restrict__ Cf,
                                                       __nv_bfloat16 *__restrict__ Cb, int64_t ldc,
-                                                      const float *__restrict__ bias, ConvGeom geom) {
+                                                      const float *__restrict__ bias) {
     constexpr int A_BYTES = kTcBM * kTcBK * 2, B_BYTES = BN * kTcBK * 2, STAGE = A_BYTES + B_BYTES;
-    // stages of the ring; gathered A: two, so that more CTAs (and gathering warps) fit on an SM
-    constexpr int NS = GATHER ? 2 : kTcStages;
+    constexpr int NS = kTcStages;
     constexpr int NCOL = BN < 32 ? 32 : BN;  // tensor-memory columns: a power of two >= 32
     static_assert(BN % 16 == 0 && BN >= 16 && BN <= 256 && (NCOL & (NCOL - 1)) == 0, "MMA N");
     extern __shared__ uint8_t smem_raw[];
@@ -140,8 +102,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const __grid_constant__ CU
     }
     if (threadIdx.x == 32) {
         for (int s = 0; s < NS; ++s) {
-            // gathered A: the B copy's arrival plus one per gathering warp
-            mbar_init_tc(full0 + 8 * s, GATHER ? 3 : 1);
+            mbar_init_tc(full0 + 8 * s, 1);
             mbar_init_tc(empty0 + 8 * s, 1);
         }
         mbar_init_tc(done, 1);
@@ -160,16 +121,15 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const __grid_constant__ CU
             if (!ok) break;
             const uint32_t fb = full0 + 8 * s;
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb),
-                         "r"(GATHER ? B_BYTES : STAGE)
+                         "r"(STAGE)
                          : "memory");
             const int k0 = (kb_lo + i) * kTcBK;
             uint8_t *sa = smem + s * STAGE;
-            if (!GATHER)
-                asm volatile(
-                    "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, "
-                    "%3}], [%4];" ::"r"(s_addr32(sa)),
-                    "l"(&tmA), "r"(k0), "r"(m0), "r"(fb)
-                    : "memory");
+            asm volatile(
+                "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
+                "[%4];" ::"r"(s_addr32(sa)),
+                "l"(&tmA), "r"(k0), "r"(m0), "r"(fb)
+                : "memory");
             asm volatile(
                 "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
                 "[%4];" ::"r"(s_addr32(sa + A_BYTES)),
@@ -199,21 +159,6 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const __grid_constant__ CU
         if (ok)
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(done)
                          : "memory");
-    } else if (GATHER && warp >= 2) {  // A gatherers: warps 2 and 3
-        for (int i = 0; i < kb_n && ok; ++i) {
-            const int s = i % NS;
-            if (i >= NS) {  // the stage's last MMAs have read it (lane 0 waits, the warp follows)
-                int w_ok = 1;
-                if (lane == 0) w_ok = mbar_wait_tc(empty0 + 8 * s, ((i / NS) - 1) & 1);
-                ok = __shfl_sync(0xffffffffu, w_ok, 0) != 0;
-                if (!ok) break;
-            }
-            gather_a(geom, M, m0, (kb_lo + i) * kTcBK, smem + s * STAGE, threadIdx.x - 64);
-            // generic-proxy stores, read next by the tensor cores' async proxy
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(full0 + 8 * s) : "memory");
-        }
     }
     // Everyone waits for the last MMA (a role that gave up lets the wait run out).
     if (kb_n > 0) ok = mbar_wait_tc(done, 0) && ok;
@@ -266,11 +211,31 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(const __grid_constant__ CU
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(NCOL) : "memory");
 }
 
-template <int EPI, int BN, bool GATHER = false>
+template <int BN>
 constexpr int tc_smem_bytes() {
-    constexpr int S = GATHER ? 2 : kTcStages;
-    return 1024 + S * (kTcBM * kTcBK * 2 + BN * kTcBK * 2) + 8 * (2 * S + 1) + 16;
+    return 1024 + kTcStages * (kTcBM * kTcBK * 2 + BN * kTcBK * 2) + 8 * (2 * kTcStages + 1) + 16;
 }
+
+// Sets a kernel's dynamic shared-memory limit once per device.
+struct SmemLimit {
+    std::mutex lock;
+    bool configured[64] = {};
+    int set(const void *kernel, int bytes) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+            cudaGetLastError();
+            return SP_ECUDA;
+        }
+        std::lock_guard<std::mutex> guard(lock);
+        if (configured[dev]) return SP_OK;
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            return SP_ECUDA;
+        }
+        configured[dev] = true;
+        return SP_OK;
+    }
+};
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
@@ -303,33 +268,15 @@ bool make_map(CUtensorMap *m, const __nv_bfloat16 *base, int64_t rows, int64_t c
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int EPI, int BN, bool GATHER = false>
+template <int EPI, int BN>
 int launch_tc(const CUtensorMap &ta, const CUtensorMap &tb, int M, int N, int kb_per_split, int kb_total, int nz,
-              float *Cf, __nv_bfloat16 *Cb, int64_t ldc, const float *bias, cudaStream_t st,
-              const ConvGeom &geom = ConvGeom{}) {
-    constexpr int smem = tc_smem_bytes<EPI, BN, GATHER>();
-    static std::mutex lock;
-    static bool configured[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
-        cudaGetLastError();
-        return SP_ECUDA;
-    }
-    {
-        std::lock_guard<std::mutex> guard(lock);
-        if (!configured[dev]) {
-            if (cudaFuncSetAttribute(gemm_tc_kernel<EPI, BN, GATHER>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     smem) !=
-                cudaSuccess) {
-                cudaGetLastError();
-                return SP_ECUDA;
-            }
-            configured[dev] = true;
-        }
-    }
+              float *Cf, __nv_bfloat16 *Cb, int64_t ldc, const float *bias, cudaStream_t st) {
+    static SmemLimit limit;
+    const int rc = limit.set(reinterpret_cast<const void *>(gemm_tc_kernel<EPI, BN>), tc_smem_bytes<BN>());
+    if (rc) return rc;
     const dim3 grid((unsigned)((N + BN - 1) / BN), (unsigned)((M + kTcBM - 1) / kTcBM), (unsigned)nz);
-    gemm_tc_kernel<EPI, BN, GATHER>
-        <<<grid, 128, smem, st>>>(ta, tb, M, N, kb_per_split, kb_total, Cf, Cb, ldc, bias, geom);
+    gemm_tc_kernel<EPI, BN>
+        <<<grid, 128, tc_smem_bytes<BN>(), st>>>(ta, tb, M, N, kb_per_split, kb_total, Cf, Cb, ldc, bias);
     note_launch();
     return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
 }
@@ -344,6 +291,221 @@ int dispatch_bn(int bn, const CUtensorMap &ta, const CUtensorMap &tb, int M, int
         case 128: return launch_tc<EPI, 128>(ta, tb, M, N, kps, kbt, nz, Cf, Cb, ldc, bias, st);
         default: return launch_tc<EPI, 256>(ta, tb, M, N, kps, kbt, nz, Cf, Cb, ldc, bias, st);
     }
+}
+
+
+// ---- 3x3 stride-2 convolution (zero padding 1) + bias + ReLU, both branches ----
+// Implicit GEMM of 128 output pixels x BN = Cout channels per CTA, K = 9 taps x
+// C input channels.  The 128 pixels are TR = 128 / Wo rows of an image (or
+// whole images), so a tap's operand is one box of the NHWC input with every
+// second column and row (the tensor map's element strides), zeros outside the
+// image (which is the padding): rows of min(C, 64) channels, K-major, in the
+// swizzle of that width -- no patch matrix and no gathering threads.  The
+// layers are bound by latency and by L2 (they read 9/4 of their input); warps 0
+// and 1 copy and multiply through a ring of NS stages, one stage per tap and 64
+// channels, and all four warps read the accumulator back.  blockIdx.y is the
+// branch: both networks' layers run in one launch.  Both branches at batch 256,
+// layers 1-4: 305, 149, 104, 67 us with patches gathered by two warps (the
+// last by im2col) -> 140, 61, 52, 35; at batch 5: 21, 30, 49, 38 -> 8, 9, 10, 19.
+struct ConvMaps {
+    CUtensorMap a[2], b[2];
+};
+struct ConvOut {
+    const float *bias[2];
+    __nv_bfloat16 *y[2];
+};
+
+template <int C>
+struct ConvShape {
+    static constexpr int KC = C < 64 ? C : 64;           // channels per stage
+    static constexpr int STEPS = 9 * (C / KC);
+    static constexpr int BN = 2 * C;                     // every layer doubles the channels
+    static constexpr int A_BYTES = kTcBM * KC * 2, B_BYTES = BN * KC * 2, STAGE = A_BYTES + B_BYTES;
+    static constexpr int NS = C == 16 ? 9 : C == 32 ? 6 : 4;
+    static constexpr int SMEM = 1024 + NS * STAGE + 8 * (2 * NS + 1) + 16;
+    static constexpr uint64_t SWIZZLE = KC == 16 ? 6 : KC == 32 ? 4 : 2;  // 32, 64, 128 bytes
+    static constexpr uint64_t SBO = 8 * KC * 2;          // 8 rows
+    static_assert(A_BYTES % 1024 == 0 && B_BYTES % 1024 == 0 && BN >= 32 && BN <= 256 && SMEM <= 227 * 1024, "stage");
+};
+
+template <int C>
+__device__ __forceinline__ uint64_t conv_desc(uint32_t addr) {
+    using S = ConvShape<C>;
+    return (uint64_t)((addr & 0x3FFFF) >> 4) | ((uint64_t)(16 >> 4) << 16) | ((S::SBO >> 4) << 32) |
+           ((uint64_t)1 << 46) | (S::SWIZZLE << 61);
+}
+
+template <int C>
+__global__ void __launch_bounds__(128) conv_tc_kernel(const __grid_constant__ ConvMaps maps, const ConvOut out, int M,
+                                                      int lwo) {
+    using S = ConvShape<C>;
+    constexpr int NS = S::NS, BN = S::BN;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = smem_raw + ((1024 - (s_addr32(smem_raw) & 1023)) & 1023);  // swizzle atoms 1024-aligned
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + NS * S::STAGE);       // full[NS], empty[NS], done
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * NS + 1);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, branch = blockIdx.y;
+    const int m0 = blockIdx.x * kTcBM;
+    const uint32_t full0 = s_addr32(bars), empty0 = s_addr32(bars + NS), done = s_addr32(bars + 2 * NS);
+
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s_addr32(tmem_slot)),
+                     "r"(BN)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (threadIdx.x == 32) {
+        for (int s = 0; s < NS; ++s) {
+            mbar_init_tc(full0 + 8 * s, 1);
+            mbar_init_tc(empty0 + 8 * s, 1);
+        }
+        mbar_init_tc(done, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = *tmem_slot;
+    bool ok = true;
+
+    if (warp == 0 && lane == 0) {  // copies
+        const int n = m0 >> (2 * lwo), ho = (m0 >> lwo) & ((1 << lwo) - 1);
+        for (int i = 0; i < S::STEPS && ok; ++i) {
+            const int s = i % NS;
+            if (i >= NS) ok = mbar_wait_tc(empty0 + 8 * s, ((i / NS) - 1) & 1);
+            if (!ok) break;
+            const uint32_t fb = full0 + 8 * s;
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb), "r"(S::STAGE) : "memory");
+            const int tap = i / (C / S::KC), c0 = (i % (C / S::KC)) * S::KC;
+            uint8_t *sa = smem + s * S::STAGE;
+            asm volatile(
+                "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
+                "%5}], [%6];" ::"r"(s_addr32(sa)),
+                "l"(&maps.a[branch]), "r"(c0), "r"(tap % 3 - 1), "r"(2 * ho + tap / 3 - 1), "r"(n), "r"(fb)
+                : "memory");
+            asm volatile(
+                "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
+                "[%4];" ::"r"(s_addr32(sa + S::A_BYTES)),
+                "l"(&maps.b[branch]), "r"(tap * C + c0), "r"(0), "r"(fb)
+                : "memory");
+        }
+    } else if (warp == 1 && lane == 0) {  // multiplications
+        for (int i = 0; i < S::STEPS && ok; ++i) {
+            const int s = i % NS;
+            ok = mbar_wait_tc(full0 + 8 * s, (i / NS) & 1);
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t sa = s_addr32(smem + s * S::STAGE), sb = sa + S::A_BYTES;
+#pragma unroll
+            for (int ks = 0; ks < S::KC / 16; ++ks) {
+                const uint32_t acc = (i > 0 || ks > 0) ? 1u : 0u;
+                asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                             "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
+                             "l"(conv_desc<C>(sa + ks * 32)), "l"(conv_desc<C>(sb + ks * 32)), "r"(mma_idesc(BN)),
+                             "r"(acc)
+                             : "memory");
+            }
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                             empty0 + 8 * s)
+                         : "memory");
+        }
+        if (ok)
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(done)
+                         : "memory");
+    }
+    // Everyone waits for the last MMA (a role that gave up lets the wait run out).
+    ok = mbar_wait_tc(done, 0) && ok;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    ok = !__syncthreads_or(!ok);
+    if (ok) {
+        // 32 columns at a time: bias, ReLU and rounding by row, then through
+        // shared memory (the stages are free) so that four lanes store a row's
+        // 64 bytes together.
+        const float *bias = branch ? out.bias[1] : out.bias[0];
+        const int row0 = m0 + warp * 32;
+        __nv_bfloat16 *y = (branch ? out.y[1] : out.y[0]) + (int64_t)row0 * BN;
+        uint4 *buf = reinterpret_cast<uint4 *>(smem) + warp * 128;
+#pragma unroll 1
+        for (int c0 = 0; c0 < BN; c0 += 32) {
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                uint32_t v[16], o[8];
+                const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(c0 + 16 * half);
+                asm volatile(
+                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
+                    "[%16];"
+                    : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+                      "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
+                      "=r"(v[15])
+                    : "r"(taddr));
+                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int c = c0 + 16 * half + 2 * j;
+                    const __nv_bfloat162 h = __floats2bfloat162_rn(fmaxf(__uint_as_float(v[2 * j]) + bias[c], 0.f),
+                                                                   fmaxf(__uint_as_float(v[2 * j + 1]) + bias[c + 1], 0.f));
+                    o[j] = *reinterpret_cast<const uint32_t *>(&h);
+                }
+                const int s = (lane >> 1) & 3;
+                buf[4 * lane + ((2 * half) ^ s)] = make_uint4(o[0], o[1], o[2], o[3]);
+                buf[4 * lane + ((2 * half + 1) ^ s)] = make_uint4(o[4], o[5], o[6], o[7]);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int r = 8 * i + (lane >> 2), c = lane & 3;
+                if (row0 + r < M)
+                    *reinterpret_cast<uint4 *>(y + (int64_t)r * BN + c0 + 8 * c) = buf[4 * r + (c ^ ((r >> 1) & 3))];
+            }
+            __syncwarp();
+        }
+    } else if (threadIdx.x == 0) {
+        atomicOr(&g_tc_status, 1);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(BN) : "memory");
+}
+
+template <int C>
+int launch_conv(const ConvPair &p, int Nb, int H, int Kp, cudaStream_t st) {
+    using S = ConvShape<C>;
+    auto fn = encode_fn();
+    if (!fn) return SP_ELIMIT;
+    const int Wo = H / 2, lwo = Wo == 64 ? 6 : Wo == 32 ? 5 : Wo == 16 ? 4 : 3;
+    const int rows = std::min(Wo, kTcBM / Wo), images = kTcBM / (rows * Wo);  // of a tile
+    const CUtensorMapSwizzle sw = S::KC == 16 ? CU_TENSOR_MAP_SWIZZLE_32B
+                                  : S::KC == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                                : CU_TENSOR_MAP_SWIZZLE_128B;
+    ConvMaps maps;
+    ConvOut out;
+    for (int b = 0; b < 2; ++b) {
+        const cuuint64_t ad[4] = {C, (cuuint64_t)H, (cuuint64_t)H, (cuuint64_t)Nb};
+        const cuuint64_t as[3] = {C * 2, (cuuint64_t)H * C * 2, (cuuint64_t)H * H * C * 2};
+        // every second column and row: the box spans twice what it holds
+        const cuuint32_t ab[4] = {S::KC, (cuuint32_t)(2 * Wo), (cuuint32_t)(2 * rows), (cuuint32_t)images};
+        const cuuint32_t ae[4] = {1, 2, 2, 1};
+        const cuuint64_t bd[2] = {(cuuint64_t)(9 * C), S::BN};
+        const cuuint64_t bs[1] = {(cuuint64_t)Kp * 2};
+        const cuuint32_t bb[2] = {S::KC, S::BN}, be[2] = {1, 1};
+        if (fn(&maps.a[b], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<__nv_bfloat16 *>(p.x[b]), ad, as, ab, ae,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS ||
+            fn(&maps.b[b], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<__nv_bfloat16 *>(p.w[b]), bd, bs, bb, be,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return SP_ELIMIT;
+        out.bias[b] = p.bias[b];
+        out.y[b] = p.y[b];
+    }
+    static SmemLimit limit;
+    const int rc = limit.set(reinterpret_cast<const void *>(conv_tc_kernel<C>), S::SMEM);
+    if (rc) return rc;
+    const int M = Nb * Wo * Wo;
+    conv_tc_kernel<C><<<dim3((unsigned)((M + kTcBM - 1) / kTcBM), 2), 128, S::SMEM, st>>>(maps, out, M, lwo);
+    note_launch();
+    return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
 }
 
 }  // namespace
@@ -374,45 +536,25 @@ int cnn_gemm_tc(int epi, const __nv_bfloat16 *A, int64_t lda, const __nv_bfloat1
     return dispatch_bn<kEpiSplit>(bn, ta, tb, M, N, kps, kbt, nz, Cf, Cb, ldc, bias, st);
 }
 
-// 3x3 stride-2 convolution (zero padding 1) with bias and ReLU as an implicit
-// GEMM on the tensor cores: y [Nb*Ho*Wo][N] = relu(patches(x) * w^T + bias),
-// the patches gathered into shared memory by the kernel.  SP_ELIMIT when the
-// shapes do not suit it (the caller then uses im2col + cnn_gemm).
-int cnn_conv_tc(const __nv_bfloat16 *x, int Nb, int H, int W, int C, int Ho, int Wo, const __nv_bfloat16 *w, int Kp,
-                int N, const float *bias, __nv_bfloat16 *y, cudaStream_t st) {
-    auto lg = [](int v) {
-        int l = 0;
-        while ((1 << l) < v) ++l;
-        return (1 << l) == v ? l : -1;
-    };
-    const int lc = lg(C), lwo = lg(Wo), lho = lg(Ho);
-    const int64_t M = (int64_t)Nb * Ho * Wo;
-    // Long K (9C > 576: the 128-channel layer) keeps more stages in flight with TMA copies of a
-    // written patch matrix than two stages of gathered patches do: left to im2col + cnn_gemm.
-    if (lc < 3 || 9 * C > 576 || lwo < 0 || lho < 0 || H != 2 * Ho || W != 2 * Wo || M < 64 || M > INT32_MAX ||
-        N % 16 || N < 16 ||
-        N > 256 || Kp < 9 * C || Kp % 8 || !bias || (reinterpret_cast<uintptr_t>(x) & 15) ||
-        (reinterpret_cast<uintptr_t>(w) & 15) || (reinterpret_cast<uintptr_t>(y) & 15))
+// Layers 1 to 4 of both branches (the header comment of conv_tc_kernel).
+// SP_ELIMIT when the shapes do not suit it (the caller then uses im2col +
+// cnn_gemm).
+int cnn_conv_tc(const ConvPair &p, int Nb, int H, int C, int N, int Kp, cudaStream_t st) {
+    uintptr_t all = 0;
+    for (int b = 0; b < 2; ++b) {
+        if (!p.bias[b]) return SP_ELIMIT;
+        all |= reinterpret_cast<uintptr_t>(p.x[b]) | reinterpret_cast<uintptr_t>(p.w[b]) |
+               reinterpret_cast<uintptr_t>(p.y[b]);
+    }
+    if ((all & 15) || N != 2 * C || Kp < 9 * C || Kp % 8 || (H != 128 && H != 64 && H != 32 && H != 16) || Nb < 1 ||
+        (int64_t)Nb * H * H > INT32_MAX)
         return SP_ELIMIT;
-    const int bn = N <= 16 ? 16 : N <= 32 ? 32 : N <= 64 ? 64 : N <= 128 ? 128 : 256;
-    CUtensorMap tb;
-    if (!make_map(&tb, w, N, 9 * C, Kp, bn)) return SP_ELIMIT;
-    const int kbt = (9 * C + kTcBK - 1) / kTcBK;
-    ConvGeom g;
-    g.x = x;
-    g.H = H;
-    g.W = W;
-    g.lc = lc;
-    g.lwo = lwo;
-    g.lho = lho;
-    switch (bn) {  // the A map is unused with gathered A
-        case 16: return launch_tc<kEpiBiasRelu, 16, true>(tb, tb, (int)M, N, kbt, kbt, 1, nullptr, y, N, bias, st, g);
-        case 32: return launch_tc<kEpiBiasRelu, 32, true>(tb, tb, (int)M, N, kbt, kbt, 1, nullptr, y, N, bias, st, g);
-        case 64: return launch_tc<kEpiBiasRelu, 64, true>(tb, tb, (int)M, N, kbt, kbt, 1, nullptr, y, N, bias, st, g);
-        case 128:
-            return launch_tc<kEpiBiasRelu, 128, true>(tb, tb, (int)M, N, kbt, kbt, 1, nullptr, y, N, bias, st, g);
-        default:
-            return launch_tc<kEpiBiasRelu, 256, true>(tb, tb, (int)M, N, kbt, kbt, 1, nullptr, y, N, bias, st, g);
+    switch (C) {
+        case 16: return launch_conv<16>(p, Nb, H, Kp, st);
+        case 32: return launch_conv<32>(p, Nb, H, Kp, st);
+        case 64: return launch_conv<64>(p, Nb, H, Kp, st);
+        case 128: return launch_conv<128>(p, Nb, H, Kp, st);
+        default: return SP_ELIMIT;
     }
 }
 

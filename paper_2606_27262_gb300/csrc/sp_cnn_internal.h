@@ -27,29 +27,40 @@ int cnn_sum_splits(const float *part, int nz, int M, int N, int64_t ldc, float *
 int cnn_gemm_tc(int epi, const __nv_bfloat16 *A, int64_t lda, const __nv_bfloat16 *B, int64_t ldb, int M, int N,
                 int64_t K, float *Cf, __nv_bfloat16 *Cb, int64_t ldc, const float *bias, int splits, cudaStream_t st,
                 int *nz_out);
-// 3x3 stride-2 convolution (zero padding 1) + bias + ReLU as an implicit GEMM
-// on the tensor cores (patches gathered into shared memory, no im2col
-// matrix): x NHWC bf16 [Nb][H][W][C], w [N][Kp] bf16 (k = tap*C + c), y
-// [Nb*Ho*Wo][N] bf16.  C, Ho, Wo powers of two, 8 <= C <= 64, H = 2 Ho,
-// W = 2 Wo; SP_ELIMIT when a shape does not suit it.
-int cnn_conv_tc(const __nv_bfloat16 *x, int Nb, int H, int W, int C, int Ho, int Wo, const __nv_bfloat16 *w, int Kp,
-                int N, const float *bias, __nv_bfloat16 *y, cudaStream_t st);
+// The two branches' operands of a layer.
+struct ConvPair {
+    const __nv_bfloat16 *x[2], *w[2];
+    const float *bias[2];
+    __nv_bfloat16 *y[2];
+};
+// 3x3 stride-2 convolution (zero padding 1) + bias + ReLU of both branches as
+// an implicit GEMM on the tensor cores (no im2col matrix): x NHWC bf16
+// [Nb][H][H][C], w [N][Kp] bf16 (k = tap*C + c), y [Nb*(H/2)^2][N] bf16.
+// C 16..128, N = 2 C, H 128..16, powers of two; SP_ELIMIT when a shape does
+// not suit it.
+int cnn_conv_tc(const ConvPair &p, int Nb, int H, int C, int N, int Kp, cudaStream_t st);
 // Device status of the tensor-core GEMMs (bit 0: a wait ran out).
 int cnn_gemm_tc_status(int *h_status, bool clear);
 int cnn_im2col(const __nv_bfloat16 *x, int Nb, int H, int W, int C, int stride, int Ho, int Wo, int Kp,
                __nv_bfloat16 *cols, cudaStream_t st);
-// Layer 0 (one input channel, 16 outputs, 3x3, stride 2, padding 1) as a
-// direct convolution with bias and ReLU: y [Nb*Ho*Wo][16] bf16 (16-byte
-// aligned), weights w [16][Kp] bf16 (taps 0..8 used), bias [16] fp32.
-int cnn_conv0(const __nv_bfloat16 *x, int Nb, int H, int W, int Ho, int Wo, const __nv_bfloat16 *w, int Kp,
-              const float *bias, __nv_bfloat16 *y, cudaStream_t st);
+// Layer 0 of both branches (one input channel, 16 outputs, 3x3, stride 2,
+// padding 1) as a direct convolution with bias and ReLU: x [Nb][H][H] (H a
+// multiple of 8), y [Nb*(H/2)^2][16] bf16, both 16-byte aligned, weights w
+// [16][Kp] bf16 (taps 0..8 used), bias [16] fp32.
+int cnn_conv0(const ConvPair &p, int Nb, int H, int Kp, cudaStream_t st);
 int cnn_col2im_relu(const float *dcols, const __nv_bfloat16 *x, int Nb, int H, int W, int C, int stride, int Ho,
                     int Wo, int Kp, __nv_bfloat16 *dz, cudaStream_t st);
 int cnn_transpose(const __nv_bfloat16 *in, int64_t R, int64_t C, __nv_bfloat16 *out, cudaStream_t st);
-int cnn_avgpool(const __nv_bfloat16 *y, int Nb, int HW, int C, float *feat, cudaStream_t st);
+// Average pooling and linear head of both branches (C = 256 channels):
+// feat[n][c] = mean over HW of y, logit[n] = feat[n] . w + b[0].
+struct HeadPair {
+    const __nv_bfloat16 *y[2];
+    const float *w[2], *b[2];
+    float *feat[2], *logit[2];
+};
+int cnn_pool_head(const HeadPair &p, int Nb, int HW, cudaStream_t st);
 int cnn_avgpool_back(const float *dfeat, const __nv_bfloat16 *y, int Nb, int HW, int C, __nv_bfloat16 *dz,
                      cudaStream_t st);
-int cnn_head(const float *feat, int Nb, int C, const float *w, const float *b, float *logit, cudaStream_t st);
 int cnn_fuse_loss(const float *l1, const float *l2, const float *label, int Nb, float *prob, float *dl1, float *dl2,
                   float *loss, cudaStream_t st);
 int cnn_head_back(const float *feat, const float *dl, int Nb, int C, const float *w, float *dfeat, float *dw,
