@@ -606,13 +606,13 @@ constexpr int kFeatStage = 8 * 336;  // floats of one stage
 template <int R>
 __global__ void __launch_bounds__(32 * kFeatRows / R) features_raw_kernel(const float *__restrict__ sub, int T_in,
                                                                         const int32_t *__restrict__ shift, bool vec,
-                                                                        float *__restrict__ dmt_raw,
+                                                                        float *dmt_raw,
                                                                         float4 *__restrict__ part) {
     constexpr int NW = kFeatRows / R, NT = 32 * NW, NI = kImg / 32;
     __shared__ __align__(16) float win[2][kFeatStage];
     __shared__ __align__(16) uint16_t rel[kImg][kFeatRows];  // bin of a row's u = 0 in its subband's window
     __shared__ int base[kImg];                               // first bin of the window (a multiple of 4)
-    __shared__ float4 row_sum[kFeatRows];
+    __shared__ float2 col_sum[2][NI];
     __shared__ int widest;
     const int b = blockIdx.y, j0 = blockIdx.x * kFeatRows, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int u0 = (T_in - kImg) / 2;
@@ -715,43 +715,44 @@ __global__ void __launch_bounds__(32 * kFeatRows / R) features_raw_kernel(const 
             }
         }
     }
-    // Sums of each row of both images: a lane's bins in order, then a warp
-    // tree; of the block's rows: another (the same for every R).
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const int j = j0 + warp * R + r;
-        float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int r = 0; r < R; ++r)
 #pragma unroll
         for (int i = 0; i < NI; ++i) {
-            const float f = sb[(size_t)j * T_in + u0 + 32 * i + lane];
             const float2 d2 = unpack2(acc[r][i >> 1]);
-            const float d = i & 1 ? d2.y : d2.x;
-            dmt_raw[((size_t)b * kImg + j) * kImg + 32 * i + lane] = d;
-            t.x += f;
-            t.y += f * f;
-            t.z += d;
-            t.w += d * d;
+            dmt_raw[((size_t)b * kImg + j0 + warp * R + r) * kImg + 32 * i + lane] = i & 1 ? d2.y : d2.x;
+        }
+    __syncthreads();
+    // The block's sums of both images: each column's rows in order, a warp tree
+    // over 32 columns, then those in turn, whatever R is (the normalisation adds
+    // the blocks in turn).  The variance is a small difference of large sums, so
+    // this order is part of the result.
+    for (int it = warp; it < 2 * NI; it += NW) {
+        const int img = it / NI, u = (it % NI) * 32 + lane;
+        const float *col = img ? dmt_raw + ((size_t)b * kImg + j0) * kImg + u : sb + (size_t)j0 * T_in + u0 + u;
+        const int row = img ? kImg : T_in;
+        float t = 0.f, t2 = 0.f;
+#pragma unroll 16
+        for (int r = 0; r < kFeatRows; ++r) {
+            const float v = col[(size_t)r * row];
+            t += v;
+            t2 += v * v;
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-            t.x += __shfl_xor_sync(0xffffffffu, t.x, o);
-            t.y += __shfl_xor_sync(0xffffffffu, t.y, o);
-            t.z += __shfl_xor_sync(0xffffffffu, t.z, o);
-            t.w += __shfl_xor_sync(0xffffffffu, t.w, o);
+            t += __shfl_xor_sync(0xffffffffu, t, o);
+            t2 += __shfl_xor_sync(0xffffffffu, t2, o);
         }
-        if (lane == 0) row_sum[warp * R + r] = t;
+        if (lane == 0) col_sum[img][it % NI] = make_float2(t, t2);
     }
     __syncthreads();
-    if (warp == 0) {
-        float4 t = row_sum[lane];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            t.x += __shfl_xor_sync(0xffffffffu, t.x, o);
-            t.y += __shfl_xor_sync(0xffffffffu, t.y, o);
-            t.z += __shfl_xor_sync(0xffffffffu, t.z, o);
-            t.w += __shfl_xor_sync(0xffffffffu, t.w, o);
+    if (threadIdx.x < 2) {
+        float2 a = col_sum[threadIdx.x][0];
+        for (int w = 1; w < NI; ++w) {
+            a.x += col_sum[threadIdx.x][w].x;
+            a.y += col_sum[threadIdx.x][w].y;
         }
-        if (lane == 0) part[(size_t)b * (kImg / kFeatRows) + blockIdx.x] = t;
+        reinterpret_cast<float2 *>(part + (size_t)b * (kImg / kFeatRows) + blockIdx.x)[threadIdx.x] = a;
     }
 }
 
