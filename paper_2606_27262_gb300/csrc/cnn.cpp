@@ -25,8 +25,7 @@ using namespace sp;
 
 namespace {
 
-constexpr int kLayers = 5;
-constexpr int kWgradSplitBudget = 304;  // split-K CTAs per weight-gradient GEMM (2 per SM)
+constexpr int kLayers = kCnnLayers;
 constexpr int kCin[kLayers] = {1, 16, 32, 64, 128};
 constexpr int kCout[kLayers] = {16, 32, 64, 128, 256};
 constexpr int kHin[kLayers] = {256, 128, 64, 32, 16};
@@ -37,18 +36,14 @@ constexpr int kAlign = 64;  // parameter segments start at multiples of 64 eleme
 constexpr int kp_of(int l) { return ((9 * kCin[l] + 31) / 32) * 32; }
 constexpr int ho_of(int l) { return kHin[l] / 2; }
 int64_t up(int64_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
-// K splits of layer l's weight-gradient GEMM dW [Co][Kp] = dz^T [Co][P] * cols [P][Kp].
-int wgrad_splits(int l, int64_t P) {
-    const int tiles = (int)(((kCout[l] + 127) / 128) * ((kp_of(l) + 63) / 64));
-    return (int)std::max<int64_t>(1, std::min<int64_t>(P / 32, kWgradSplitBudget / tiles));
-}
+int part_cols(int l) { return l == 0 ? 10 * kCout[0] : kCout[l]; }  // of cnn_conv0_wgrad, cnn_bias_part
 
 struct Branch {
     int64_t off_w[kLayers] = {}, off_b[kLayers] = {}, off_hw = 0, off_hb = 0, n = 0;
     float *params = nullptr, *grads = nullptr, *m = nullptr, *v = nullptr;
     __nv_bfloat16 *pb = nullptr;  // bf16 mirror of params (GEMM weights)
-    __nv_bfloat16 *cols[kLayers] = {}, *y[kLayers] = {}, *dz[kLayers] = {};
-    float *feat = nullptr, *logit = nullptr, *dl = nullptr, *dfeat = nullptr;
+    __nv_bfloat16 *y[kLayers] = {}, *dz[kLayers] = {};
+    float *feat = nullptr, *logit = nullptr, *dl = nullptr;
 };
 
 }  // namespace
@@ -57,10 +52,9 @@ struct sp_cnn {
     int device = 0;
     int32_t max_batch = 0;
     Branch br[2];
-    __nv_bfloat16 *dzT = nullptr, *colsT = nullptr, *wT = nullptr;
-    float *dcols = nullptr, *prob = nullptr, *loss = nullptr;
-    float *bias_part = nullptr;  // [kBiasChunks][256] partial bias gradients
-    float *wpart = nullptr;      // split-K partials of a weight gradient (summed in order)
+    float *prob = nullptr, *loss = nullptr;
+    float *sums = nullptr;   // partial sums of layer 0's gradients and of every bias gradient
+    float *wpart = nullptr;  // partial weight gradients of a layer
     int64_t step = 0;
     bool have_grads = false;
 };
@@ -131,20 +125,14 @@ void free_cnn(sp_cnn *c) {
         cudaFree(b.v);
         cudaFree(b.pb);
         for (int l = 0; l < kLayers; ++l) {
-            cudaFree(b.cols[l]);
             cudaFree(b.y[l]);
             cudaFree(b.dz[l]);
         }
         cudaFree(b.feat);
         cudaFree(b.logit);
         cudaFree(b.dl);
-        cudaFree(b.dfeat);
     }
-    cudaFree(c->dzT);
-    cudaFree(c->colsT);
-    cudaFree(c->wT);
-    cudaFree(c->dcols);
-    cudaFree(c->bias_part);
+    cudaFree(c->sums);
     cudaFree(c->wpart);
     cudaFree(c->prob);
     cudaFree(c->loss);
@@ -170,34 +158,19 @@ int upload_params(sp_cnn *c, int br, const std::vector<float> &h) {
 int forward(sp_cnn *c, const __nv_bfloat16 *ft, const __nv_bfloat16 *dmt, int B, const float *labels, float *prob,
             cudaStream_t st) {
     // Both branches' layers go in one launch each: with a few candidates a
-    // layer is bound by its latency, not by its work.  No patch matrix in the
-    // forward pass (the backward pass builds the patches it needs for the
-    // weight gradients), the same in training and inference: the first layer
-    // directly, the others as implicit GEMMs on the tensor cores, or im2col +
-    // GEMM where a shape does not suit those.
+    // layer is bound by its latency, not by its work.
     int rc = SP_OK;
     ConvPair p;
     p.x[0] = ft;
     p.x[1] = dmt;
     for (int l = 0; l < kLayers && !rc; ++l) {
-        const int H = kHin[l], Ho = ho_of(l), Kp = kp_of(l);
         for (int bi = 0; bi < 2; ++bi) {
             Branch &b = c->br[bi];
             p.w[bi] = b.pb + b.off_w[l];
             p.bias[bi] = b.params + b.off_b[l];
             p.y[bi] = b.y[l];
         }
-        rc = l == 0 ? cnn_conv0(p, B, H, Kp, st) : cnn_conv_tc(p, B, H, kCin[l], kCout[l], Kp, st);
-        if (rc == SP_ELIMIT) {
-            rc = SP_OK;
-            for (int bi = 0; bi < 2 && !rc; ++bi) {
-                __nv_bfloat16 *cols = c->br[bi].cols[l];
-                rc = cnn_im2col(p.x[bi], B, H, H, kCin[l], 2, Ho, Ho, Kp, cols, st);
-                if (!rc)
-                    rc = cnn_gemm(kEpiBiasRelu, cols, Kp, p.w[bi], Kp, B * Ho * Ho, kCout[l], Kp, nullptr, p.y[bi],
-                                  kCout[l], p.bias[bi], 1, st);
-            }
-        }
+        rc = l == 0 ? cnn_conv0(p, B, kHin[l], kp_of(l), st) : cnn_conv_fwd(p, B, kHin[l], kCin[l], kp_of(l), st);
         p.x[0] = p.y[0];
         p.x[1] = p.y[1];
     }
@@ -220,45 +193,48 @@ int forward(sp_cnn *c, const __nv_bfloat16 *ft, const __nv_bfloat16 *dmt, int B,
 }
 
 int backward(sp_cnn *c, const __nv_bfloat16 *ft, const __nv_bfloat16 *dmt, int B, cudaStream_t st) {
-    int rc = SP_OK;
-    for (int bi = 0; bi < 2 && !rc; ++bi) {
+    HeadGrad h;
+    ColumnSums sums;
+    for (int bi = 0; bi < 2; ++bi) {
         Branch &b = c->br[bi];
         if (cudaMemsetAsync(b.grads, 0, (size_t)b.n * 4, st) != cudaSuccess) return SP_ECUDA;
-        rc = cnn_head_back(b.feat, b.dl, B, kFeat, b.params + b.off_hw, b.dfeat, b.grads + b.off_hw,
-                           b.grads + b.off_hb, st);
-        const int hw = ho_of(kLayers - 1) * ho_of(kLayers - 1);
-        if (!rc) rc = cnn_avgpool_back(b.dfeat, b.y[kLayers - 1], B, hw, kFeat, b.dz[kLayers - 1], st);
-        for (int l = kLayers - 1; l >= 0 && !rc; --l) {
-            const int Ho = ho_of(l), Kp = kp_of(l), Co = kCout[l];
-            const int64_t P = (int64_t)B * Ho * Ho;
-            rc = cnn_bias_grad(b.dz[l], P, Co, b.grads + b.off_b[l], c->bias_part, st);
-            // the layer's patches (the forward pass writes them only where it
-            // falls back to im2col)
-            if (!rc)
-                rc = cnn_im2col(l == 0 ? (bi == 0 ? ft : dmt) : b.y[l - 1], B, kHin[l], kHin[l], kCin[l], 2, Ho, Ho, Kp,
-                                b.cols[l], st);
-            // dW [Co][Kp] = dz^T [Co][P] * cols [P][Kp], split over P.
-            if (!rc) rc = cnn_transpose(b.dz[l], P, Co, c->dzT, st);
-            if (!rc) rc = cnn_transpose(b.cols[l], P, Kp, c->colsT, st);
-            const int splits = wgrad_splits(l, P);
-            int nz = 0;
-            if (!rc)
-                rc = cnn_gemm(kEpiSplit, c->dzT, P, c->colsT, P, Co, Kp, P, c->wpart, nullptr, Kp, nullptr, splits, st,
-                              &nz);
-            if (!rc) rc = cnn_sum_splits(c->wpart, nz, Co, Kp, Kp, b.grads + b.off_w[l], st);
-            if (l == 0 || rc) continue;
-            // dcols [P][Kp] = dz [P][Co] * W [Co][Kp]; then the gradient of the
-            // layer input, masked by the ReLU that produced it.
-            rc = cnn_transpose(b.pb + b.off_w[l], Co, Kp, c->wT, st);
-            if (!rc)
-                rc = cnn_gemm(kEpiStore, b.dz[l], Co, c->wT, Co, (int)P, Kp, Co, c->dcols, nullptr, Kp, nullptr, 1,
-                              st);
-            if (!rc)
-                rc = cnn_col2im_relu(c->dcols, b.y[l - 1], B, kHin[l], kHin[l], kCin[l], 2, Ho, Ho, Kp, b.dz[l - 1],
-                                     st);
-        }
+        h.feat[bi] = b.feat;
+        h.dl[bi] = b.dl;
+        h.w[bi] = b.params + b.off_hw;
+        h.y[bi] = b.y[kLayers - 1];
+        h.dz[bi] = b.dz[kLayers - 1];
+        h.dw[bi] = b.grads + b.off_hw;
+        h.db[bi] = b.grads + b.off_hb;
+        sums.dw0[bi] = b.grads + b.off_w[0];
     }
-    return rc;
+    sums.kp0 = kp_of(0);
+    int rc = cnn_head_back(h, B, ho_of(kLayers - 1) * ho_of(kLayers - 1), st);
+    float *part = c->sums;
+    for (int l = kLayers - 1; l >= 0 && !rc; --l) {
+        const int H = kHin[l], C = kCin[l], Kp = kp_of(l);
+        GradPair p{};
+        for (int bi = 0; bi < 2; ++bi) {
+            Branch &b = c->br[bi];
+            p.x[bi] = l == 0 ? (bi == 0 ? ft : dmt) : b.y[l - 1];
+            p.dz[bi] = b.dz[l];
+            p.w[bi] = b.pb + b.off_w[l];
+            p.dx[bi] = l == 0 ? nullptr : b.dz[l - 1];
+            p.dw[bi] = b.grads + b.off_w[l];
+            sums.db[bi][l] = b.grads + b.off_b[l];
+        }
+        sums.part[l] = part;
+        sums.cols[l] = part_cols(l);
+        part += (int64_t)2 * kBiasChunks * part_cols(l);
+        if (l == 0) {
+            rc = cnn_conv0_wgrad(p, B, H, const_cast<float *>(sums.part[l]), &sums.rows[l], st);
+            break;
+        }
+        rc = cnn_bias_part(p, (int64_t)B * ho_of(l) * ho_of(l), kCout[l], const_cast<float *>(sums.part[l]),
+                           &sums.rows[l], st);
+        if (!rc) rc = cnn_conv_wgrad(p, B, H, C, Kp, c->wpart, st);
+        if (!rc) rc = cnn_conv_dgrad(p, B, H, C, Kp, st);
+    }
+    return rc ? rc : cnn_column_sums(sums, st);
 }
 
 int check_batch(const sp_cnn *c, const void *ft, const void *dmt, int32_t B) {
@@ -290,12 +266,10 @@ extern "C" int sp_cnn_create(int32_t max_batch, uint64_t seed, sp_cnn **out) {
         if (!rc) rc = dalloc((void **)&b.pb, b.n * 2);
         for (int l = 0; l < kLayers && !rc; ++l) {
             const int64_t P = B * ho_of(l) * ho_of(l);
-            rc = dalloc((void **)&b.cols[l], P * kp_of(l) * 2);
-            if (!rc) rc = dalloc((void **)&b.y[l], P * kCout[l] * 2);
+            rc = dalloc((void **)&b.y[l], P * kCout[l] * 2);
             if (!rc) rc = dalloc((void **)&b.dz[l], P * kCout[l] * 2);
         }
         if (!rc) rc = dalloc((void **)&b.feat, B * kFeat * 4);
-        if (!rc) rc = dalloc((void **)&b.dfeat, B * kFeat * 4);
         if (!rc) rc = dalloc((void **)&b.logit, B * 4);
         if (!rc) rc = dalloc((void **)&b.dl, B * 4);
         if (!rc && (cudaMemset(b.m, 0, (size_t)b.n * 4) != cudaSuccess ||
@@ -303,22 +277,13 @@ extern "C" int sp_cnn_create(int32_t max_batch, uint64_t seed, sp_cnn **out) {
                     cudaMemset(b.grads, 0, (size_t)b.n * 4) != cudaSuccess))
             rc = SP_ECUDA;
     }
-    int64_t dz_max = 0, cols_max = 0, dcols_max = 0;
+    int64_t sums = 0, wpart = 0;
     for (int l = 0; l < kLayers; ++l) {
-        const int64_t P = B * ho_of(l) * ho_of(l);
-        dz_max = std::max(dz_max, P * kCout[l]);
-        cols_max = std::max(cols_max, P * kp_of(l));
-        if (l > 0) dcols_max = std::max(dcols_max, P * kp_of(l));
+        sums += (int64_t)2 * kBiasChunks * part_cols(l);
+        if (l > 0) wpart = std::max(wpart, cnn_wgrad_part_floats(max_batch, kHin[l], kCin[l], kp_of(l)));
     }
-    if (!rc) rc = dalloc((void **)&c->dzT, dz_max * 2);
-    if (!rc) rc = dalloc((void **)&c->colsT, cols_max * 2);
-    if (!rc) rc = dalloc((void **)&c->wT, (int64_t)kp_of(kLayers - 1) * kCout[kLayers - 1] * 2);
-    if (!rc) rc = dalloc((void **)&c->dcols, dcols_max * 4);
-    if (!rc) rc = dalloc((void **)&c->bias_part, (int64_t)kBiasChunks * 256 * 4);
-    int64_t wpart_max = 0;
-    for (int l = 0; l < kLayers; ++l)
-        wpart_max = std::max(wpart_max, (int64_t)wgrad_splits(l, B * ho_of(l) * ho_of(l)) * kCout[l] * kp_of(l));
-    if (!rc) rc = dalloc((void **)&c->wpart, wpart_max * 4);
+    if (!rc) rc = dalloc((void **)&c->sums, sums * 4);
+    if (!rc) rc = dalloc((void **)&c->wpart, wpart * 4);
     if (!rc) rc = dalloc((void **)&c->prob, B * 4);
     if (!rc) rc = dalloc((void **)&c->loss, 4);
     // He-normal convolution weights, zero biases, small head weights.

@@ -3,22 +3,16 @@
 // dedispersed dynamic spectrum and its DM transform; two networks, one per
 // image, fused multiplicatively into one probability).
 //
-// Every layer is built from these kernels:
-//   gemm_nt_kernel      C[M,N] = A[M,K] * B[N,K]^T, bf16 operands, fp32
-//                       accumulate on the tensor cores (mma.sync m16n8k16),
-//                       cp.async double buffering, optional split-K; the
-//                       epilogue adds a bias and applies ReLU (bf16 out),
-//                       stores fp32, or adds fp32 atomically.
-//   im2col_*_kernel     3x3 / stride / pad-1 patches of an NHWC bf16 tensor
-//                       as GEMM rows, k = (ky*3 + kx)*C + c, zero padded
-//                       (16-byte copies for C % 8 == 0 and for C == 1).
-//   col2im_relu_kernel  the adjoint of im2col (a gather, no atomics) fused
-//                       with the ReLU derivative of the layer below.
-//   transpose_kernel    bf16 [R][C] -> [C][R] (operands of the backward GEMMs).
+// The convolutions of layers 1 to 4 and their gradients are in cnn_tc.cu; here:
+//   conv0_kernel, conv0_wgrad_kernel   the one-channel first layer, directly
+//   pool_head_kernel, head_back_kernel pooling and linear head, and back
+//   fuse_loss_kernel    fused probability, loss and its derivative
+//   bias_part_kernel, column_sums_kernel   bias gradients
+//   adam_kernel         the update
 //   features_raw_kernel DM-time images of subband dynamic spectra
 //   normalise_kernel    frequency-time and DM-time images normalised to zero
-//                       mean and unit variance, as bf16.
-//   plus average pooling, the linear heads, the fused loss and Adam.
+//                       mean and unit variance, as bf16
+//   extract_kernel      subband spectra of candidates from the staged beam
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -28,9 +22,6 @@
 
 namespace sp {
 namespace {
-
-constexpr int kBM = 128, kBN = 64, kBK = 32, kPad = 8;
-constexpr int kLds = kBK + kPad;  // smem row stride (bf16): 80 bytes, conflict-free ldmatrix
 
 __device__ __forceinline__ uint32_t s_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -46,19 +37,6 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
-__device__ __forceinline__ void ldmatrix_x4(uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3, const void *p) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-                 : "r"(s_addr(p)));
-}
-__device__ __forceinline__ void mma_bf16(float *c, const uint32_t *a, uint32_t b0, uint32_t b1) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-        "{%0,%1,%2,%3};"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
 // Two fp32 lanes of a 64-bit register (one instruction, each lane rounded as by the scalar one).
 __device__ __forceinline__ void add2(unsigned long long &a, unsigned long long b) {
     asm("add.rn.f32x2 %0, %0, %1;" : "+l"(a) : "l"(b));
@@ -72,155 +50,6 @@ __device__ __forceinline__ float2 unpack2(unsigned long long v) {
     float2 r;
     asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
     return r;
-}
-
-// 256 threads: warp (wm, wn) = (warp % 4, warp / 4) owns a 32 x 32 block of
-// the 128 x 64 tile: 2 x 4 mma tiles of 16 x 8.  blockIdx.z = K split.
-template <int EPI>
-__global__ void __launch_bounds__(256) gemm_nt_kernel(const __nv_bfloat16 *__restrict__ A, int64_t lda,
-                                                      const __nv_bfloat16 *__restrict__ B, int64_t ldb, int M, int N,
-                                                      int64_t K, int64_t k_split, float *__restrict__ Cf,
-                                                      __nv_bfloat16 *__restrict__ Cb, int64_t ldc,
-                                                      const float *__restrict__ bias) {
-    __shared__ __align__(16) __nv_bfloat16 As[2][kBM][kLds];
-    __shared__ __align__(16) __nv_bfloat16 Bs[2][kBN][kLds];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int wm = warp & 3, wn = warp >> 2;
-    const int64_t m0 = (int64_t)blockIdx.y * kBM, n0 = (int64_t)blockIdx.x * kBN;
-    const int64_t k_lo = (int64_t)blockIdx.z * k_split;
-    const int64_t k_hi = min(K, k_lo + k_split);
-    const int nk = (int)((k_hi - k_lo) / kBK);
-
-    auto load = [&](int kt, int buf) {
-        const int64_t k0 = k_lo + (int64_t)kt * kBK;
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {  // A: 128 rows x 4 chunks of 8
-            const int c = tid + i * 256;
-            const int r = c >> 2, q = (c & 3) * 8;
-            const int64_t gr = m0 + r;
-            const bool ok = gr < M;
-            cp_async16(&As[buf][r][q], A + (ok ? gr : 0) * lda + k0 + q, ok);
-        }
-        {  // B: 64 rows x 4 chunks
-            const int r = tid >> 2, q = (tid & 3) * 8;
-            const int64_t gr = n0 + r;
-            const bool ok = gr < N;
-            cp_async16(&Bs[buf][r][q], B + (ok ? gr : 0) * ldb + k0 + q, ok);
-        }
-    };
-
-    float acc[2][4][4];
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.f;
-
-    if (nk > 0) {
-        load(0, 0);
-        cp_async_commit();
-    }
-    for (int kt = 0; kt < nk; ++kt) {
-        const int buf = kt & 1;
-        if (kt + 1 < nk) {
-            load(kt + 1, buf ^ 1);
-            cp_async_commit();
-            cp_async_wait<1>();
-        } else {
-            cp_async_wait<0>();
-        }
-        __syncthreads();
-#pragma unroll
-        for (int ks = 0; ks < kBK; ks += 16) {
-            uint32_t a[2][4], b[4][2];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int r = wm * 32 + i * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
-                const int c = ks + (lane >> 4) * 8;
-                ldmatrix_x4(a[i][0], a[i][1], a[i][2], a[i][3], &As[buf][r][c]);
-            }
-#pragma unroll
-            for (int jj = 0; jj < 2; ++jj) {
-                const int r = wn * 32 + jj * 16 + (lane & 7) + (lane >> 4) * 8;
-                const int c = ks + ((lane >> 3) & 1) * 8;
-                ldmatrix_x4(b[2 * jj][0], b[2 * jj][1], b[2 * jj + 1][0], b[2 * jj + 1][1], &Bs[buf][r][c]);
-            }
-#pragma unroll
-            for (int i = 0; i < 2; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) mma_bf16(acc[i][j], a[i], b[j][0], b[j][1]);
-        }
-        __syncthreads();
-    }
-
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int64_t row = m0 + wm * 32 + i * 16 + (lane >> 2) + h * 8;
-                if (row >= M) continue;
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const int64_t col = n0 + wn * 32 + j * 8 + (lane & 3) * 2 + e;
-                    if (col >= N) continue;
-                    float v = acc[i][j][2 * h + e];
-                    if (EPI == kEpiBiasRelu) {
-                        v = fmaxf(v + bias[col], 0.f);
-                        Cb[row * ldc + col] = __float2bfloat16(v);
-                    } else if (EPI == kEpiStore) {
-                        Cf[row * ldc + col] = v;
-                    } else {  // this K range's partial product
-                        Cf[(int64_t)blockIdx.z * M * ldc + row * ldc + col] = v;
-                    }
-                }
-            }
-}
-
-// cols[p][k] for p = (n, ho, wo), k = (ky*3 + kx)*C + c (k < 9C; zero up to Kp).
-// Channels a multiple of 8: one thread per (patch row p, chunk j of 8
-// columns).  Chunk j is one tap (ky, kx) = divmod(8j / C, 3) and channels
-// 8j % C .. + 7 of one pixel: a single 16-byte copy (zero outside the image
-// and past 9C).  32-bit index arithmetic (the launcher checks the sizes).
-__global__ void im2col_vec_kernel(const __nv_bfloat16 *__restrict__ x, int H, int W, int C, int stride, int Ho,
-                                  int Wo, uint32_t chunks, uint32_t total, __nv_bfloat16 *__restrict__ cols) {
-    for (uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += gridDim.x * blockDim.x) {
-        const uint32_t p = idx / chunks, j = idx - p * chunks;
-        const uint32_t k0 = j * 8u, tap = k0 / (uint32_t)C, c0 = k0 - tap * (uint32_t)C;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (tap < 9u) {
-            const uint32_t t = p / (uint32_t)Wo, wo = p - t * (uint32_t)Wo;
-            const uint32_t n = t / (uint32_t)Ho, ho = t - n * (uint32_t)Ho;
-            const int h = (int)ho * stride - 1 + (int)(tap / 3u), w = (int)wo * stride - 1 + (int)(tap % 3u);
-            if (h >= 0 && h < H && w >= 0 && w < W)
-                v = *reinterpret_cast<const uint4 *>(x + ((size_t)(n * (uint32_t)H + (uint32_t)h) * W + w) * C + c0);
-        }
-        reinterpret_cast<uint4 *>(cols)[idx] = v;
-    }
-}
-
-// One channel (the first layer): one thread per patch row, its nine taps
-// gathered and the row of Kp columns written as 16-byte stores.
-__global__ void im2col_c1_kernel(const __nv_bfloat16 *__restrict__ x, int H, int W, int stride, int Ho, int Wo,
-                                 uint32_t kp_chunks, uint32_t P, __nv_bfloat16 *__restrict__ cols) {
-    for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
-        const uint32_t t = p / (uint32_t)Wo, wo = p - t * (uint32_t)Wo;
-        const uint32_t n = t / (uint32_t)Ho, ho = t - n * (uint32_t)Ho;
-        __align__(16) __nv_bfloat16 v[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k) v[k] = __float2bfloat16(0.f);
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            const int h = (int)ho * stride - 1 + k / 3, w = (int)wo * stride - 1 + k % 3;
-            if (h >= 0 && h < H && w >= 0 && w < W) v[k] = x[((size_t)n * H + h) * W + w];
-        }
-        uint4 *dst = reinterpret_cast<uint4 *>(cols) + (size_t)p * kp_chunks;
-        dst[0] = *reinterpret_cast<const uint4 *>(&v[0]);
-        dst[1] = *reinterpret_cast<const uint4 *>(&v[8]);
-        for (uint32_t j = 2; j < kp_chunks; ++j) dst[j] = make_uint4(0u, 0u, 0u, 0u);
-    }
 }
 
 // Layer 0 (one input channel, 3x3, stride 2, zero padding 1) of both branches
@@ -319,127 +148,85 @@ __global__ void __launch_bounds__(256) conv0_kernel(const ConvPair p, int H, int
     }
 }
 
-// Any channel count (reference form, one element per thread).
-__global__ void im2col_kernel(const __nv_bfloat16 *__restrict__ x, int Nb, int H, int W, int C, int stride, int Ho,
-                              int Wo, int Kp, __nv_bfloat16 *__restrict__ cols) {
-    const int64_t total = (int64_t)Nb * Ho * Wo * Kp;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int k = (int)(idx % Kp);
-        const int64_t p = idx / Kp;
-        __nv_bfloat16 v = __float2bfloat16(0.f);
-        if (k < 9 * C) {
-            const int c = k % C, kk = k / C, ky = kk / 3, kx = kk % 3;
-            const int wo = (int)(p % Wo), ho = (int)((p / Wo) % Ho), n = (int)(p / ((int64_t)Wo * Ho));
-            const int h = ho * stride - 1 + ky, w = wo * stride - 1 + kx;
-            if (h >= 0 && h < H && w >= 0 && w < W) v = x[(((int64_t)n * H + h) * W + w) * C + c];
-        }
-        cols[idx] = v;
-    }
-}
-
-// dz[n][h][w][c] = (sum over the patches that read (h, w) of dcols) *
-// (x[n][h][w][c] > 0): the gradient of im2col's input, masked by the ReLU
-// that produced x.
-__global__ void col2im_relu_kernel(const float *__restrict__ dcols, const __nv_bfloat16 *__restrict__ x, int Nb, int H,
-                                   int W, int C, int stride, int Ho, int Wo, int Kp,
-                                   __nv_bfloat16 *__restrict__ dz) {
-    const int64_t total = (int64_t)Nb * H * W * C;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int c = (int)(idx % C);
-        const int w = (int)((idx / C) % W), h = (int)((idx / ((int64_t)C * W)) % H);
-        const int n = (int)(idx / ((int64_t)C * W * H));
-        float s = 0.f;
-        if (__bfloat162float(x[idx]) > 0.f) {
-            for (int ky = 0; ky < 3; ++ky) {
-                const int hh = h + 1 - ky;
-                if (hh < 0 || hh % stride) continue;
-                const int ho = hh / stride;
-                if (ho >= Ho) continue;
-                for (int kx = 0; kx < 3; ++kx) {
-                    const int ww = w + 1 - kx;
-                    if (ww < 0 || ww % stride) continue;
-                    const int wo = ww / stride;
-                    if (wo >= Wo) continue;
-                    s += dcols[(((int64_t)n * Ho + ho) * Wo + wo) * Kp + (ky * 3 + kx) * C + c];
-                }
+// Layer 0's weight and bias gradients: part[branch][block][k * 16 + co] = sum of
+// dz[p][co] * x[p at tap k] over the block's pixels (k = 9: of dz alone), which
+// column_sums_kernel adds in block order.  Bound by reading dz (134 MB a branch
+// at batch 256) and by the 160 fp32 sums a pixel feeds, two to an fma.f32x2: a
+// thread keeps the 80 of eight channels in registers over all its pixels, four
+// neighbours at a time.  36 us for both branches at batch 64 (as im2col,
+// transposes and a GEMM: about 400 us).
+constexpr int kW0Sums = 10 * kConv0Out, kW0Blocks = 152;  // blocks of a branch: two an SM
+__global__ void __launch_bounds__(256, 2) conv0_wgrad_kernel(const GradPair p, int H, int lwo4, uint32_t quads,
+                                                             float *__restrict__ part) {
+    __shared__ float red[8][kW0Sums];
+    const bool br = blockIdx.y;
+    const __nv_bfloat16 *img0 = br ? p.x[1] : p.x[0];
+    const uint4 *dz = reinterpret_cast<const uint4 *>(br ? p.dz[1] : p.dz[0]);
+    const int half = threadIdx.x & 1, Ho = H / 2;
+    unsigned long long acc[10][4];
+#pragma unroll
+    for (int k = 0; k < 10; ++k)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[k][j] = 0ull;
+#pragma unroll 1
+    for (uint32_t g = (blockIdx.x * 256 + threadIdx.x) >> 1; g < quads; g += gridDim.x * 128) {  // pixels 4g .. 4g + 3
+        const int wq = (int)(g & ((1u << lwo4) - 1)), ho = (int)((g >> lwo4) % (uint32_t)Ho);
+        const __nv_bfloat16 *img = img0 + (size_t)((g >> lwo4) / (uint32_t)Ho) * H * H;
+        unsigned long long d[4][4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint4 v = __ldg(dz + ((size_t)g * 4 + q) * 2 + half);
+            const uint32_t vs[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {  // bf16 = the upper half of an fp32
+                d[q][j] = pack2(__uint_as_float(vs[j] << 16), __uint_as_float(vs[j] & 0xFFFF0000u));
+                add2(acc[9][j], d[q][j]);
             }
         }
-        dz[idx] = __float2bfloat16(s);
-    }
-}
-
-// The same for C % 8 == 0: one thread per (pixel, 8 channels), 32-bit
-// indices, 16-byte loads of the ReLU input and stores of dz, two 16-byte
-// loads per tap of dcols; taps added in the same order (ky, then kx).
-__global__ void col2im_relu_vec_kernel(const float *__restrict__ dcols, const __nv_bfloat16 *__restrict__ x, int H,
-                                       int W, int C, int stride, int Ho, int Wo, int Kp, uint32_t total,
-                                       __nv_bfloat16 *__restrict__ dz) {
-    const uint32_t cg = (uint32_t)C / 8u;
-    for (uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += gridDim.x * blockDim.x) {
-        const uint32_t pix = idx / cg, c0 = (idx - pix * cg) * 8u;
-        const uint32_t t = pix / (uint32_t)W, w = pix - t * (uint32_t)W;
-        const uint32_t n = t / (uint32_t)H, h = t - n * (uint32_t)H;
-        const uint4 xv = *reinterpret_cast<const uint4 *>(x + (size_t)pix * C + c0);
-        const __nv_bfloat16 *xb = reinterpret_cast<const __nv_bfloat16 *>(&xv);
-        float s[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) s[e] = 0.f;
-        bool any = false;
+        for (int ky = 0; ky < 3; ++ky) {
+            const int h = 2 * ho - 1 + ky;  // < H: only the row above the image is missing
+            if (h < 0) continue;
+            const __nv_bfloat16 *row = img + (size_t)h * H + 8 * wq;  // columns 8 wq - 1 .. 8 wq + 7
+            const uint4 x = __ldg(reinterpret_cast<const uint4 *>(row));
+            const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
+            float v[9];
+            v[0] = wq > 0 ? __bfloat162float(row[-1]) : 0.f;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) any = any || __bfloat162float(xb[e]) > 0.f;
-        if (any) {
-            for (int ky = 0; ky < 3; ++ky) {
-                const int hh = (int)h + 1 - ky;
-                if (hh < 0 || hh % stride) continue;
-                const int ho = hh / stride;
-                if (ho >= Ho) continue;
-                for (int kx = 0; kx < 3; ++kx) {
-                    const int ww = (int)w + 1 - kx;
-                    if (ww < 0 || ww % stride) continue;
-                    const int wo = ww / stride;
-                    if (wo >= Wo) continue;
-                    const float4 *src = reinterpret_cast<const float4 *>(
-                        dcols + ((size_t)((n * (uint32_t)Ho + (uint32_t)ho) * (uint32_t)Wo + (uint32_t)wo)) * Kp +
-                        (ky * 3 + kx) * C + c0);
-                    const float4 a = src[0], b = src[1];
-                    s[0] += a.x; s[1] += a.y; s[2] += a.z; s[3] += a.w;
-                    s[4] += b.x; s[5] += b.y; s[6] += b.z; s[7] += b.w;
-                }
+            for (int i = 0; i < 4; ++i) {
+                v[2 * i + 1] = __uint_as_float(xs[i] << 16);
+                v[2 * i + 2] = __uint_as_float(xs[i] & 0xFFFF0000u);
             }
-        }
-        __align__(16) __nv_bfloat16 o[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) o[e] = __float2bfloat16(__bfloat162float(xb[e]) > 0.f ? s[e] : 0.f);
-        *reinterpret_cast<uint4 *>(dz + (size_t)pix * C + c0) = *reinterpret_cast<const uint4 *>(o);
+            for (int kx = 0; kx < 3; ++kx)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const unsigned long long vv = pack2(v[2 * q + kx], v[2 * q + kx]);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) fma2(acc[3 * ky + kx][j], vv, d[q][j]);
+                }
+        }
     }
-}
-
-// C[i][j] += the nz split partials of element (i, j), added in split order.
-__global__ void sum_splits_kernel(const float *__restrict__ part, int nz, int M, int N, int64_t ldc,
-                                  float *__restrict__ C) {
-    const int64_t total = (int64_t)M * N, zs = (int64_t)M * ldc;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = e / N, j = e - i * N, o = i * ldc + j;
-        float a = 0.f;
-        for (int z = 0; z < nz; ++z) a += part[z * zs + o];
-        C[o] += a;
-    }
-}
-
-__global__ void transpose_kernel(const __nv_bfloat16 *__restrict__ in, int64_t R, int64_t C,
-                                 __nv_bfloat16 *__restrict__ out) {
-    __shared__ __nv_bfloat16 t[32][33];
-    const int64_t r0 = (int64_t)blockIdx.x * 32, c0 = (int64_t)blockIdx.y * 32;  // rows on x: R can be large
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int64_t r = r0 + i, c = c0 + threadIdx.x;
-        if (r < R && c < C) t[i][threadIdx.x] = in[r * C + c];
-    }
+    // Over the lanes of equal half, then over the warps.
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int k = 0; k < 10; ++k)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            float2 a = unpack2(acc[k][j]);
+#pragma unroll
+            for (int o = 16; o > 1; o >>= 1) {
+                a.x += __shfl_xor_sync(0xffffffffu, a.x, o);
+                a.y += __shfl_xor_sync(0xffffffffu, a.y, o);
+            }
+            if (lane < 2) *reinterpret_cast<float2 *>(&red[threadIdx.x >> 5][k * kConv0Out + 8 * half + 2 * j]) = a;
+        }
     __syncthreads();
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int64_t c = c0 + i, r = r0 + threadIdx.x;
-        if (r < R && c < C) out[c * R + r] = t[threadIdx.x][i];
+    if (threadIdx.x < kW0Sums) {
+        float t = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) t += red[w][threadIdx.x];
+        part[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * kW0Sums + threadIdx.x] = t;
     }
 }
 
@@ -468,19 +255,6 @@ __global__ void __launch_bounds__(256) pool_head_kernel(const HeadPair p, int HW
     }
 }
 
-// dz[n][i][c] = dfeat[n][c] / HW * (y > 0): pooling and ReLU backward.
-__global__ void avgpool_back_kernel(const float *__restrict__ dfeat, const __nv_bfloat16 *__restrict__ y, int Nb,
-                                    int HW, int C, __nv_bfloat16 *__restrict__ dz) {
-    const int64_t total = (int64_t)Nb * HW * C;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int c = (int)(idx % C);
-        const int64_t n = idx / ((int64_t)HW * C);
-        const float g = __bfloat162float(y[idx]) > 0.f ? dfeat[n * C + c] / (float)HW : 0.f;
-        dz[idx] = __float2bfloat16(g);
-    }
-}
-
 __device__ __forceinline__ float sigmoidf(float x) { return 1.f / (1.f + expf(-x)); }
 
 // Fused probability p = s1 * s2 (s = sigmoid of each branch's logit) and,
@@ -504,57 +278,123 @@ __global__ void fuse_loss_kernel(const float *__restrict__ l1, const float *__re
     dl2[n] = g * (1.f - s2);
 }
 
-// Head backward: dfeat[n][c] = dl[n] * w[c]; dw[c] += sum_n dl[n] feat[n][c];
-// db += sum_n dl[n].
-__global__ void head_back_kernel(const float *__restrict__ feat, const float *__restrict__ dl, int Nb, int C,
-                                 const float *__restrict__ w, float *__restrict__ dfeat, float *__restrict__ dw,
-                                 float *__restrict__ db) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < C) {
+// Head, pooling and last ReLU backward of both branches (blockIdx.y; C = 256
+// channels).  Blocks 0 .. 7: dw[c] += sum_n dl[n] feat[n][c] of 32 channels, and
+// db += sum_n dl[n] (block 0); block 8 + n: example n's
+// dz[n][i][c] = dl[n] w[c] / HW where y > 0.
+constexpr int kHeadBlocks = 8;
+__global__ void __launch_bounds__(256) head_back_kernel(const HeadGrad p, int Nb, int HW) {
+    constexpr int C = 256;
+    __shared__ float red[8][32];
+    const bool br = blockIdx.y;
+    const float *dl = br ? p.dl[1] : p.dl[0];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (blockIdx.x < kHeadBlocks) {
+        const int c = blockIdx.x * 32 + lane;
+        const float *feat = br ? p.feat[1] : p.feat[0];
         float s = 0.f;
-        for (int n = 0; n < Nb; ++n) {
-            s += dl[n] * feat[(int64_t)n * C + c];
-            dfeat[(int64_t)n * C + c] = dl[n] * w[c];
+#pragma unroll 8
+        for (int n = warp; n < Nb; n += 8) s += dl[n] * feat[n * C + c];
+        red[warp][lane] = s;
+        __syncthreads();
+        if (warp == 0) {
+            float t = 0.f;
+#pragma unroll
+            for (int w = 0; w < 8; ++w) t += red[w][lane];
+            (br ? p.dw[1] : p.dw[0])[c] += t;
+        } else if (warp == 1 && blockIdx.x == 0) {
+            float t = 0.f;
+            for (int n = lane; n < Nb; n += 32) t += dl[n];
+#pragma unroll
+            for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (lane == 0) (br ? p.db[1] : p.db[0])[0] += t;
         }
-        dw[c] += s;
+        return;
     }
-    if (c == 0) {
-        float s = 0.f;
-        for (int n = 0; n < Nb; ++n) s += dl[n];
-        db[0] += s;
+    const int n = blockIdx.x - kHeadBlocks;
+    const float *w = (br ? p.w[1] : p.w[0]) + 8 * lane;
+    uint32_t g[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) g[e] = __bfloat16_as_ushort(__float2bfloat16(dl[n] * w[e] / (float)HW));
+    const size_t at = (size_t)n * HW * (C / 8) + lane;
+    const uint4 *y = reinterpret_cast<const uint4 *>(br ? p.y[1] : p.y[0]) + at;
+    uint4 *dz = reinterpret_cast<uint4 *>(br ? p.dz[1] : p.dz[0]) + at;
+#pragma unroll 4
+    for (int i = warp; i < HW; i += 8) {
+        const uint4 v = y[(size_t)i * (C / 8)];
+        const uint32_t vs[4] = {v.x, v.y, v.z, v.w};
+        uint32_t o[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            o[e] = (__uint_as_float(vs[e] << 16) > 0.f ? g[2 * e] : 0u) |
+                   (__uint_as_float(vs[e] & 0xFFFF0000u) > 0.f ? g[2 * e + 1] << 16 : 0u);
+        dz[(size_t)i * (C / 8)] = make_uint4(o[0], o[1], o[2], o[3]);
     }
 }
 
-// db[c] += sum over rows of dz[.][c] (bias gradient of a conv layer).
-// Bias gradients db[c] += sum over the P rows of dz[p][c], in two
-// deterministic stages.  Stage 1: chunk blockIdx.x of rows; thread t sums
-// channel t % C over rows t / C + k * (256 / C) (consecutive threads read
-// consecutive bytes of a row), then the 256 / C row lanes are added in a
-// fixed order into part[chunk][c].  Stage 2: one thread per channel adds the
-// chunks in order.  C divides 256.
-__global__ void __launch_bounds__(256) bias_grad_part_kernel(const __nv_bfloat16 *__restrict__ dz, int64_t P, int C,
-                                                             int64_t rows_per_chunk, float *__restrict__ part) {
-    __shared__ float red[256];
-    const int c = threadIdx.x % C, rl = threadIdx.x / C, lanes = 256 / C;
-    const int64_t p0 = (int64_t)blockIdx.x * rows_per_chunk;
-    const int64_t p1 = min(P, p0 + rows_per_chunk);
+// Bias gradients, the sums of dz[p][c] over the pixels, in two deterministic
+// stages.  Here chunk blockIdx.x of the P rows of both branches (blockIdx.y) to
+// part[branch][chunk][c]: a thread adds eight channels (16 bytes) of every
+// (2048 / C)-th row, then the block's threads of equal channels form a tree.  Bound
+// by reading dz; all layers of both branches at batch 64, both stages: 415 us with
+// 2-byte loads and a serial second stage -> 38 us.
+__global__ void __launch_bounds__(256, 4) bias_part_kernel(const __nv_bfloat16 *__restrict__ dz0,
+                                                        const __nv_bfloat16 *__restrict__ dz1, int64_t P, int C,
+                                                        int64_t rows_per_chunk, float *__restrict__ part) {
+    __shared__ float red[8][256];
+    const int c8 = C / 8, lanes = 256 / c8, row = threadIdx.x / c8, col = threadIdx.x - row * c8;
+    const uint4 *dz = reinterpret_cast<const uint4 *>(blockIdx.y ? dz1 : dz0) + col;
+    const int64_t p1 = min(P, (blockIdx.x + 1) * rows_per_chunk);
+    float a[8] = {};
+#pragma unroll 4
+    for (int64_t p = blockIdx.x * rows_per_chunk + row; p < p1; p += lanes) {
+        const uint4 v = __ldg(dz + p * c8);
+        const uint32_t vs[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            a[2 * e] += __uint_as_float(vs[e] << 16);
+            a[2 * e + 1] += __uint_as_float(vs[e] & 0xFFFF0000u);
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) red[e][threadIdx.x] = a[e];
+    for (int s = lanes / 2; s; s >>= 1) {
+        __syncthreads();
+        if (row < s)
+#pragma unroll
+            for (int e = 0; e < 8; ++e) red[e][threadIdx.x] += red[e][threadIdx.x + s * c8];
+    }
+    // the first c8 threads hold the sums (each its own: no barrier needed)
+    if (row == 0)
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            part[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * C + 8 * col + e] = red[e][threadIdx.x];
+}
+
+// The second stage for every layer (blockIdx.z) of both branches (blockIdx.y):
+// 32 columns a block; warp w adds rows w, w + 32, ... in order, then the warps' sums
+// are added in order.  Layer 0's columns are its weight gradients' and biases'.
+__global__ void __launch_bounds__(1024) column_sums_kernel(const ColumnSums p) {
+    __shared__ float red[32][33];
+    const int l = blockIdx.z, cols = p.cols[l], n = p.rows[l];
+    const int c = blockIdx.x * 32 + threadIdx.x, w = threadIdx.y;
+    if ((int)blockIdx.x * 32 >= cols) return;
     float s = 0.f;
-    for (int64_t p = p0 + rl; p < p1; p += lanes) s += __bfloat162float(dz[p * C + c]);
-    red[threadIdx.x] = s;
+    if (c < cols) {
+        const float *q = p.part[l] + (size_t)blockIdx.y * n * cols + c;
+#pragma unroll 4
+        for (int r = w; r < n; r += 32) s += q[(size_t)r * cols];
+    }
+    red[w][threadIdx.x] = s;
     __syncthreads();
-    if ((int)threadIdx.x < C) {
-        float t = 0.f;
-        for (int r = 0; r < lanes; ++r) t += red[r * C + threadIdx.x];
-        part[(int64_t)blockIdx.x * C + threadIdx.x] = t;
-    }
-}
-
-__global__ void bias_grad_sum_kernel(const float *__restrict__ part, int nchunk, int C, float *__restrict__ db) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= C) return;
-    float s = 0.f;
-    for (int k = 0; k < nchunk; ++k) s += part[(int64_t)k * C + c];
-    db[c] += s;
+    if (w || c >= cols) return;
+    float t = 0.f;
+#pragma unroll
+    for (int r = 0; r < 32; ++r) t += red[r][threadIdx.x];
+    float *db = blockIdx.y ? p.db[1][l] : p.db[0][l];
+    if (l > 0) db[c] += t;
+    else if (c < 9 * kConv0Out) (blockIdx.y ? p.dw0[1] : p.dw0[0])[(c & 15) * p.kp0 + (c >> 4)] += t;
+    else db[c - 9 * kConv0Out] += t;
 }
 
 // Adam on fp32 master weights; bf16 copy refreshed for the GEMMs.
@@ -820,53 +660,6 @@ int grid_for(int64_t n, int threads = 256) {
 
 }  // namespace
 
-int cnn_gemm(int epi, const __nv_bfloat16 *A, int64_t lda, const __nv_bfloat16 *B, int64_t ldb, int M, int N,
-             int64_t K, float *Cf, __nv_bfloat16 *Cb, int64_t ldc, const float *bias, int splits, cudaStream_t st,
-             int *nz_out) {
-    // the tensor cores (tcgen05) where the shapes suit them
-    const int rc = cnn_gemm_tc(epi, A, lda, B, ldb, M, N, K, Cf, Cb, ldc, bias, splits, st, nz_out);
-    if (rc != SP_ELIMIT) return rc;
-    if (K % kBK) return SP_EINVAL;
-    if (splits < 1 || epi != kEpiSplit) splits = 1;
-    int64_t ks = ((K / kBK + splits - 1) / splits) * kBK;
-    const int nz = (int)((K + ks - 1) / ks);
-    if (nz_out) *nz_out = nz;
-    const dim3 grid((unsigned)((N + kBN - 1) / kBN), (unsigned)((M + kBM - 1) / kBM), (unsigned)nz);
-    if (epi == kEpiBiasRelu)
-        gemm_nt_kernel<kEpiBiasRelu><<<grid, 256, 0, st>>>(A, lda, B, ldb, M, N, K, ks, Cf, Cb, ldc, bias);
-    else if (epi == kEpiStore)
-        gemm_nt_kernel<kEpiStore><<<grid, 256, 0, st>>>(A, lda, B, ldb, M, N, K, ks, Cf, Cb, ldc, bias);
-    else
-        gemm_nt_kernel<kEpiSplit><<<grid, 256, 0, st>>>(A, lda, B, ldb, M, N, K, ks, Cf, Cb, ldc, bias);
-    note_launch();
-    return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
-}
-
-int cnn_sum_splits(const float *part, int nz, int M, int N, int64_t ldc, float *C, cudaStream_t st) {
-    if (nz < 1) return SP_EINVAL;
-    sum_splits_kernel<<<grid_for((int64_t)M * N), 256, 0, st>>>(part, nz, M, N, ldc, C);
-    note_launch();
-    return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
-}
-
-int cnn_im2col(const __nv_bfloat16 *x, int Nb, int H, int W, int C, int stride, int Ho, int Wo, int Kp,
-               __nv_bfloat16 *cols, cudaStream_t st) {
-    const int64_t P = (int64_t)Nb * Ho * Wo;
-    const bool small = P * Kp < (int64_t)1 << 31 && (int64_t)Nb * H * W * C < (int64_t)1 << 31;
-    const bool aligned = (reinterpret_cast<uintptr_t>(x) & 15) == 0 && (reinterpret_cast<uintptr_t>(cols) & 15) == 0;
-    if (small && aligned && Kp % 8 == 0 && C % 8 == 0) {
-        const int64_t total = P * (Kp / 8);
-        im2col_vec_kernel<<<grid_for(total), 256, 0, st>>>(x, H, W, C, stride, Ho, Wo, (uint32_t)(Kp / 8),
-                                                           (uint32_t)total, cols);
-    } else if (small && aligned && Kp % 8 == 0 && Kp >= 16 && C == 1) {
-        im2col_c1_kernel<<<grid_for(P), 256, 0, st>>>(x, H, W, stride, Ho, Wo, (uint32_t)(Kp / 8), (uint32_t)P, cols);
-    } else {
-        im2col_kernel<<<grid_for(P * Kp), 256, 0, st>>>(x, Nb, H, W, C, stride, Ho, Wo, Kp, cols);
-    }
-    note_launch();
-    return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
-}
-
 int cnn_conv0(const ConvPair &p, int Nb, int H, int Kp, cudaStream_t st) {
     const int Ho = H / 2;
     const int64_t P = (int64_t)Nb * Ho * Ho;
@@ -881,38 +674,35 @@ int cnn_conv0(const ConvPair &p, int Nb, int H, int Kp, cudaStream_t st) {
     return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
 }
 
-int cnn_col2im_relu(const float *dcols, const __nv_bfloat16 *x, int Nb, int H, int W, int C, int stride, int Ho,
-                    int Wo, int Kp, __nv_bfloat16 *dz, cudaStream_t st) {
-    const int64_t total = (int64_t)Nb * H * W * C;
-    const bool aligned = (reinterpret_cast<uintptr_t>(dcols) & 15) == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0 &&
-                         (reinterpret_cast<uintptr_t>(dz) & 15) == 0;
-    if (aligned && C % 8 == 0 && Kp % 4 == 0 && total < ((int64_t)1 << 31) &&
-        (int64_t)Nb * Ho * Wo * Kp < ((int64_t)1 << 31))
-        col2im_relu_vec_kernel<<<grid_for(total / 8), 256, 0, st>>>(dcols, x, H, W, C, stride, Ho, Wo, Kp,
-                                                                     (uint32_t)(total / 8), dz);
-    else
-        col2im_relu_kernel<<<grid_for(total), 256, 0, st>>>(dcols, x, Nb, H, W, C, stride, Ho, Wo, Kp, dz);
+int cnn_conv0_wgrad(const GradPair &p, int Nb, int H, float *part, int *rows, cudaStream_t st) {
+    const uint32_t quads = (uint32_t)((int64_t)Nb * (H / 2) * (H / 2) / 4);
+    int lwo4 = 0;
+    while ((8 << lwo4) < H) ++lwo4;
+    *rows = (int)std::min<uint32_t>(kW0Blocks, (quads + 127) / 128);
+    conv0_wgrad_kernel<<<dim3((unsigned)*rows, 2), 256, 0, st>>>(p, H, lwo4, quads, part);
     note_launch();
     return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
 }
 
-int cnn_transpose(const __nv_bfloat16 *in, int64_t R, int64_t C, __nv_bfloat16 *out, cudaStream_t st) {
-    if ((C + 31) / 32 > 65535) return SP_ELIMIT;
-    const dim3 grid((unsigned)((R + 31) / 32), (unsigned)((C + 31) / 32));
-    transpose_kernel<<<grid, dim3(32, 8), 0, st>>>(in, R, C, out);
+int cnn_bias_part(const GradPair &p, int64_t P, int C, float *part, int *rows, cudaStream_t st) {
+    if (C < 16 || C > 256 || 256 % C || P < 1) return SP_EINVAL;
+    const int64_t chunks = std::min<int64_t>(kBiasChunks, (P + 255) / 256), per = (P + chunks - 1) / chunks;
+    *rows = (int)((P + per - 1) / per);
+    bias_part_kernel<<<dim3((unsigned)*rows, 2), 256, 0, st>>>(p.dz[0], p.dz[1], P, C, per, part);
+    note_launch();
+    return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
+}
+
+int cnn_column_sums(const ColumnSums &p, cudaStream_t st) {
+    int most = 0;
+    for (int l = 0; l < kCnnLayers; ++l) most = std::max(most, p.cols[l]);
+    column_sums_kernel<<<dim3((unsigned)((most + 31) / 32), 2, kCnnLayers), dim3(32, 32), 0, st>>>(p);
     note_launch();
     return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
 }
 
 int cnn_pool_head(const HeadPair &p, int Nb, int HW, cudaStream_t st) {
     pool_head_kernel<<<dim3((unsigned)Nb, 2), 256, 0, st>>>(p, HW);
-    note_launch();
-    return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
-}
-
-int cnn_avgpool_back(const float *dfeat, const __nv_bfloat16 *y, int Nb, int HW, int C, __nv_bfloat16 *dz,
-                     cudaStream_t st) {
-    avgpool_back_kernel<<<grid_for((int64_t)Nb * HW * C), 256, 0, st>>>(dfeat, y, Nb, HW, C, dz);
     note_launch();
     return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
 }
@@ -924,20 +714,9 @@ int cnn_fuse_loss(const float *l1, const float *l2, const float *label, int Nb, 
     return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
 }
 
-int cnn_head_back(const float *feat, const float *dl, int Nb, int C, const float *w, float *dfeat, float *dw,
-                  float *db, cudaStream_t st) {
-    head_back_kernel<<<(C + 255) / 256, 256, 0, st>>>(feat, dl, Nb, C, w, dfeat, dw, db);
+int cnn_head_back(const HeadGrad &p, int Nb, int HW, cudaStream_t st) {
+    head_back_kernel<<<dim3((unsigned)(kHeadBlocks + Nb), 2), 256, 0, st>>>(p, Nb, HW);
     note_launch();
-    return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
-}
-
-int cnn_bias_grad(const __nv_bfloat16 *dz, int64_t P, int C, float *db, float *part, cudaStream_t st) {
-    if (C < 1 || C > 256 || 256 % C || P < 1) return SP_EINVAL;
-    const int nchunk = (int)std::min<int64_t>(kBiasChunks, (P + 255) / 256);
-    const int64_t rows = (P + nchunk - 1) / nchunk;
-    bias_grad_part_kernel<<<nchunk, 256, 0, st>>>(dz, P, C, rows, part);
-    bias_grad_sum_kernel<<<(C + 255) / 256, 256, 0, st>>>(part, nchunk, C, db);
-    note_launch(2);
     return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
 }
 
