@@ -7,9 +7,9 @@
 //   sps_stats_kernel   one CTA per (row, normalisation block): exact sum
 //                      (64-bit) and sum of squares (128-bit: int32 values
 //                      near 2^31 square to 2^62 each), 16-byte loads.
-//   sps_coef_kernel    one thread per (row, block): m0, the 128-bit
-//                      variance term, the per-width float coefficients of the
-//                      S/N affine map and the candidate pre-filter constants.
+//   sps_coef_kernel    per (row, block): m0, the 128-bit variance term; per
+//                      width: the float coefficients of the S/N affine map
+//                      and the candidate pre-filter constants.
 //   sps_stream_kernel  candidate search for power-of-two widths: one CTA per
 //                      14 rows (+1 halo row on each side) and a segment of
 //                      chunks of 256 samples, walked with a two-chunk ring of
@@ -169,43 +169,54 @@ __device__ int32_t prefilter_bound(float thr, float cx, float cy, double rcx) {
     return (int32_t)x;
 }
 
-// Per (row, block), one thread each: m0 = floor(Sx/n), f = Sx/n - m0, the
-// per-width float coefficients of the S/N affine map (inv = n/(sqrt(w)
-// sqrt(V)), bias = w f inv) and the pre-filter constants w*m0 + X (32-bit
-// wrap-around: the search subtracts them from a window's prefix difference
-// to get x - X exactly).  The double arithmetic runs here, spread over
-// threads, not at the end of every reduction CTA.
+// Per (row, block): m0 = floor(Sx/n), f = Sx/n - m0; per width too: the float
+// coefficients of the S/N affine map (inv = n/(sqrt(w) sqrt(V)), bias = w f inv)
+// and the pre-filter constants w*m0 + X (32-bit wrap-around: the search
+// subtracts them from a window's prefix difference to get x - X exactly).  The
+// double arithmetic runs here, not at the end of every reduction CTA.  Bound by the
+// latency of its chain of double divisions and a square root, and on a large plane by
+// the double pipe: 32 blocks a CTA, one warp for what a block's widths share, then a
+// thread per block and width (501 x 3 blocks, ten widths: 16 us with the widths in
+// a thread's loop, 6 us now; 5751 x 4, nine widths: 15 -> 12 us).
+constexpr int kCoefBlocks = 32;
 __global__ void __launch_bounds__(256) sps_coef_kernel(const BlockSums *__restrict__ sums, int64_t nrb,
                                                        int64_t n_out, int64_t norm_block, int64_t nblk,
                                                        WidthList wl, WidthRoots wr, float thr,
                                                        int32_t *__restrict__ m0_out, float2 *__restrict__ coef_out,
                                                        uint32_t *__restrict__ cthr_out) {
-    const int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    if (idx >= nrb) return;
-    const int64_t b = idx % nblk;
-    const int64_t lo = (nblk == 1) ? 0 : b * norm_block;
-    const int64_t hi = (b == nblk - 1) ? n_out : (b + 1) * norm_block;
-    const int64_t n = hi - lo;
-    const BlockSums sm = sums[idx];
-    const int64_t S1 = sm.s1;
-    const u128 S2 = ((u128)sm.s2_hi << 64) | sm.s2_lo;
-    int64_t m0 = S1 / n;
-    if (S1 - m0 * n < 0) --m0;  // floor for negative sums
-    const double rn = 1.0 / (double)n;
-    const double frac = (double)(S1 - m0 * n) * rn;
-    // n <= 2^31 and S2 <= n * 2^62: the product stays below 2^124.
-    const __int128 var_n2 = (__int128)n * (__int128)S2 - (__int128)S1 * S1;
-    const double sq = var_n2 > 0 ? sqrt((double)var_n2) : 0.0;
-    const double inv_sigma = var_n2 > 0 ? (double)n / sq : 0.0;
-    const double sig_n = sq * rn;
-    m0_out[idx] = (int32_t)m0;
-    for (int k = 0; k < wl.nw; ++k) {
-        const double w = (double)wl.w[k];
-        const double inv = inv_sigma * wr.rsw[k];
-        const float cx = (float)inv, cy = (float)(w * frac * inv);
-        coef_out[idx * wl.nw + k] = make_float2(cx, cy);
-        cthr_out[idx * wl.nw + k] =
-            (uint32_t)wl.w[k] * (uint32_t)m0 + (uint32_t)prefilter_bound(thr, cx, cy, wr.sw[k] * sig_n);
+    __shared__ double inv_s[kCoefBlocks], frac_s[kCoefBlocks], sig_s[kCoefBlocks];
+    __shared__ int32_t m0_s[kCoefBlocks];
+    const int64_t first = (int64_t)blockIdx.x * kCoefBlocks;
+    const int tid = threadIdx.x;
+    if (tid < kCoefBlocks && first + tid < nrb) {
+        const int64_t idx = first + tid;
+        const int64_t b = idx % nblk;
+        const int64_t lo = (nblk == 1) ? 0 : b * norm_block;
+        const int64_t hi = (b == nblk - 1) ? n_out : (b + 1) * norm_block;
+        const int64_t n = hi - lo;
+        const BlockSums sm = sums[idx];
+        const int64_t S1 = sm.s1;
+        const u128 S2 = ((u128)sm.s2_hi << 64) | sm.s2_lo;
+        int64_t m0 = S1 / n;
+        if (S1 - m0 * n < 0) --m0;  // floor for negative sums
+        const double rn = 1.0 / (double)n;
+        // n <= 2^31 and S2 <= n * 2^62: the product stays below 2^124.
+        const __int128 var_n2 = (__int128)n * (__int128)S2 - (__int128)S1 * S1;
+        const double sq = var_n2 > 0 ? sqrt((double)var_n2) : 0.0;
+        m0_out[idx] = m0_s[tid] = (int32_t)m0;
+        frac_s[tid] = (double)(S1 - m0 * n) * rn;
+        inv_s[tid] = var_n2 > 0 ? (double)n / sq : 0.0;
+        sig_s[tid] = sq * rn;
+    }
+    __syncthreads();
+    const int count = (int)min((int64_t)kCoefBlocks, nrb - first) * wl.nw;
+    for (int i = tid; i < count; i += 256) {
+        const int q = i / wl.nw, k = i - q * wl.nw;
+        const double w = (double)wl.w[k], inv = inv_s[q] * wr.rsw[k];
+        const float cx = (float)inv, cy = (float)(w * frac_s[q] * inv);
+        const int64_t id = first * wl.nw + i;
+        coef_out[id] = make_float2(cx, cy);
+        cthr_out[id] = (uint32_t)wl.w[k] * (uint32_t)m0_s[q] + (uint32_t)prefilter_bound(thr, cx, cy, wr.sw[k] * sig_s[q]);
     }
 }
 
@@ -1208,7 +1219,7 @@ int launch_sps(const SpsArgs &a, cudaStream_t stream) {
     const int64_t nrb = (int64_t)a.ndm * a.nblk;
     sps_stats_kernel<<<dim3((unsigned)a.nblk, (unsigned)a.ndm), 256, 0, stream>>>(a.dmt, a.n_out, a.norm_block,
                                                                                 a.nblk, sums);
-    sps_coef_kernel<<<(unsigned)((nrb + 255) / 256), 256, 0, stream>>>(sums, nrb, a.n_out, a.norm_block, a.nblk, wl,
+    sps_coef_kernel<<<(unsigned)((nrb + kCoefBlocks - 1) / kCoefBlocks), 256, 0, stream>>>(sums, nrb, a.n_out, a.norm_block, a.nblk, wl,
                                                                       wr, a.threshold, m0s, coefs, cthr);
     note_launch(2);
     if (cudaGetLastError() != cudaSuccess) return SP_ECUDA;
