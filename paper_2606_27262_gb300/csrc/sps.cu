@@ -19,6 +19,10 @@
 //                      for the candidate append.  Chunks it cannot prove
 //                      exact in 32-bit float-convertible arithmetic, and the
 //                      beam's last chunk(s), are listed for the tile kernel.
+//   sps_map_kernel     best-S/N map for widths up to 256: one warp per row, the
+//                      same ring of prefix sums, points that are bit for bit
+//                      the tile kernel's; lists what it cannot prove exact.
+//   sps_peaks_window_kernel  peak filter with a (2R+1)^2 window over the map.
 //   sps_boxcar_kernel  the tile kernel: one CTA per 14 rows x 256 samples
 //                      (+1 halo row and sample on each side).  Stages prefix
 //                      sums of the rows in shared memory (warp-shuffle scans),
@@ -42,6 +46,7 @@
 // kernel proves per CTA from the staged values (|x| <= w * max|v - m0|);
 // 8-bit beams of up to 8192 channels always qualify.  A CTA that cannot
 // prove it evaluates the same formula in 64-bit integers instead.
+#include <algorithm>
 #include <cmath>
 #include <mutex>
 
@@ -690,12 +695,13 @@ __global__ void __launch_bounds__(256, 4) sps_boxcar_kernel(BoxcarArgs a) {
 // row group and the chunks it could not prove exact in 2^22), in the 32-bit
 // tile kernel (persistent grid); a tile it cannot prove exact goes on to the
 // 64-bit pass.
+template <bool MAP>
 __global__ void __launch_bounds__(256, 4) sps_boxcar_listed_kernel(BoxcarArgs a) {
     extern __shared__ __align__(16) uint8_t smem[];
     const int n = *a.slow_count;
     for (int i = blockIdx.x; i < n; i += gridDim.x) {
         const int2 tile = a.slow_list[i];
-        if (!boxcar_tile<uint32_t, false>(a, tile.x, tile.y, smem) && threadIdx.x == 0) {
+        if (!boxcar_tile<uint32_t, MAP>(a, tile.x, tile.y, smem) && threadIdx.x == 0) {
             const int slot = atomicAdd(a.wide_count, 1);
             a.wide_list[slot] = tile;
         }
@@ -1051,56 +1057,367 @@ __global__ void __launch_bounds__(256, 4) sps_stream_kernel(BoxcarArgs a) {
     }
 }
 
-// Peak filter with a (2R+1) x (2R+1) window (Sec. 3.1.2: the paper's
-// second stencil is 11 x 11, R = 5) over a best-S/N map the boxcar kernel
-// wrote: one CTA per 32 rows x 256 samples, staged with an R-wide halo (-inf
-// outside the map); a point at or above the threshold is kept when it is
-// above every neighbour that precedes it in (row, t) order and not below any
-// that follows (the same tie rule as the 3 x 3 filter); kept points are
-// appended with one atomic per warp.
-constexpr int kPkRows = 32;
-constexpr int kPkT = 256;
+// Streamed best-S/N map: one warp per DM row, 14 rows (+1 halo row on each side,
+// which only takes part in the proof below) and a segment of chunks of 256
+// samples per CTA.  A warp keeps the exclusive prefix R of its row's chunks c
+// and c+1 in shared memory (R[t0 + i] at i, so that a width is an offset of the
+// address and nothing wraps), each sample is loaded and scanned once, and
+// a lane scores the points lane + 32 j: five instructions per point and width,
+// the subtraction and the fused multiply-add of two points in one each
+// (f32x2, the same rounding).  Bound by the integer and min/max pipe and by issue.
+//
+// The map is bit for bit the tile kernel's.  The same proof over the same rows
+// and samples (its staged range, cover = nq - 4 samples from t0 and the four before)
+// decides which tiles keep 19 bits of the S/N; a tile that fails goes to the tile
+// kernel's list.  The tile kernel scores points p = l + 16 j (p = 0 is sample
+// t0 - 1), j < 8, and 128 + l + 16 j together and p = 256 alone, and compares the
+// full S/N where the points of such a group lie in several blocks, or one lies
+// outside the beam or has a width that leaves it: those points are scored
+// again that way here.  Used for widths up to 256 and blocks of a multiple of
+// 256 samples (or one), any row alignment; there it is the faster one at every
+// size (501 x 20011, ten widths, odd rows: 111 -> 61 us; 1751 x 16384, nine
+// widths: 225 -> 155 us).
+constexpr int kMapSeg = 16;  // chunks per CTA at most (a segment loads and scans one chunk more)
+constexpr int kMapMaxWidth = 256;
 
-__host__ __device__ inline size_t peaks_smem(int radius) {
-    return (size_t)(kPkRows + 2 * radius) * (kPkT + 2 * radius) * sizeof(float);
+__device__ __forceinline__ unsigned long long f32x2(float lo, float hi) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
 }
+__device__ __forceinline__ float2 f32x2_parts(unsigned long long v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+
+// Samples 128 m + 4 lane + e (m < 2, e < 4) of the 256 from `src`, of which `n` exist (others 0).
+__device__ __forceinline__ void map_load(const int32_t *__restrict__ src, int n, int lane, bool vec, int32_t (&v)[8]) {
+    src += 4 * lane;
+    if (vec && n >= kBxT) {
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+            const int4 x = __ldg(reinterpret_cast<const int4 *>(src + 128 * m));
+            v[4 * m] = x.x;
+            v[4 * m + 1] = x.y;
+            v[4 * m + 2] = x.z;
+            v[4 * m + 3] = x.w;
+        }
+    } else {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int i = 128 * (e >> 2) + (e & 3);
+            v[e] = 4 * lane + i < n ? __ldg(src + i) : 0;
+        }
+    }
+}
+
+struct MinMax {
+    int32_t lo, hi;
+};
+__device__ __forceinline__ MinMax join(MinMax a, MinMax b) { return {min(a.lo, b.lo), max(a.hi, b.hi)}; }
+__device__ __forceinline__ MinMax warp_minmax(MinMax a) {
+    return {__reduce_min_sync(0xffffffffu, a.lo), __reduce_max_sync(0xffffffffu, a.hi)};
+}
+
+__global__ void __launch_bounds__(512, 2) sps_map_kernel(BoxcarArgs a, int seg) {
+    __shared__ __align__(16) uint32_t ring_s[kBxRows][2 * kBxT];
+    __shared__ __align__(16) uint4 tab_s[kBxRows][SP_MAX_WIDTHS];  // per width: magic constant, slope, -offset, width
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int ty = blockIdx.y, cs = (int)blockIdx.x * seg, ce = min(cs + seg, a.n_fast);
+    const int64_t d = (int64_t)ty * kBxIn - 1 + warp;
+    const bool present = d >= 0 && d < a.ndm, scored = present && warp > 0 && warp <= kBxIn;
+    const int32_t *row = a.dmt + (present ? d : 0) * a.n_out;
+    uint32_t *ring = ring_s[warp];
+    const int nw = a.wl.nw;
+    const int cover = boxcar_nq(a.maxw) - kBxOrg;  // 256 < cover <= 524
+    const MinMax none = {INT32_MAX, INT32_MIN};
+    // Samples the beam has from chunk cs on (a segment's reach is far below 2^30), and in the k-th chunk of `room`.
+    int room = (int)min(a.n_out - (int64_t)cs * kBxT, (int64_t)1 << 30);
+    auto left = [&](int k) { return max(0, min(kBxT, room - k * kBxT)); };
+    // Scans a chunk of n samples from `carry` into o; the extremes of all, of the first lim and of the last four.
+    uint32_t carry = 0;
+    auto scan = [&](const int32_t (&v)[8], int n, int lim, uint32_t (&o)[8], MinMax &full, MinMax &part, MinMax &last4) {
+        uint32_t incl[2], g[2];
+        auto extremes = [&](int upto) {
+            MinMax p = none;
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (128 * (e >> 2) + 4 * lane + (e & 3) < upto) p = join(p, {v[e], v[e]});
+            return warp_minmax(p);
+        };
+        MinMax m4 = none, f = none;
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+            g[m] = (uint32_t)v[4 * m] + (uint32_t)v[4 * m + 1] + (uint32_t)v[4 * m + 2] + (uint32_t)v[4 * m + 3];
+            incl[m] = g[m];
+            m4 = join(join({v[4 * m], v[4 * m]}, {v[4 * m + 1], v[4 * m + 1]}),
+                      join({v[4 * m + 2], v[4 * m + 2]}, {v[4 * m + 3], v[4 * m + 3]}));
+            f = join(f, m4);
+        }
+        last4 = {__shfl_sync(0xffffffffu, m4.lo, 31), __shfl_sync(0xffffffffu, m4.hi, 31)};  // of a whole chunk
+        full = n < kBxT ? extremes(n) : warp_minmax(f);
+        part = lim < n ? extremes(lim) : full;
+#pragma unroll
+        for (int s = 1; s < 32; s <<= 1) {
+#pragma unroll
+            for (int m = 0; m < 2; ++m) {
+                const uint32_t u = __shfl_up_sync(0xffffffffu, incl[m], s);
+                if (lane >= s) incl[m] += u;
+            }
+        }
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+            o[4 * m] = carry + incl[m] - g[m];
+            o[4 * m + 1] = o[4 * m] + (uint32_t)v[4 * m];
+            o[4 * m + 2] = o[4 * m + 1] + (uint32_t)v[4 * m + 1];
+            o[4 * m + 3] = o[4 * m + 2] + (uint32_t)v[4 * m + 2];
+            carry += __shfl_sync(0xffffffffu, incl[m], 31);
+        }
+    };
+    auto put = [&](const uint32_t (&o)[8], int at) {
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+            *reinterpret_cast<uint4 *>(ring + at + 128 * m + 4 * lane) =
+                make_uint4(o[4 * m], o[4 * m + 1], o[4 * m + 2], o[4 * m + 3]);
+    };
+
+    const int lim = min(cover - kBxT, kBxT), over = cover - 2 * kBxT;  // samples of the next chunk and of the one after
+    uint32_t R[8] = {};                                // prefix of the chunk to be scored
+    int32_t v[8] = {}, tail = 0;                       // samples of the next one, the lane's of the one after
+    MinMax full = none, own4 = none, prev4 = none;     // extremes of that chunk, its last four, the four before it
+    if (present) {
+        const int32_t *src = row + (int64_t)cs * kBxT;
+        if (cs > 0) {
+            const int32_t x = __ldg(src - 4 + (lane & 3));
+            prev4 = warp_minmax({x, x});
+        }
+        int32_t w[8];
+        map_load(src, left(0), lane, a.vec, w);
+        map_load(src + kBxT, left(1), lane, a.vec, v);
+        if (lane < min(over, left(2))) tail = __ldg(src + 2 * kBxT + lane);
+        MinMax part;
+        scan(w, left(0), kBxT, R, full, part, own4);
+    }
+    // The chunk's block, the sample at which the next one starts, and whether this chunk starts its own.
+    int64_t blk = block_of((int64_t)cs * kBxT, a.norm_block, a.nblk), next = INT64_MAX;
+    bool starts = cs == 0 || block_of((int64_t)cs * kBxT - 1, a.norm_block, a.nblk) != blk, fresh = true;
+    if (blk + 1 < a.nblk) next = (blk + 1) * a.norm_block;
+    for (int c = cs; c < ce; ++c, room -= kBxT) {
+        const int64_t t0 = (int64_t)c * kBxT;
+        if (t0 >= next) {
+            ++blk;
+            next = blk + 1 < a.nblk ? next + a.norm_block : INT64_MAX;
+            starts = fresh = true;
+        }
+        uint32_t Rn[8] = {};
+        MinMax full_n = none, own4_n = none;
+        bool bad = false;
+        __syncwarp();
+        if (present) {
+            MinMax range;
+            scan(v, left(1), lim, Rn, full_n, range, own4_n);
+            range = join(join(range, full), prev4);
+            if (over > 0) range = join(range, warp_minmax(lane < min(over, left(2)) ? MinMax{tail, tail} : none));
+            put(R, 0);
+            put(Rn, kBxT);
+            if (c + 1 < ce) {
+                map_load(row + t0 + 2 * kBxT, left(2), lane, a.vec, v);
+                if (lane < min(over, left(3))) tail = __ldg(row + t0 + 3 * kBxT + lane);
+            }
+            // the tile kernel's proof, against the blocks of t0 - 1, t0 and t0 + 256
+            if (lane < 3 && (lane > 0 || t0 > 0)) {
+                const int64_t b = blk - (lane == 0 && starts) + (lane == 2 && t0 + kBxT >= next);
+                const int64_t m0 = __ldg(a.m0s + d * a.nblk + b);
+                bad = max((int64_t)range.hi - m0, m0 - (int64_t)range.lo) * a.maxw >= (int64_t)(1 << 22);
+            }
+        }
+        if (__syncthreads_or(bad)) {
+            if (threadIdx.x == 0) a.slow_list[atomicAdd(a.slow_count, 1)] = make_int2(c, ty);
+        } else if (scored) {
+            if (fresh) {
+                fresh = false;
+                const int64_t rb = d * a.nblk + blk;
+                if (lane < nw) {
+                    const float2 cf = __ldg(a.coefs + rb * nw + lane);
+                    const uint32_t w = (uint32_t)a.wl.w[lane];
+                    tab_s[warp][lane] = make_uint4(kMagicBits - w * (uint32_t)__ldg(a.m0s + rb), __float_as_uint(cf.x),
+                                                   __float_as_uint(-cf.y), w);
+                }
+                __syncwarp();
+            }
+            uint32_t q0[8];
+            float best[8];
+            int kb[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                q0[j] = ring[lane + 32 * j];
+                best[j] = -INFINITY;
+            }
+            const unsigned long long magic2 = f32x2(-kMagicValue, -kMagicValue);
+#pragma unroll 2
+            for (int k = 0; k < nw; ++k) {
+                const uint4 e = tab_s[warp][k];
+                const uint32_t *Rw = ring + lane + e.w;
+                const unsigned long long cx = f32x2(__uint_as_float(e.y), __uint_as_float(e.y));
+                const unsigned long long cy = f32x2(__uint_as_float(e.z), __uint_as_float(e.z));
+                const uint32_t code = 15u - (uint32_t)k;
+#pragma unroll
+                for (int j = 0; j < 8; j += 2) {
+                    unsigned long long x = f32x2(__uint_as_float(Rw[32 * j] - q0[j] + e.x),
+                                                 __uint_as_float(Rw[32 * j + 32] - q0[j + 1] + e.x));
+                    asm("add.rn.f32x2 %0, %0, %1;" : "+l"(x) : "l"(magic2));
+                    asm("fma.rn.f32x2 %0, %0, %1, %2;" : "+l"(x) : "l"(cx), "l"(cy));
+                    const float2 sv = f32x2_parts(x);
+                    best[j] = fmaxf(best[j], __uint_as_float((__float_as_uint(sv.x) & ~15u) | code));
+                    best[j + 1] = fmaxf(best[j + 1], __uint_as_float((__float_as_uint(sv.y) & ~15u) | code));
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const uint32_t bits = __float_as_uint(best[j]);
+                kb[j] = 15 - (int)(bits & 15u);
+                best[j] = __uint_as_float(bits & ~15u);
+            }
+            const bool ends = 255 + a.maxw > room;
+            if (starts || ends) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int o = lane + 32 * j, p = o + 1, last = p == 256 ? 256 : (p & 15) + 112 + (p & 128);
+                    if (!(starts && (p & 15) == 0 && p < 128) && last - 1 + a.maxw <= room) continue;
+                    best[j] = -INFINITY;
+                    kb[j] = -1;
+#pragma unroll 1
+                    for (int k = 0; k < nw; ++k) {
+                        const uint4 e = tab_s[warp][k];
+                        if (o + (int)e.w > room) break;
+                        const uint32_t x = ring[o + e.w] - q0[j] + (e.x - kMagicBits);
+                        const float sv = fmaf((float)(int32_t)x, __uint_as_float(e.y), __uint_as_float(e.z));
+                        if (sv > best[j]) {
+                            best[j] = sv;
+                            kb[j] = k;
+                        }
+                    }
+                }
+            }
+            float *mb = a.map_best + d * a.n_out + t0 + lane;
+            int8_t *mk = a.map_k + d * a.n_out + t0 + lane;
+            if (room >= kBxT) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    mb[32 * j] = best[j];
+                    mk[32 * j] = (int8_t)kb[j];
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if (lane + 32 * j < room) {
+                        mb[32 * j] = best[j];
+                        mk[32 * j] = (int8_t)kb[j];
+                    }
+            }
+        }
+        starts = false;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) R[e] = Rn[e];
+        prev4 = own4;
+        own4 = own4_n;
+        full = full_n;
+    }
+}
+
+// Peak filter with a (2R+1) x (2R+1) window (Sec. 3.1.2: the paper's
+// second stencil is 11 x 11, R = 5) over a best-S/N map the boxcar kernels
+// wrote; outside the map counts -inf.  A point at or above the threshold is kept
+// when it is above every neighbour that precedes it in (row, t) order and not
+// below any that follows (the same tie rule as the 3 x 3 filter).
+//
+// Few points reach a threshold worth searching with, so the kernel is a read of
+// the map (bound by memory), a warp per row and 512 samples: nothing is staged.
+// Where a warp has such points, it compares all its points with their eight
+// neighbours in registers (a bright burst puts most of a warp's points above the
+// threshold, but one in nine or fewer above their neighbours); a lane takes those
+// of its points that are left through the window, nearest rows first.  32 x 256 points
+// staged with their halo and compared by one thread each, 1751 x 16384, R = 5: 200 -> 55 us.
+constexpr int kPkT = 512, kPkRows = 8;  // samples of a warp, rows of a CTA
 
 __global__ void __launch_bounds__(256) sps_peaks_window_kernel(const float *__restrict__ best,
                                                                const int8_t *__restrict__ wbest, int32_t ndm,
-                                                               int64_t n_out, int radius, float thr,
+                                                               int64_t n_out, int radius, float thr, bool vec,
                                                                sp_cand *__restrict__ cands, int64_t cap,
                                                                unsigned long long *__restrict__ count) {
-    extern __shared__ __align__(16) float tile[];
-    const int W = kPkT + 2 * radius;
-    const int H = kPkRows + 2 * radius;
+    const int lane = threadIdx.x & 31, d = (int)blockIdx.y * kPkRows + ((int)threadIdx.x >> 5);
     const int64_t t0 = (int64_t)blockIdx.x * kPkT;
-    const int d0 = blockIdx.y * kPkRows;
-    for (int i = threadIdx.x; i < H * W; i += blockDim.x) {
-        const int rr = i / W, cc = i - rr * W;
-        const int d = d0 - radius + rr;
-        const int64_t t = t0 - radius + cc;
-        tile[i] = (d >= 0 && d < ndm && t >= 0 && t < n_out) ? __ldg(best + (int64_t)d * n_out + t) : -INFINITY;
+    if (d >= ndm) return;
+    auto at = [&](int dd, int64_t t) {
+        return dd >= 0 && dd < ndm && t >= 0 && t < n_out ? __ldg(best + (int64_t)dd * n_out + t) : -INFINITY;
+    };
+    // The lane's points of a row: x[4 m + e] is sample t0 + 128 m + 4 lane + e.
+    auto load = [&](int dd, float (&x)[16]) {
+        if (vec && t0 + kPkT <= n_out && dd >= 0 && dd < ndm) {
+            const float4 *src = reinterpret_cast<const float4 *>(best + (int64_t)dd * n_out + t0) + lane;
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                const float4 q = __ldg(src + 32 * m);
+                x[4 * m] = q.x;
+                x[4 * m + 1] = q.y;
+                x[4 * m + 2] = q.z;
+                x[4 * m + 3] = q.w;
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) x[i] = at(dd, t0 + 128 * (i >> 2) + 4 * lane + (i & 3));
+        }
+    };
+    float v[16];
+    load(d, v);
+    uint32_t todo = 0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        const bool in = t0 + 128 * (i >> 2) + 4 * lane + (i & 3) < n_out;
+        todo |= (uint32_t)(in && v[i] >= thr) << i;
     }
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    for (int i = threadIdx.x; i < kPkRows * kPkT; i += blockDim.x) {
-        const int r = i / kPkT, c = i - r * kPkT;
-        const int d = d0 + r;
-        const int64_t t = t0 + c;
-        const float v = tile[(r + radius) * W + c + radius];
-        bool keep = d < ndm && t < n_out && v >= thr;
-        for (int dr = -radius; dr <= radius && keep; ++dr) {
-            const float *row = tile + (r + radius + dr) * W + c + radius;
-            for (int dc = -radius; dc <= radius; ++dc) {
-                if (dr == 0 && dc == 0) continue;
-                const float u = row[dc];
-                const bool before = dr < 0 || (dr == 0 && dc < 0);
-                if (before ? !(v > u) : !(v >= u)) {
-                    keep = false;
-                    break;
-                }
+    if (!__any_sync(0xffffffffu, todo != 0)) return;
+#pragma unroll 1
+    for (int dr = -1; dr <= 1; ++dr) {
+        float x[16];
+        load(d + dr, x);
+        const float before = at(d + dr, t0 - 1), after = at(d + dr, t0 + kPkT);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            float l = __shfl_up_sync(0xffffffffu, x[4 * m + 3], 1), r = __shfl_down_sync(0xffffffffu, x[4 * m], 1);
+            const float pl = m ? __shfl_sync(0xffffffffu, x[4 * m - 1], 31) : before;
+            const float pr = m < 3 ? __shfl_sync(0xffffffffu, x[(4 * m + 4) & 15], 0) : after;
+            if (lane == 0) l = pl;
+            if (lane == 31) r = pr;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int i = 4 * m + e;
+                const float left = e ? x[(i + 15) & 15] : l, right = e < 3 ? x[(i + 1) & 15] : r;
+                const bool ok = dr < 0   ? v[i] > left && v[i] > x[i] && v[i] > right
+                                : dr > 0 ? v[i] >= left && v[i] >= x[i] && v[i] >= right
+                                         : v[i] > left && v[i] >= right;
+                if (!ok) todo &= ~(1u << i);
             }
         }
+    }
+    while (__any_sync(0xffffffffu, todo != 0)) {
+        bool keep = todo != 0;
+        const int i = __ffs(todo) - 1;
+        const int64_t t = t0 + 128 * (i >> 2) + 4 * lane + (i & 3);
+        const float p = keep ? at(d, t) : 0.f;
+        todo &= todo - 1;
+        // The largest of row d + dr over the samples [from, to] of the window (map values are never NaN).
+        auto most = [&](int dr, int from, int to) {
+            float m = -INFINITY;
+#pragma unroll
+            for (int dc = -kMaxPeakRadius; dc <= kMaxPeakRadius; ++dc)
+                if (dc >= from && dc <= to) m = fmaxf(m, at(d + dr, t + dc));
+            return m;
+        };
+        if (keep) keep = p > most(0, -radius, -1) && p >= most(0, 1, radius);
+        for (int dr = 1; dr <= radius && keep; ++dr) keep = p > most(-dr, -radius, radius) && p >= most(dr, -radius, radius);
+        __syncwarp();
         const unsigned mask = __ballot_sync(0xffffffffu, keep);
         if (mask) {
             const int leader = __ffs(mask) - 1;
@@ -1114,7 +1431,7 @@ __global__ void __launch_bounds__(256) sps_peaks_window_kernel(const float *__re
                     cd.dm_idx = d;
                     cd.t = (int32_t)t;
                     cd.width_idx = __ldg(wbest + (int64_t)d * n_out + t);
-                    cd.snr = v;
+                    cd.snr = p;
                     cands[pos] = cd;
                 }
             }
@@ -1150,7 +1467,7 @@ int64_t sps_workspace_bytes(int32_t ndm, int64_t n_out, int32_t nw, int64_t norm
 
 namespace {
 std::mutex g_sps_lock;
-size_t g_sps_smem[64][7] = {};  // configured boxcar shared memory per (device, kernel)
+size_t g_sps_smem[64][8] = {};  // configured boxcar shared memory per (device, kernel)
 
 template <typename K>
 int configure_kernel(K kernel, int slot, size_t smem) {
@@ -1176,7 +1493,9 @@ int configure_boxcar(bool map, int maxw) {
     if (!rc)
         rc = map ? configure_kernel(sps_boxcar_wide_kernel<true>, 2, boxcar_wide_smem(maxw))
                  : configure_kernel(sps_boxcar_wide_kernel<false>, 3, boxcar_wide_smem(maxw));
-    if (!rc && !map) rc = configure_kernel(sps_boxcar_listed_kernel, 4, boxcar_smem(maxw));
+    if (!rc)
+        rc = map ? configure_kernel(sps_boxcar_listed_kernel<true>, 7, boxcar_smem(maxw))
+                 : configure_kernel(sps_boxcar_listed_kernel<false>, 4, boxcar_smem(maxw));
     if (!rc && !map) rc = configure_kernel(sps_stream_kernel<0>, 5, stream_smem());
     if (!rc && !map) rc = configure_kernel(sps_stream_kernel<9>, 6, stream_smem());
     return rc;
@@ -1258,7 +1577,24 @@ int launch_sps(const SpsArgs &a, cudaStream_t stream) {
         return SP_ECUDA;
     }
     if (map) {
-        sps_boxcar_kernel<true><<<dim3((unsigned)ntx, ngroups), 256, boxcar_smem(maxw), stream>>>(b);
+        if (maxw <= kMapMaxWidth && (a.nblk == 1 || a.norm_block % kBxT == 0) && ntx <= INT32_MAX) {
+            // The segment length of the least time: whole waves of two CTAs per SM, each as long as its chunks and
+            // about 3/4 of one more to load and scan the first (501 x 20011: 2 chunks 72 us, 10 chunks 62 us).
+            int64_t seg = 1, least = INT64_MAX;
+            for (int64_t n = 2; n <= kMapSeg; ++n) {
+                const int64_t waves = ((ntx + n - 1) / n * ngroups + 2 * nsm - 1) / (2 * nsm);
+                if (waves * (4 * n + 3) < least) {
+                    least = waves * (4 * n + 3);
+                    seg = n;
+                }
+            }
+            b.n_fast = (int32_t)ntx;
+            sps_map_kernel<<<dim3((unsigned)((ntx + seg - 1) / seg), ngroups), 512, 0, stream>>>(b, (int)seg);
+            sps_boxcar_listed_kernel<true><<<nsm * 4, 256, boxcar_smem(maxw), stream>>>(b);
+            note_launch();
+        } else {
+            sps_boxcar_kernel<true><<<dim3((unsigned)ntx, ngroups), 256, boxcar_smem(maxw), stream>>>(b);
+        }
         sps_boxcar_wide_kernel<true><<<nsm, 256, boxcar_wide_smem(maxw), stream>>>(b);
         note_launch(2);
         return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
@@ -1276,7 +1612,7 @@ int launch_sps(const SpsArgs &a, cudaStream_t stream) {
             sps_stream_kernel<9><<<sgrid, 256, stream_smem(), stream>>>(b);
         else
             sps_stream_kernel<0><<<sgrid, 256, stream_smem(), stream>>>(b);
-        sps_boxcar_listed_kernel<<<nsm * 4, 256, boxcar_smem(maxw), stream>>>(b);
+        sps_boxcar_listed_kernel<false><<<nsm * 4, 256, boxcar_smem(maxw), stream>>>(b);
         note_launch(2);
     } else {
         sps_boxcar_kernel<false><<<dim3((unsigned)ntx, ngroups), 256, boxcar_smem(maxw), stream>>>(b);
@@ -1311,29 +1647,10 @@ int launch_sps_window(SpsArgs a, int32_t radius, cudaStream_t stream) {
     a.map_wbest = wmap;
     int rc = launch_sps(a, stream);
     if (rc) return rc;
-    static std::mutex lock;
-    static size_t configured[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
-        cudaGetLastError();
-        return SP_ECUDA;
-    }
-    const size_t smem = peaks_smem(radius);
-    {
-        std::lock_guard<std::mutex> guard(lock);
-        if (configured[dev] < smem) {
-            if (cudaFuncSetAttribute(sps_peaks_window_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem) != cudaSuccess) {
-                cudaGetLastError();
-                return SP_ECUDA;
-            }
-            configured[dev] = smem;
-        }
-    }
     if (cudaMemsetAsync(count, 0, sizeof(int64_t), stream) != cudaSuccess) return SP_ECUDA;
     const dim3 grid((unsigned)((a.n_out + kPkT - 1) / kPkT), (unsigned)((a.ndm + kPkRows - 1) / kPkRows));
-    sps_peaks_window_kernel<<<grid, 256, smem, stream>>>(map, wmap, a.ndm, a.n_out, radius, thr, cands, cap,
-                                                         reinterpret_cast<unsigned long long *>(count));
+    sps_peaks_window_kernel<<<grid, 256, 0, stream>>>(map, wmap, a.ndm, a.n_out, radius, thr, (a.n_out & 3) == 0, cands,
+                                                      cap, reinterpret_cast<unsigned long long *>(count));
     note_launch();
     return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
 }
