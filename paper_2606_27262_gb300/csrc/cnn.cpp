@@ -15,6 +15,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <random>
 #include <vector>
@@ -55,6 +56,8 @@ struct sp_cnn {
     float *prob = nullptr, *loss = nullptr;
     float *sums = nullptr;   // partial sums of layer 0's gradients and of every bias gradient
     float *wpart = nullptr;  // partial weight gradients of a layer
+    float *flat = nullptr;  // parameters or gradients in the external order, on their way out
+    std::mutex flat_lock;   // held while `flat` is filled and copied
     int64_t step = 0;
     bool have_grads = false;
 };
@@ -92,18 +95,6 @@ int64_t flat_count() {
     return n + kFeat + 1;
 }
 
-void to_flat(const Branch &b, const std::vector<float> &dev, float *out) {
-    int64_t k = 0;
-    for (int l = 0; l < kLayers; ++l) {
-        const int K9 = 9 * kCin[l], Kp = kp_of(l);
-        for (int co = 0; co < kCout[l]; ++co)
-            for (int kk = 0; kk < K9; ++kk) out[k++] = dev[(size_t)(b.off_w[l] + (int64_t)co * Kp + kk)];
-        for (int co = 0; co < kCout[l]; ++co) out[k++] = dev[(size_t)(b.off_b[l] + co)];
-    }
-    for (int c = 0; c < kFeat; ++c) out[k++] = dev[(size_t)(b.off_hw + c)];
-    out[k++] = dev[(size_t)b.off_hb];
-}
-
 void from_flat(const Branch &b, const float *in, std::vector<float> &dev) {
     dev.assign((size_t)b.n, 0.f);
     int64_t k = 0;
@@ -133,6 +124,7 @@ void free_cnn(sp_cnn *c) {
         cudaFree(b.dl);
     }
     cudaFree(c->sums);
+    cudaFree(c->flat);
     cudaFree(c->wpart);
     cudaFree(c->prob);
     cudaFree(c->loss);
@@ -284,6 +276,7 @@ extern "C" int sp_cnn_create(int32_t max_batch, uint64_t seed, sp_cnn **out) {
     }
     if (!rc) rc = dalloc((void **)&c->sums, sums * 4);
     if (!rc) rc = dalloc((void **)&c->wpart, wpart * 4);
+    if (!rc) rc = dalloc((void **)&c->flat, 2 * flat_count() * 4);
     if (!rc) rc = dalloc((void **)&c->prob, B * 4);
     if (!rc) rc = dalloc((void **)&c->loss, 4);
     // He-normal convolution weights, zero biases, small head weights.
@@ -317,17 +310,38 @@ extern "C" int sp_cnn_destroy(sp_cnn *c) {
     return SP_OK;
 }
 
+// Device values of both branches in the external order to the host: gathered by a
+// kernel and copied once (a training pass with its gradients, batch 64: 861 us with
+// a zeroed host copy of each branch, gathered value by value; 537 us so).
+static int get_flat(const sp_cnn *c, const float *b0, const float *b1, float *h) {
+    sp_cnn *m = const_cast<sp_cnn *>(c);
+    std::lock_guard<std::mutex> guard(m->flat_lock);
+    const int rc = cudaDeviceSynchronize() == cudaSuccess ? SP_OK : SP_ECUDA;
+    if (rc) return rc;
+    FlatLayout f;
+    f.segments = 0;
+    auto add = [&](int64_t off, int rows, int cols, int ld) {
+        f.off[f.segments] = off;
+        f.rows[f.segments] = rows;
+        f.cols[f.segments] = cols;
+        f.ld[f.segments++] = ld;
+    };
+    const Branch &b = c->br[0];  // the branches are laid out alike
+    for (int l = 0; l < kLayers; ++l) {
+        add(b.off_w[l], kCout[l], 9 * kCin[l], kp_of(l));
+        add(b.off_b[l], 1, kCout[l], kCout[l]);
+    }
+    add(b.off_hw, 1, kFeat, kFeat);
+    add(b.off_hb, 1, 1, 1);
+    const int rp = cnn_to_flat(f, b0, b1, flat_count(), m->flat, nullptr);
+    if (rp) return rp;
+    return cudaMemcpy(h, m->flat, (size_t)(2 * flat_count()) * 4, cudaMemcpyDeviceToHost) == cudaSuccess ? SP_OK
+                                                                                                        : SP_ECUDA;
+}
+
 extern "C" int sp_cnn_get_params(const sp_cnn *c, float *h) {
     if (!c || !h || !on_cnn_device(c)) return SP_EINVAL;
-    const int64_t nf = flat_count();
-    for (int bi = 0; bi < 2; ++bi) {
-        std::vector<float> d((size_t)c->br[bi].n);
-        if (cudaDeviceSynchronize() != cudaSuccess ||
-            cudaMemcpy(d.data(), c->br[bi].params, d.size() * 4, cudaMemcpyDeviceToHost) != cudaSuccess)
-            return SP_ECUDA;
-        to_flat(c->br[bi], d, h + bi * nf);
-    }
-    return SP_OK;
+    return get_flat(c, c->br[0].params, c->br[1].params, h);
 }
 
 extern "C" int sp_cnn_set_params(sp_cnn *c, const float *h) {
@@ -345,15 +359,7 @@ extern "C" int sp_cnn_set_params(sp_cnn *c, const float *h) {
 
 extern "C" int sp_cnn_get_grads(const sp_cnn *c, float *h) {
     if (!c || !h || !c->have_grads || !on_cnn_device(c)) return SP_EINVAL;
-    const int64_t nf = flat_count();
-    for (int bi = 0; bi < 2; ++bi) {
-        std::vector<float> d((size_t)c->br[bi].n);
-        if (cudaDeviceSynchronize() != cudaSuccess ||
-            cudaMemcpy(d.data(), c->br[bi].grads, d.size() * 4, cudaMemcpyDeviceToHost) != cudaSuccess)
-            return SP_ECUDA;
-        to_flat(c->br[bi], d, h + bi * nf);
-    }
-    return SP_OK;
+    return get_flat(c, c->br[0].grads, c->br[1].grads, h);
 }
 
 extern "C" int sp_cnn_forward(sp_cnn *c, const void *d_ft, const void *d_dmt, int32_t batch, float *d_prob,

@@ -418,6 +418,18 @@ __global__ void to_bf16_kernel(const float *__restrict__ a, int64_t n, __nv_bflo
         b[i] = __float2bfloat16(a[i]);
 }
 
+__global__ void to_flat_kernel(const FlatLayout f, const float *__restrict__ b0, const float *__restrict__ b1,
+                               int64_t count, float *__restrict__ out) {
+    const float *src = blockIdx.y ? b1 : b0;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    int e = i, s = 0;
+    while (s < f.segments && e >= f.rows[s] * f.cols[s]) {
+        e -= f.rows[s] * f.cols[s];
+        ++s;
+    }
+    if (s < f.segments) out[blockIdx.y * count + i] = src[f.off[s] + (int64_t)(e / f.cols[s]) * f.ld[s] + e % f.cols[s]];
+}
+
 // Images of one candidate from its subband dynamic spectrum sub[S][T_in]
 // (already dedispersed at the candidate DM within each subband; time bins):
 //   ft[s][u]  = sub[s][u0 + u]                         (S x 256)
@@ -724,6 +736,12 @@ int cnn_adam(float *w, const float *g, float *m, float *v, int64_t n, float lr, 
              int64_t step, __nv_bfloat16 *wb, cudaStream_t st) {
     const float c1 = 1.f - powf(b1, (float)step), c2 = 1.f - powf(b2, (float)step);
     adam_kernel<<<grid_for(n), 256, 0, st>>>(w, g, m, v, n, lr, b1, b2, eps, c1, c2, wb);
+    note_launch();
+    return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
+}
+
+int cnn_to_flat(const FlatLayout &f, const float *b0, const float *b1, int64_t count, float *out, cudaStream_t st) {
+    to_flat_kernel<<<dim3((unsigned)((count + 255) / 256), 2), 256, 0, st>>>(f, b0, b1, count, out);
     note_launch();
     return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
 }

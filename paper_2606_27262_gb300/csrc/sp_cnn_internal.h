@@ -78,6 +78,14 @@ int cnn_fuse_loss(const float *l1, const float *l2, const float *label, int Nb, 
                   float *loss, cudaStream_t st);
 int cnn_adam(float *w, const float *g, float *m, float *v, int64_t n, float lr, float b1, float b2, float eps,
              int64_t step, __nv_bfloat16 *wb, cudaStream_t st);
+// out[branch][0 .. count) = the branch's segments one after the other, rows x cols
+// each from rows of ld at off.
+struct FlatLayout {
+    int segments;
+    int64_t off[2 * kCnnLayers + 2];
+    int rows[2 * kCnnLayers + 2], cols[2 * kCnnLayers + 2], ld[2 * kCnnLayers + 2];
+};
+int cnn_to_flat(const FlatLayout &f, const float *b0, const float *b1, int64_t count, float *out, cudaStream_t st);
 int cnn_to_bf16(const float *a, int64_t n, __nv_bfloat16 *b, cudaStream_t st);
 // Decimation and half width of each trial width, passed by value.
 struct ExtractWidths {
