@@ -639,30 +639,75 @@ __global__ void __launch_bounds__(kImg) normalise_kernel(const float *__restrict
 // [nchan][pitch]: sub[q][s][u] = sum over the channels c of subband s and
 // i < dec of xt[c][t0 + (u - t_in/2) * dec + i + delay[dm][c]], with t0 the
 // centre of the candidate's boxcar window; samples outside [0, n_in) count 0.
-// One CTA per (candidate, subband), threads over time bins.
-__global__ void extract_kernel(const uint8_t *__restrict__ xt, int64_t pitch, int64_t n_in, int32_t nchan,
-                               const int32_t *__restrict__ delays, const sp_cand *__restrict__ cands,
-                               ExtractWidths wt, int32_t nsub, int32_t t_in, float *__restrict__ sub) {
+// One CTA per (candidate, subband), threads over time bins; the sums are
+// integers, so their order is free.  Bound by instruction issue on addresses and bounds
+// and, for bins of many samples, by loads whose lanes lie far apart: a window that
+// lies inside the beam in every channel of the subband is read without checks
+// from one address and offsets the CTA shares, and bins of eight samples or more four
+// samples at a time (the ends of a bin masked) where rows are 4-byte aligned.
+// Five candidates of a gulp, 4096 channels, 512 bins: 40 -> 31 us.
+constexpr int kExtractPer = 64;  // channels of a subband that share offsets
+
+__global__ void __launch_bounds__(256) extract_kernel(const uint8_t *__restrict__ xt, int64_t pitch, int64_t n_in,
+                                                      int32_t nchan, const int32_t *__restrict__ delays,
+                                                      const sp_cand *__restrict__ cands, ExtractWidths wt, int32_t nsub,
+                                                      int32_t t_in, bool words, float *__restrict__ sub) {
+    __shared__ int64_t off_s[kExtractPer];
     const int q = blockIdx.y, s = blockIdx.x;
     const sp_cand c = cands[q];
     const int per = nchan / nsub;
     const int wi = min(max(c.width_idx, 0), SP_MAX_WIDTHS - 1);
     const int dec = wt.dec[wi];
-    const int64_t t0 = (int64_t)c.t + wt.half[wi];
-    const int32_t *dl = delays + (int64_t)c.dm_idx * nchan;
-    for (int u = threadIdx.x; u < t_in; u += blockDim.x) {
-        const int64_t tb = t0 + (int64_t)(u - t_in / 2) * dec;
-        float acc = 0.f;
-        for (int k = 0; k < per; ++k) {
-            const int ch = s * per + k;
-            const uint8_t *row = xt + (int64_t)ch * pitch;
-            const int64_t base = tb + dl[ch];
-            for (int i = 0; i < dec; ++i) {
-                const int64_t t = base + i;
-                if (t >= 0 && t < n_in) acc += (float)row[t];
+    const int64_t first = (int64_t)c.t + wt.half[wi] - (int64_t)(t_in / 2) * dec;  // sample of bin 0 without delay
+    const int32_t *dl = delays + (int64_t)c.dm_idx * nchan + s * per;
+    const uint8_t *rows = xt + (int64_t)s * per * pitch;
+    float *out = sub + ((int64_t)q * nsub + s) * t_in;
+    bool inside = per <= kExtractPer;
+    if (inside && (int)threadIdx.x < per) {
+        const int64_t d = dl[threadIdx.x];
+        inside = first + d >= 0 && first + d + (int64_t)t_in * dec <= n_in;
+        off_s[threadIdx.x] = threadIdx.x * pitch + d;
+    }
+    if (__syncthreads_and(inside)) {
+        for (int u = threadIdx.x; u < t_in; u += 256) {
+            const uint8_t *p = rows + first + u * dec;
+            uint32_t acc = 0;
+            if (dec == 1) {
+#pragma unroll 8
+                for (int k = 0; k < per; ++k) acc += __ldg(p + off_s[k]);
+            } else if (dec < 8 || !words) {
+#pragma unroll 4
+                for (int k = 0; k < per; ++k) {
+                    const uint8_t *r = p + off_s[k];
+#pragma unroll 4
+                    for (int i = 0; i < dec; ++i) acc += __ldg(r + i);
+                }
+            } else {
+#pragma unroll 2
+                for (int k = 0; k < per; ++k) {
+                    const uint8_t *r = p + off_s[k];
+                    const int skip = (int)(reinterpret_cast<uintptr_t>(r) & 3);
+                    const uint32_t *w = reinterpret_cast<const uint32_t *>(r - skip);
+                    const int last = (skip + dec - 1) >> 2;  // >= 1; a word of the row, whose pitch is whole words
+                    acc = __dp4a(__ldg(w) >> (8 * skip), 0x01010101u, acc);
+#pragma unroll 4
+                    for (int i = 1; i < last; ++i) acc = __dp4a(__ldg(w + i), 0x01010101u, acc);
+                    acc = __dp4a(__ldg(w + last) & (0xFFFFFFFFu >> (8 * (3 - ((skip + dec - 1) & 3)))), 0x01010101u, acc);
+                }
             }
+            out[u] = (float)acc;
         }
-        sub[((int64_t)q * nsub + s) * t_in + u] = acc;
+        return;
+    }
+    for (int u = threadIdx.x; u < t_in; u += 256) {
+        const int64_t tb = first + (int64_t)u * dec;
+        uint32_t acc = 0;
+        for (int k = 0; k < per; ++k) {
+            const uint8_t *row = rows + (int64_t)k * pitch;
+            const int64_t base = tb + __ldg(dl + k), lo = max(base, (int64_t)0), hi = min(base + dec, n_in);
+            for (int64_t t = lo; t < hi; ++t) acc += __ldg(row + t);
+        }
+        out[u] = (float)acc;
     }
 }
 
@@ -755,8 +800,9 @@ int cnn_to_bf16(const float *a, int64_t n, __nv_bfloat16 *b, cudaStream_t st) {
 int cnn_extract(const uint8_t *xt, int64_t pitch, int64_t n_in, int32_t nchan, const int32_t *delays,
                 const sp_cand *cands, int32_t ncand, const ExtractWidths &wt, int32_t nsub, int32_t t_in, float *sub,
                 cudaStream_t st) {
+    const bool words = ((reinterpret_cast<uintptr_t>(xt) | (uintptr_t)pitch) & 3) == 0;
     extract_kernel<<<dim3((unsigned)nsub, (unsigned)ncand), 256, 0, st>>>(xt, pitch, n_in, nchan, delays, cands, wt,
-                                                                        nsub, t_in, sub);
+                                                                        nsub, t_in, words, sub);
     note_launch();
     return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
 }

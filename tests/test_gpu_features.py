@@ -60,3 +60,28 @@ def test_images_do_not_depend_on_the_batch():
     for n in (15, 16, 47, 48, 64):
         many = _images(sub[:n].contiguous(), shift)
         assert all(np.array_equal(a[0], m[3]) for a, m in zip(alone, many))
+
+
+@pytest.mark.parametrize("odd", [0, 1])
+def test_extracted_spectra_are_exact(odd):
+    """Bins of 1, 3, 4, 16 and 64 samples that start anywhere, windows over both
+    ends of the beam and outside it, rows read four bytes at a time and (a
+    beam at an odd address) one at a time: integers, so equal."""
+    rng = np.random.default_rng(11)
+    freqs, n_in, t_in, widths = 500.0 - np.arange(512) * (200.0 / 512), 3001, 300, [1, 15, 16, 64, 256]
+    plan = sp.Plan(freqs, 0.00131072, np.array([0.0, 100.0, 333.0]))
+    dl = plan.delays()
+    data = rng.integers(0, 256, size=(512, n_in), dtype=np.uint8)
+    pitch = sp.staged_pitch(n_in)
+    staged = torch.zeros(512 * pitch + odd, dtype=torch.uint8, device="cuda")[odd:].view(512, pitch)
+    staged[:, :n_in] = torch.from_numpy(data).cuda()
+    cands = [(d, t, w) for d in range(3) for w in range(5) for t in (-40000, 0, 5, 1234, n_in - 2, 2 ** 30)]
+    rec = np.array([(d, t, w, 0) for d, t, w in cands], dtype=np.int32)
+    sub = sp.cnn_extract(plan, staged, n_in, torch.from_numpy(rec).cuda(), widths, t_in=t_in).cpu().numpy()
+    total = np.concatenate([np.zeros((512, 1), np.int64), np.cumsum(data, axis=1, dtype=np.int64)], axis=1)
+    for q, (d, t, w) in enumerate(cands):
+        dec = max(1, widths[w] // 4)
+        start = t + widths[w] // 2 + (np.arange(t_in) - t_in // 2) * dec + dl[d][:, None].astype(np.int64)
+        at = lambda x: np.take_along_axis(total, np.clip(x, 0, n_in), axis=1)
+        want = (at(start + dec) - at(start)).reshape(256, 2, t_in).sum(axis=1)
+        assert np.array_equal(sub[q], want.astype(np.float32)), (d, t, w)
