@@ -17,8 +17,9 @@
 //                      and width, the exact S/N where it passes, the
 //                      threshold and the 3x3 peak filter, one atomic per warp
 //                      for the candidate append.  Chunks it cannot prove
-//                      exact in 32-bit float-convertible arithmetic, and the
-//                      beam's last chunk(s), are listed for the tile kernel.
+//                      exact in 32-bit float-convertible arithmetic are listed
+//                      for the tile kernel; the beam's last chunk(s) too, or
+//                      (small planes) are scored as tiles by CTAs of their own.
 //   sps_map_kernel     best-S/N map for widths up to 256: one warp per row, the
 //                      same ring of prefix sums, points that are bit for bit
 //                      the tile kernel's; lists what it cannot prove exact.
@@ -691,8 +692,8 @@ __global__ void __launch_bounds__(256, 4) sps_boxcar_kernel(BoxcarArgs a) {
     }
 }
 
-// The tiles the streamed search listed (the beam's last chunk(s) of every
-// row group and the chunks it could not prove exact in 2^22), in the 32-bit
+// The tiles a streamed kernel listed (chunks it could not prove exact in 2^22
+// and, on large planes, a search's last chunk(s)), in the 32-bit
 // tile kernel (persistent grid); a tile it cannot prove exact goes on to the
 // 64-bit pass.
 template <bool MAP>
@@ -747,7 +748,7 @@ constexpr int kStSeg = 16;  // chunks per CTA
 
 __host__ __device__ inline size_t stream_smem() {
     return (size_t)kBxRows * kStRing * 4 + (size_t)kBxRows * kStSS * 4 + (size_t)kBxRows * kStSS +
-           (size_t)kBxRows * 16 * 4;
+           (size_t)kBxRows * 16 * 4;  // a tile of widths up to 256 needs less
 }
 
 __device__ __forceinline__ uint4 lds128(const uint32_t *p) { return *reinterpret_cast<const uint4 *>(p); }
@@ -915,7 +916,7 @@ __device__ __forceinline__ float stream_halo(const BoxcarArgs &a, const uint32_t
     return stream_exact(Rw, Rt, nw, __ldg(a.m0s + rb), a.coefs + rb * nw, kb);
 }
 
-template <int NW>
+template <int NW, bool TAIL>
 __global__ void __launch_bounds__(256, 4) sps_stream_kernel(BoxcarArgs a) {
     extern __shared__ __align__(16) uint8_t smem[];
     uint32_t *ring_all = reinterpret_cast<uint32_t *>(smem);
@@ -933,16 +934,24 @@ __global__ void __launch_bounds__(256, 4) sps_stream_kernel(BoxcarArgs a) {
     uint32_t *cw = cw_all + r * 16;
     const int nw = NW > 0 ? NW : a.wl.nw;
     const int64_t lim = ((1 << 22) - 1) / a.maxw;
-    const int cs = (int)blockIdx.x * kStSeg;
+    // The beam's last chunk(s): a CTA of their own per row group, first in the grid, or the tile kernel's list.
+    const int n_tiles = (int)((a.n_out + kBxT - 1) / kBxT);
+    if (TAIL && blockIdx.x == 0) {
+        for (int x = a.n_fast; x < n_tiles; ++x) {
+            if (!boxcar_tile<uint32_t, false>(a, x, ty, smem) && tid == 0)
+                a.wide_list[atomicAdd(a.wide_count, 1)] = make_int2(x, ty);
+            __syncthreads();
+        }
+        return;
+    }
+    const int cs = ((int)blockIdx.x - TAIL) * kStSeg;
     const int ce = min(cs + kStSeg, a.n_fast);
-    if (!present)
-        for (int p = l; p < kStSS; p += 16) snr_s[r * kStSS + p] = -INFINITY;
-    // The beam's last chunk(s) go to the tile kernel's list.
-    const int n_tail = (int)((a.n_out + kBxT - 1) / kBxT) - a.n_fast;
-    if (blockIdx.x == gridDim.x - 1 && tid < n_tail) {
+    if (!TAIL && blockIdx.x == gridDim.x - 1 && tid < n_tiles - a.n_fast) {
         const int slot = atomicAdd(a.slow_count, 1);
         a.slow_list[slot] = make_int2(a.n_fast + tid, ty);
     }
+    if (!present)
+        for (int p = l; p < kStSS; p += 16) snr_s[r * kStSS + p] = -INFINITY;
 
     uint32_t carry = 0;
     int32_t mnA, mxA, mnB, mxB;  // chunks c and c+1
@@ -1467,7 +1476,7 @@ int64_t sps_workspace_bytes(int32_t ndm, int64_t n_out, int32_t nw, int64_t norm
 
 namespace {
 std::mutex g_sps_lock;
-size_t g_sps_smem[64][8] = {};  // configured boxcar shared memory per (device, kernel)
+size_t g_sps_smem[64][10] = {};  // configured boxcar shared memory per (device, kernel)
 
 template <typename K>
 int configure_kernel(K kernel, int slot, size_t smem) {
@@ -1496,8 +1505,10 @@ int configure_boxcar(bool map, int maxw) {
     if (!rc)
         rc = map ? configure_kernel(sps_boxcar_listed_kernel<true>, 7, boxcar_smem(maxw))
                  : configure_kernel(sps_boxcar_listed_kernel<false>, 4, boxcar_smem(maxw));
-    if (!rc && !map) rc = configure_kernel(sps_stream_kernel<0>, 5, stream_smem());
-    if (!rc && !map) rc = configure_kernel(sps_stream_kernel<9>, 6, stream_smem());
+    if (!rc && !map) rc = configure_kernel(sps_stream_kernel<0, false>, 5, stream_smem());
+    if (!rc && !map) rc = configure_kernel(sps_stream_kernel<9, false>, 6, stream_smem());
+    if (!rc && !map) rc = configure_kernel(sps_stream_kernel<0, true>, 8, stream_smem());
+    if (!rc && !map) rc = configure_kernel(sps_stream_kernel<9, true>, 9, stream_smem());
     return rc;
 }
 }  // namespace
@@ -1607,11 +1618,15 @@ int launch_sps(const SpsArgs &a, cudaStream_t stream) {
     const int64_t n_fast = a.n_out / kBxT - 1;
     if (pow2 && b.vec && (a.nblk == 1 || a.norm_block % kBxT == 0) && n_fast >= 1 && n_fast <= INT32_MAX) {
         b.n_fast = (int32_t)n_fast;
-        const dim3 sgrid((unsigned)((n_fast + kStSeg - 1) / kStSeg), ngroups);
-        if (a.nw == 9)  // widths 1..256
-            sps_stream_kernel<9><<<sgrid, 256, stream_smem(), stream>>>(b);
-        else
-            sps_stream_kernel<0><<<sgrid, 256, stream_smem(), stream>>>(b);
+        // A tile by itself takes 15 us, whatever the plane: where the whole search fits about two waves of CTAs, the
+        // last chunk(s) run beside the others (a beam of 501 x 16384: 78 -> 69 us); on a large plane the larger
+        // kernel costs more than that (5751 x 32768: 454 -> 512 us), so they go to the list.
+        const int64_t segs = (n_fast + kStSeg - 1) / kStSeg;
+        const bool tail = (segs + 1) * ngroups <= 8 * (int64_t)nsm;
+        const dim3 sgrid((unsigned)(segs + tail), ngroups);
+        const auto kernel = a.nw == 9 ? (tail ? sps_stream_kernel<9, true> : sps_stream_kernel<9, false>)  // widths 1..256
+                                      : (tail ? sps_stream_kernel<0, true> : sps_stream_kernel<0, false>);
+        kernel<<<sgrid, 256, stream_smem(), stream>>>(b);
         sps_boxcar_listed_kernel<false><<<nsm * 4, 256, boxcar_smem(maxw), stream>>>(b);
         note_launch(2);
     } else {
