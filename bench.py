@@ -18,9 +18,13 @@ so no L2 flush is needed between steps.
           back (sp_searcher_submit_host / sp_searcher_collect, two in flight,
           so each input copy overlaps the previous beam's search), with the
           one-beam-at-a-time sp_searcher_run_host figure beside it.
-  roofline  dedispersion kernel alone: channel x DM x sample adds per launch
-          over its CUDA-event time, against the integer-add issue rate
-          (SMs x measured 32-bit add lanes per SM per clock x max SM clock).
+  roofline  dedispersion kernel alone.  `achieved` counts the channel x DM x
+          sample adds of the direct sum over its CUDA-event time; the kernel
+          forms sums that trial DMs share once, so it performs fewer, and
+          `frac`, against the integer-add issue rate (SMs x measured
+          32-bit add lanes per SM per clock x max SM clock), passes 1.  What
+          bounds it stands in `issue`: lane instructions per such add (from
+          the committed ncu capture) against the SMs' issue rate.
 
 `--impl reference` times the CPU oracle (test infrastructure) on a bounded
 sample of the same workload on the host cores.
@@ -73,8 +77,9 @@ sys.path.insert(0, ROOT)
 
 METRIC = "real-time beams per GB300; dedispersion G(chan·DM·samp)/s vs roofline"
 MAX_SM_MHZ = 2070.0  # GB300 maximum SM clock
+DIRECT_ADDS = "adds of the direct sum; sums that trial DMs share are formed once, so fewer are performed"
 PROFILE_JSON = os.path.join(ROOT, "profiles", "dedisperse_config2_traffic.json")
-DEDISP_SRC = os.path.join(ROOT, "paper_2606_27262_gb300", "csrc", "dedisperse.cu")
+DEDISP_SRC = os.path.join(ROOT, "paper_2606_27262_gb300", "csrc", "dedisp_sums.cu")
 
 
 def parse_args(argv=None):
@@ -403,7 +408,7 @@ def run_ours(args):
         "candidates_per_beam": ncand,
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tadd/s",
                      "frac": achieved / peak, "traffic": profiled_traffic(wl.n_out),
-                     "kernel": "dedisperse_kernel",
+                     "counts": DIRECT_ADDS, "kernel": "dedisp_sums_kernel",
                      "kernel_shape": dict(zip(("dm_tile", "time_tile", "chan_chunk"), sp.shape_info(plan.shape)))
                      | {"shape": plan.shape, "dm_tiles": plan.ntiles},
                      "issue": issue_roofline(achieved, nsm),
@@ -592,8 +597,9 @@ def run_batched(args):
         "speedup_vs_per_beam": (per_beam["ms_per_step"] / ms_step) if per_beam else None,
         "candidates": int(sum(counts)),
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tadd/s", "frac": achieved / peak,
-                     "traffic": None,
-                     "kernel": "dedisperse_items_kernel" if args.batch_mode == "grid" else "dedisperse_batch_kernel",
+                     "traffic": None, "counts": DIRECT_ADDS,
+                     "kernel": "dedisp_sums_items_kernel, or the direct kernel (%s) where sharing does not pay"
+                     % ("dedisperse_items_kernel" if args.batch_mode == "grid" else "dedisperse_batch_kernel"),
                      "kernel_ms_per_step": dd_ms,
                      "peak_basis": f"{nsm} SMs x {lanes:.1f} measured 32-bit add lanes/SM/clk x "
                                    f"{MAX_SM_MHZ:.0f} MHz"},
@@ -906,7 +912,7 @@ def run_stream(args):
                     "search_p50_s": float(np.percentile(lat_search, 50)),
                     "search_p99_s": float(np.percentile(lat_search, 99)),
                     "candidates": cand_total, "kept": kept_total},
-        "roofline": {"bound": "alu", "achieved": adds_per_gulp * rate_b / 1e12, "unit": "Tadd/s",
+        "roofline": {"bound": "alu", "achieved": adds_per_gulp * rate_b / 1e12, "unit": "Tadd/s", "counts": DIRECT_ADDS,
                      "kernel": "whole streaming chain at saturation (copies, staging, dedispersion, search, sifter, "
                                "classifier)",
                      "peak": None, "frac": None, "traffic": None},

@@ -182,7 +182,7 @@ __device__ int32_t prefilter_bound(float thr, float cx, float cy, double rcx) {
 // double arithmetic runs here, not at the end of every reduction CTA.  Bound by the
 // latency of its chain of double divisions and a square root, and on a large plane by
 // the double pipe: 32 blocks a CTA, one warp for what a block's widths share, then a
-// thread per block and width (501 x 3 blocks, ten widths: 16 us with the widths in
+// thread per block and width (501 x 2 blocks, ten widths: 16 us with the widths in
 // a thread's loop, 6 us now; 5751 x 4, nine widths: 15 -> 12 us).
 constexpr int kCoefBlocks = 32;
 __global__ void __launch_bounds__(256) sps_coef_kernel(const BlockSums *__restrict__ sums, int64_t nrb,
@@ -1619,7 +1619,7 @@ int launch_sps(const SpsArgs &a, cudaStream_t stream) {
     if (pow2 && b.vec && (a.nblk == 1 || a.norm_block % kBxT == 0) && n_fast >= 1 && n_fast <= INT32_MAX) {
         b.n_fast = (int32_t)n_fast;
         // A tile by itself takes 15 us, whatever the plane: where the whole search fits about two waves of CTAs, the
-        // last chunk(s) run beside the others (a beam of 501 x 16384: 78 -> 69 us); on a large plane the larger
+        // last chunk(s) run beside the others (501 x 8192, six widths: 78 -> 68 us); on a large plane the larger
         // kernel costs more than that (5751 x 32768: 454 -> 512 us), so they go to the list.
         const int64_t segs = (n_fast + kStSeg - 1) / kStSeg;
         const bool tail = (segs + 1) * ngroups <= 8 * (int64_t)nsm;
