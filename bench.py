@@ -1030,7 +1030,7 @@ def run_classifier(args):
                      "tflops": tr_tflops} if train_ms else None,
         "roofline": {"bound": "tensor", "achieved": in_tflops, "peak": peak, "unit": "TFLOP/s",
                      "frac": in_tflops / peak, "traffic": None,
-                     "kernel": "inference step (features, first layer, im2col + tcgen05 GEMMs, pooling/head), "
+                     "kernel": "inference step (images, first layer, implicit-GEMM convolutions on tcgen05, pooling/head), "
                                "algorithmic convolution FLOPs over the step time",
                      "peak_basis": "measured bf16 GEMM burst (MEASURED_PEAKS.json)"},
         "e2e": None, "cpu_baseline": None, "clocks": clk, "gpu_launches": launches,

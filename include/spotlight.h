@@ -1,7 +1,7 @@
 /*
  * spotlight.h -- C ABI of libspotlight, the GB300 (sm_103a) search hot path
  * of the SPOTLIGHT real-time transient pipeline (arXiv 2606.27262, Sec. 3.1):
- * brute-force incoherent dedispersion of an 8-bit filterbank beam over a list
+ * incoherent dedispersion of an 8-bit filterbank beam over a list
  * of trial DMs, then a multi-width boxcar single-pulse search with per-block
  * mean/sigma normalisation, a threshold and a 3x3 peak filter that emit a
  * candidate list.

@@ -670,7 +670,7 @@ __global__ void __launch_bounds__(256) extract_kernel(const uint8_t *__restrict_
     }
     if (__syncthreads_and(inside)) {
         for (int u = threadIdx.x; u < t_in; u += 256) {
-            const uint8_t *p = rows + first + u * dec;
+            const uint8_t *p = rows + first + (int64_t)u * dec;
             uint32_t acc = 0;
             if (dec == 1) {
 #pragma unroll 8
