@@ -213,27 +213,28 @@ struct ConvOut {
 // L2 (the layers read 9/4 of their input).  Both branches at batch 256, layers
 // 1-4: 305, 149, 104, 67 us with patches gathered by two warps (the last by
 // im2col) -> 140, 61, 52, 35; at batch 5: 21, 30, 49, 38 -> 8, 9, 10, 19.
-template <int C>
+// NB: CTAs that share a tile's output channels, 2 C / NB each.
+template <int C, int NB>
 struct FwdShape {
-    static constexpr int KC = C < 64 ? C : 64, STEPS = 9 * (C / KC), N = 2 * C;  // KC channels of a tap per stage
+    static constexpr int KC = C < 64 ? C : 64, STEPS = 9 * (C / KC), N = 2 * C / NB;  // KC channels of a tap per stage
     static constexpr int A_BYTES = kTcBM * KC * 2, B_BYTES = N * KC * 2;
     using Pipe = Pipeline<C == 16 ? 9 : C == 32 ? 6 : 4, A_BYTES + B_BYTES, N>;
 };
-template <int C>
+template <int C, int NB>
 __global__ void __launch_bounds__(128) conv_fwd_kernel(const __grid_constant__ ConvMaps maps, const ConvOut out, int M,
                                                        int lwo) {
-    using S = FwdShape<C>;
+    using S = FwdShape<C, NB>;
     extern __shared__ uint8_t smem_raw[];
     typename S::Pipe pipe(smem_raw);
     const bool branch = blockIdx.y;
-    const int m0 = blockIdx.x * kTcBM;
+    const int m0 = blockIdx.x * kTcBM, n0 = blockIdx.z * S::N;
     const bool ok = pipe.run(
         S::STEPS,
         [&](int i, uint8_t *stage, uint32_t full) {
             const int tap = i / (C / S::KC), c0 = (i % (C / S::KC)) * S::KC;
             expect(full, S::A_BYTES + S::B_BYTES);
             load_box4(stage, &maps.a[branch], c0, tap % 3 - 1, 2 * tile_row(m0, lwo) + tap / 3 - 1, tile_image(m0, lwo), full);
-            load_box2(stage + S::A_BYTES, &maps.b[branch], tap * C + c0, 0, full);
+            load_box2(stage + S::A_BYTES, &maps.b[branch], tap * C + c0, n0, full);
         },
         [&](int i, uint32_t stage) {
 #pragma unroll
@@ -246,8 +247,8 @@ __global__ void __launch_bounds__(128) conv_fwd_kernel(const __grid_constant__ C
         // shared memory (the stages are free) so that four lanes store a row's
         // 64 bytes together.
         const int lane = pipe.lane, row0 = m0 + pipe.warp * 32;
-        const float *bias = branch ? out.bias[1] : out.bias[0];
-        __nv_bfloat16 *y = (branch ? out.y[1] : out.y[0]) + (int64_t)row0 * S::N;
+        const float *bias = (branch ? out.bias[1] : out.bias[0]) + n0;
+        __nv_bfloat16 *y = (branch ? out.y[1] : out.y[0]) + (int64_t)row0 * 2 * C + n0;
         uint4 *buf = reinterpret_cast<uint4 *>(pipe.smem) + pipe.warp * 128;
 #pragma unroll 1
         for (int c0 = 0; c0 < S::N; c0 += 32) {
@@ -271,7 +272,7 @@ __global__ void __launch_bounds__(128) conv_fwd_kernel(const __grid_constant__ C
             for (int i = 0; i < 4; ++i) {
                 const int r = 8 * i + (lane >> 2), c = lane & 3;
                 if (row0 + r < M)
-                    *reinterpret_cast<uint4 *>(y + (int64_t)r * S::N + c0 + 8 * c) = buf[4 * r + (c ^ ((r >> 1) & 3))];
+                    *reinterpret_cast<uint4 *>(y + (int64_t)r * 2 * C + c0 + 8 * c) = buf[4 * r + (c ^ ((r >> 1) & 3))];
             }
             __syncwarp();
         }
@@ -542,22 +543,23 @@ int launched() {
     return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
 }
 
-template <int C>
+template <int C, int NB>
 int fwd(const ConvPair &p, int Nb, int H, int Kp, cudaStream_t st) {
-    using S = FwdShape<C>;
+    using S = FwdShape<C, NB>;
     ConvMaps maps;
     ConvOut out;
     for (int b = 0; b < 2; ++b) {
-        if (!map_pixels(&maps.a[b], p.x[b], Nb, H, C, S::KC, 2) || !map_matrix(&maps.b[b], p.w[b], S::N, 9 * C, Kp, S::KC, S::N))
+        if (!map_pixels(&maps.a[b], p.x[b], Nb, H, C, S::KC, 2) || !map_matrix(&maps.b[b], p.w[b], 2 * C, 9 * C, Kp, S::KC, S::N))
             return SP_ECUDA;
         out.bias[b] = p.bias[b];
         out.y[b] = p.y[b];
     }
     static SmemLimit limit;
-    const int rc = limit.set(reinterpret_cast<const void *>(conv_fwd_kernel<C>), S::Pipe::SMEM);
+    const int rc = limit.set(reinterpret_cast<const void *>(conv_fwd_kernel<C, NB>), S::Pipe::SMEM);
     if (rc) return rc;
     const int M = Nb * (H / 2) * (H / 2);
-    conv_fwd_kernel<C><<<dim3((unsigned)((M + kTcBM - 1) / kTcBM), 2), 128, S::Pipe::SMEM, st>>>(maps, out, M, lwo_of(H / 2));
+    conv_fwd_kernel<C, NB><<<dim3((unsigned)((M + kTcBM - 1) / kTcBM), 2, NB), 128, S::Pipe::SMEM, st>>>(maps, out, M,
+                                                                                                       lwo_of(H / 2));
     return launched();
 }
 
@@ -617,11 +619,14 @@ bool aligned(std::initializer_list<const void *> ps, uintptr_t to = 16) {
 
 int cnn_conv_fwd(const ConvPair &p, int Nb, int H, int C, int Kp, cudaStream_t st) {
     if (!shape_ok(Nb, H, C, Kp) || !aligned({p.x[0], p.x[1], p.w[0], p.w[1], p.y[0], p.y[1]})) return SP_EINVAL;
+    // A few tiles leave SMs idle while each streams all of a layer's weights: where four times the CTAs still fit two
+    // an SM, four share a tile's output channels (layers 3, 4 at batch 5: 11, 19 -> 7, 11 us; layer 4 at batch 64: 19 -> 13).
+    const bool few = ((int64_t)Nb * (H / 2) * (H / 2) + kTcBM - 1) / kTcBM * 2 * 4 <= 2 * 152;
     switch (C) {
-        case 16: return fwd<16>(p, Nb, H, Kp, st);
-        case 32: return fwd<32>(p, Nb, H, Kp, st);
-        case 64: return fwd<64>(p, Nb, H, Kp, st);
-        default: return fwd<128>(p, Nb, H, Kp, st);
+        case 16: return fwd<16, 1>(p, Nb, H, Kp, st);
+        case 32: return fwd<32, 1>(p, Nb, H, Kp, st);
+        case 64: return few ? fwd<64, 4>(p, Nb, H, Kp, st) : fwd<64, 1>(p, Nb, H, Kp, st);
+        default: return few ? fwd<128, 4>(p, Nb, H, Kp, st) : fwd<128, 1>(p, Nb, H, Kp, st);
     }
 }
 

@@ -39,3 +39,19 @@ def test_gradients_at_tile_edges(batch):
                 err = np.linalg.norm(grads[0][s] - want[s]) / np.linalg.norm(want[s])
                 assert err <= 0.02, (cin, size, branch, err)
             o += size
+
+
+@pytest.mark.parametrize("batch", [20, 77])
+def test_split_layers_equal_whole_ones(batch):
+    """A few tiles' output channels are shared by several thread blocks; layer 3
+    stops at batch 19, layer 4 at 76.  Either way the same sums in the same order."""
+    spbuild.build()
+    gen = torch.Generator(device="cuda").manual_seed(batch)
+    ft, dmt = (torch.randn((batch, 256, 256), device="cuda", generator=gen).to(torch.bfloat16) for _ in range(2))
+    clf = sp.Classifier(max_batch=batch, seed=3)
+    whole, part = torch.empty(batch, device="cuda"), torch.empty(2, device="cuda")
+    clf.forward(ft, dmt, whole)
+    for i in (0, batch - 2):
+        clf.forward(ft[i:i + 2].contiguous(), dmt[i:i + 2].contiguous(), part)
+        torch.cuda.synchronize()
+        assert torch.equal(whole[i:i + 2], part)
