@@ -32,31 +32,28 @@ int compute_delays(const double *freqs, int32_t nchan, double tsamp, const doubl
     out.resize((size_t)ndm * nchan);
     const double ftop = freqs[0];
     // Trials are independent: blocks of them on the host's cores.
-    std::atomic<int32_t> next{0}, mx{0};
+    std::atomic<int32_t> mx{0};
     std::atomic<bool> beyond{false};
-    constexpr int32_t kBlock = 64;
-    auto work = [&]() {
+    blocks_on_cores(ndm, 64, [&](int64_t first, int64_t end) {
         int32_t most = 0;
-        for (int32_t d0; (d0 = next.fetch_add(kBlock)) < ndm && !beyond;) {
-            for (int32_t d = d0; d < std::min(ndm, d0 + kBlock); ++d) {
-                const double dm = dms[d];
-                for (int32_t c = 0; c < nchan; ++c) {
-                    const double f = freqs[c];
-                    const double x = kDispersionConstant * dm * (1.0 / (f * f) - 1.0 / (ftop * ftop)) / tsamp;
-                    const double r = std::floor(x + 0.5);
-                    if (!(r < 1.0e9)) {
-                        beyond = true;
-                        return;
-                    }
-                    const int32_t v = (int32_t)r;
-                    out[(size_t)d * nchan + c] = v;
-                    most = std::max(most, v);
+        for (int64_t d = first; d < end; ++d) {
+            const double dm = dms[d];
+            for (int32_t c = 0; c < nchan; ++c) {
+                const double f = freqs[c];
+                const double x = kDispersionConstant * dm * (1.0 / (f * f) - 1.0 / (ftop * ftop)) / tsamp;
+                const double r = std::floor(x + 0.5);
+                if (!(r < 1.0e9)) {
+                    beyond = true;
+                    return false;
                 }
+                const int32_t v = (int32_t)r;
+                out[(size_t)d * nchan + c] = v;
+                most = std::max(most, v);
             }
         }
         for (int32_t seen = mx.load(); most > seen && !mx.compare_exchange_weak(seen, most);) {}
-    };
-    run_on_cores(work, (ndm + kBlock - 1) / kBlock);
+        return true;
+    });
     if (beyond) return SP_ELIMIT;
     *max_delay = mx;
     return SP_OK;

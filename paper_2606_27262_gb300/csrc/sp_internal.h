@@ -3,6 +3,7 @@
 #pragma once
 
 #include <algorithm>
+#include <atomic>
 #include <cstdint>
 #include <thread>
 #include <vector>
@@ -253,6 +254,19 @@ inline void run_on_cores(F &work, int64_t pieces) {
     }
     work();
     for (std::thread &t : pool) t.join();
+}
+
+// f(first, end) for blocks of pieces 0 .. n - 1, each once, in no order, until one
+// returns false.  The counter runs past n by a block for every thread: 64 bits.
+template <class F>
+inline void blocks_on_cores(int64_t n, int64_t block, F f) {
+    std::atomic<int64_t> next{0};
+    std::atomic<bool> stop{false};
+    auto work = [&]() {
+        for (int64_t first; !stop && (first = next.fetch_add(block)) < n;)
+            if (!f(first, std::min(n, first + block))) stop = true;
+    };
+    run_on_cores(work, (n + block - 1) / block);
 }
 
 inline int64_t align256(int64_t x) { return (x + 255) & ~int64_t(255); }

@@ -1,0 +1,33 @@
+"""Host code of the plans (plan.cpp, plan_sums.cpp) without a GPU: built here
+with the undefined-behaviour sanitizer and a CUDA runtime made of host memory
+(plan_host.cpp)."""
+import os
+import subprocess
+
+import pytest
+
+from paper_2606_27262_gb300 import build as spbuild
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def run(tmp_path_factory):
+    exe = str(tmp_path_factory.mktemp("plan_host") / "plan_host")
+    src = [os.path.join(HERE, "plan_host.cpp")] + [os.path.join(spbuild.CSRC, f) for f in ("plan.cpp", "plan_sums.cpp")]
+    inc = ["-I", os.path.join(spbuild.cuda_home(), "include"), "-I", os.path.join(spbuild.ROOT, "include")]
+    subprocess.run(["g++", "-std=c++17", "-O1", "-g", "-ffp-contract=off", "-fsanitize=undefined",
+                    "-fno-sanitize-recover=all", *inc, *src, "-o", exe, "-pthread"], check=True)
+
+    def call(*args):
+        r = subprocess.run([exe, *map(str, args)], capture_output=True, text=True, timeout=300)
+        assert r.returncode == 0, r.stdout + r.stderr
+        return r.stdout
+
+    return call
+
+
+def test_trial_blocks_end_at_the_last_trial(run):
+    """Threads take blocks from a counter that passes the end: near 2^31 trials
+    it may not wrap."""
+    run("blocks")
