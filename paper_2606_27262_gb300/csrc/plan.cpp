@@ -273,6 +273,7 @@ static int create_plan(const double *freqs_mhz, int32_t nchan, double tsamp_s, c
     const int32_t zero = 0;
     if (!rc) rc = upload(&p->d_status, &zero, 1);
     if (!rc && shape == 0) {  // the default shape's plans; the others stay the direct kernel's
+        // Without room for these tables, here or on the device, the plan is the direct kernel's as well.
         try {
             SumTables t;
             if (build_sum_tables(*p, t) == SP_OK && sum_tables_pay(*p, t)) {
@@ -282,6 +283,7 @@ static int create_plan(const double *freqs_mhz, int32_t nchan, double tsamp_s, c
         } catch (const std::bad_alloc &) {
             rc = SP_ENOMEM;
         }
+        if (rc == SP_ENOMEM) rc = SP_OK;
     }
     if (!rc) rc = dedisp_configure(p);
     if (rc) {
@@ -410,6 +412,7 @@ extern "C" int sp_plan_check_tables(const double *freqs_mhz, int32_t nchan, doub
     if (shape == 0) {
         SumTables t;
         const int src = build_sum_tables(p, t);
+        if (src == SP_ENOMEM) return src;
         if (src == SP_OK) bad += check_sum_tables(p, t, n_out);
         else bad += src != SP_ELIMIT;
     }

@@ -22,6 +22,7 @@
 #include <climits>
 #include <cmath>
 #include <cstring>
+#include <new>
 
 #include "sp_internal.h"
 
@@ -341,7 +342,7 @@ void build_tile(const sp_plan &p, int32_t d0, int cnt, Tile &t) {
 // Tiles of up to kSumDms consecutive DMs, halved where a tile's delay spread
 // leaves no group that fits a row slot.  SP_ELIMIT: the plan has no tables
 // (too many channels for the 16-bit carries, or a table beyond int32).
-int build_sum_tables(const sp_plan &p, SumTables &t) {
+static int build_tables(const sp_plan &p, SumTables &t) {
     t = SumTables();
     if (p.nchan > kSumMaxChan) return SP_ELIMIT;
     struct Span {
@@ -352,7 +353,7 @@ int build_sum_tables(const sp_plan &p, SumTables &t) {
     std::vector<Span> spans;
     for (int32_t d = 0; d < p.ndm; d += kSumDms) spans.push_back({d, std::min(kSumDms, p.ndm - d), {}, {}});
     std::atomic<size_t> next{0};
-    std::atomic<bool> bad{false};
+    std::atomic<bool> bad{false}, no_memory{false};
     auto work = [&]() {
         try {
             for (size_t i; (i = next.fetch_add(1)) < spans.size() && !bad;) {
@@ -374,12 +375,12 @@ int build_sum_tables(const sp_plan &p, SumTables &t) {
                     d += cnt;
                 }
             }
-        } catch (...) {  // out of host memory: the plan goes without tables
-            bad = true;
+        } catch (...) {
+            bad = no_memory = true;
         }
     };
     run_on_cores(work, (int64_t)spans.size());
-    if (bad) return SP_ELIMIT;
+    if (bad) return no_memory ? SP_ENOMEM : SP_ELIMIT;
     double clocks = 0.0;
     t.tile_chunk.push_back(0);
     t.tile_group.push_back(0);
@@ -413,6 +414,14 @@ int build_sum_tables(const sp_plan &p, SumTables &t) {
     }
     t.tile_clocks = clocks / (double)t.tile_first.size();
     return SP_OK;
+}
+
+int build_sum_tables(const sp_plan &p, SumTables &t) {
+    try {
+        return build_tables(p, t);
+    } catch (const std::bad_alloc &) {
+        return SP_ENOMEM;
+    }
 }
 
 namespace {

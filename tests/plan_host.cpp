@@ -1,6 +1,6 @@
 // Host checks of plan.cpp and plan_sums.cpp without a GPU: the driver links
-// them with a CUDA runtime of its own (host memory; allocations of g_refuse_from bytes
-// or more fail) and is built with the undefined-behaviour sanitizer.
+// them with a CUDA runtime of its own (host memory; allocation number g_refuse
+// fails) and is built with the undefined-behaviour sanitizer.
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -8,12 +8,11 @@
 
 #include "../paper_2606_27262_gb300/csrc/sp_internal.h"
 
-static size_t g_refuse_from = SIZE_MAX;
-static int64_t g_live = 0;  // allocations not freed
+static int64_t g_refuse = -1, g_asked = 0, g_live = 0;  // g_live: allocations not freed
 
 extern "C" {
 cudaError_t cudaMalloc(void **p, size_t n) {
-    if (n >= g_refuse_from) return cudaErrorMemoryAllocation;
+    if (g_asked++ == g_refuse) return cudaErrorMemoryAllocation;
     *p = std::malloc(n);
     ++g_live;
     return cudaSuccess;
@@ -33,7 +32,10 @@ cudaError_t cudaMemset(void *d, int v, size_t n) {
 }
 cudaError_t cudaGetDevice(int *d) { return *d = 0, cudaSuccess; }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
-cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr, int) { return *v = 152, cudaSuccess; }
+cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr a, int) {
+    *v = a == cudaDevAttrMultiProcessorCount ? 152 : 227 * 1024;
+    return cudaSuccess;
+}
 int sp_autotune_dedisperse(const double *, int32_t, double, const double *, int32_t, int64_t, int32_t, float *,
                            int32_t *, void *) {
     return SP_EINVAL;
@@ -61,8 +63,43 @@ static int blocks() {
     return bad || pieces != n;
 }
 
+static std::vector<double> band(int nchan) {
+    std::vector<double> f((size_t)nchan);
+    for (int c = 0; c < nchan; ++c) f[(size_t)c] = 500.0 - 200.0 * c / nchan;
+    return f;
+}
+
+// Device memory runs out at each allocation of a plan in turn: at the shared-sum
+// tables (the last) the plan goes without them, earlier it is refused.
+static int no_room() {
+    const std::vector<double> f = band(1024);
+    std::vector<double> dms;
+    for (int d = 0; d < 128; ++d) dms.push_back(0.1 * d);
+    sp_plan *p = nullptr;
+    auto create = [&]() { return sp_plan_create(f.data(), 1024, 1.31072e-3, dms.data(), 128, &p); };
+    int bad = create() != SP_OK || !p->d_sums;
+    const int64_t n = g_asked;
+    sp_plan_destroy(p);
+    for (int64_t i = 0; i < n; ++i) {
+        g_asked = 0;
+        g_refuse = i;
+        const int rc = create();
+        std::printf("allocation %lld of %lld refused: %d\n", (long long)i, (long long)n, rc);
+        if (i < n - 1) {
+            bad += rc != SP_ENOMEM || p;
+            continue;
+        }
+        if (rc != SP_OK || p->d_sums) return 1;
+        const int64_t n_out = 1 << 20;
+        bad += sp::sums_pay(&p, &n_out, 1);
+        sp_plan_destroy(p);
+    }
+    return bad || g_live;
+}
+
 int main(int argc, char **argv) {
     const std::string what = argc > 1 ? argv[1] : "";
     if (what == "blocks") return blocks();
+    if (what == "no_room") return no_room();
     return 2;
 }

@@ -31,3 +31,8 @@ def test_trial_blocks_end_at_the_last_trial(run):
     """Threads take blocks from a counter that passes the end: near 2^31 trials
     it may not wrap."""
     run("blocks")
+
+
+def test_no_room_for_the_shared_sum_tables(run):
+    """A plan whose direct tables fit is not refused for the larger tables."""
+    run("no_room")
