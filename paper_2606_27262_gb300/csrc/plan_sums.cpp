@@ -37,7 +37,7 @@ struct Group {
     int32_t base = 0, spread = 0;     // smallest delay of channel c0 over the tile, and its range
     int32_t quads = 0;                // quads (4 words) that the rows reach over
     int32_t npat = 0;
-    int32_t row_quads = 0;            // sum of the rows' own quads
+    int64_t row_quads = 0;            // sum of the rows' own quads
     int32_t inits = 0, steps = 0, rows = 0, jobs = 0;  // summed over the passes
     int8_t pat_of[kMaxDms];           // pattern of each DM
     int32_t r[kMaxDms][kSumMaxGroup]; // relative delays of the patterns
@@ -50,7 +50,9 @@ struct Group {
     std::vector<Visit> path;
     std::vector<int32_t> pass_end;    // [passes] end of each pass's entries
     int passes() const { return (quads + 31) / 32; }
-    int64_t row_bytes() const { return (int64_t)row_quads * 16; }
+    int64_t row_bytes() const { return row_quads * 16; }
+    // Whether a row slot takes the rows and a raw slot a window of this reach.
+    bool may_fit() const { return row_bytes() <= kSumRowBytes && quads <= kSumRawBytes / 4; }
 };
 
 // Modelled SM clocks of a group: shared-memory wavefronts (128 bytes a clock;
@@ -95,6 +97,7 @@ void analyse(const sp_plan &p, int32_t d0, int cnt, int32_t c0, int n, Group &g)
         g.qe[k] = (bmax[k] - lo + kSumHalf + 3) / 4;
         g.row_quads += g.qe[k] - g.qs[k];
     }
+    if (!g.may_fit()) return;  // no paths for a group that no slot takes: it may have millions of passes
     // Moves from one pattern to another: channels that differ, if each does by
     // one sample.
     constexpr int kFar = 255;
@@ -166,8 +169,8 @@ Window window_of(const Group &g, int i) {
 int32_t prog_words(const Group &g) {  // 32-bit words of a group's program
     return g.jobs * (4 + 2 * ((g.n + 1) & ~1) + 4 * 4) + 4 * g.steps;
 }
-int32_t raw_bytes(const Group &g) {
-    int32_t b = 0;
+int64_t raw_bytes(const Group &g) {  // delays reach 1e9 samples: a sum of windows does not fit 32 bits
+    int64_t b = 0;
     for (int i = 0; i < g.n; ++i) b += window_of(g, i).bytes;
     return b;
 }
@@ -303,7 +306,7 @@ void build_tile(const sp_plan &p, int32_t d0, int cnt, Tile &t) {
             for (int32_t c = 0; c < block && fits; c += G) {
                 Group &g = cand[n++];
                 analyse(p, d0, cnt, c0 + c, std::min(G, block - c), g);
-                fits = g.row_bytes() <= kSumRowBytes && 16 + 4 * prog_words(g) + raw_bytes(g) <= kSumRawBytes &&
+                fits = g.may_fit() && 16 + 4 * prog_words(g) + raw_bytes(g) <= kSumRawBytes &&
                        g.jobs <= kSumJobArrivals;
                 clocks += group_clocks(g, cnt);
                 bytes += (double)g.row_bytes();

@@ -4,6 +4,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <ctime>
 #include <string>
 
 #include "../paper_2606_27262_gb300/csrc/sp_internal.h"
@@ -97,9 +98,25 @@ static int no_room() {
     return bad || g_live;
 }
 
+// Two bands of 16 almost equal channels, the lower one up to 8e8 samples late: no
+// group of it fits a slot until a tile is a few trials (apart: one trial).
+static int late_band(bool apart) {
+    std::vector<double> f, dms;
+    for (int c = 0; c < 16; ++c) f.push_back(1000.0 - 1e-7 * c);
+    for (int c = 0; c < 16; ++c) f.push_back(100.0 - 3e-7 * c);
+    for (int d = 0; d < 64; ++d) dms.push_back(apart ? 2000.0 * (d & 1) : 2000.0 / 63 * d);
+    int64_t report[8];
+    const int rc = sp_plan_check_tables(f.data(), 32, 1e-6, dms.data(), 64, 0, 1000, report);
+    const double seconds = (double)std::clock() / CLOCKS_PER_SEC;  // 5 s and more with a path for every pass, else 0.01
+    std::printf("rc %d, violations %lld, largest delay %lld, %.2f s\n", rc, (long long)report[5], (long long)report[6],
+                seconds);
+    return rc || report[5] || report[6] < 800000000 || seconds > 2.0;
+}
+
 int main(int argc, char **argv) {
     const std::string what = argc > 1 ? argv[1] : "";
     if (what == "blocks") return blocks();
     if (what == "no_room") return no_room();
+    if (what == "late_band") return late_band(argc > 2);
     return 2;
 }

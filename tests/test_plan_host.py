@@ -36,3 +36,10 @@ def test_trial_blocks_end_at_the_last_trial(run):
 def test_no_room_for_the_shared_sum_tables(run):
     """A plan whose direct tables fit is not refused for the larger tables."""
     run("no_room")
+
+
+@pytest.mark.parametrize("apart", [[], ["apart"]])
+def test_delays_that_differ_by_hundreds_of_millions_of_samples(run, apart):
+    """Windows and rows too long for any slot: their sizes are not summed in 32
+    bits, and no paths are laid out for them (a plan of 64 trials took seconds)."""
+    run("late_band", *apart)
