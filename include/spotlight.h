@@ -108,8 +108,9 @@ int sp_plan_status(const sp_plan *plan, int32_t *h_status, int32_t clear);
  * 1024).  With extra_bytes > 0 the first wait of every CTA runs out, the CTA
  * waits once more (bounded) and leaves, and the status word gets
  * SP_STATUS_STAGING_TIMEOUT; no access leaves its buffers and the device
- * stays usable.  sp_debug_staging_fault(0, 1LL << 31) restores the
- * defaults.  Not for use while dedispersion kernels are in flight. */
+ * stays usable.  The classifier's tensor-core kernels (sp_cnn_status) take
+ * the same from their next launch on.  sp_debug_staging_fault(0, 1LL << 31)
+ * restores the defaults.  Not for use while such kernels are in flight. */
 int sp_debug_staging_fault(int32_t extra_bytes, int64_t wait_limit_cycles);
 /* Copies the delay table, int32 [ndm][nchan], to host memory. */
 int sp_plan_delays(const sp_plan *plan, int32_t *h_out);
@@ -552,12 +553,20 @@ int sp_sift(const sp_cand *h_cands, int64_t n, const double *h_dms, int32_t ndm,
  *   d_labels [batch] (1 = astrophysical, 0 = not), gradients, and the loss
  *   in *h_loss (synchronises; NULL = no copy).  sp_cnn_adam_step applies the
  *   stored gradients; sp_cnn_train_step = backward + adam step.
- * Errors: SP_EINVAL, SP_ENOMEM, SP_EWORKSPACE, SP_ECUDA. */
+ * sp_cnn_status: status word of the handle's passes, 0 or
+ *   SP_STATUS_STAGING_TIMEOUT: a bounded wait of a tensor-core kernel ran out
+ *   and the probabilities, gradients or updates of a pass since the last
+ *   report are void.  Synchronises the device; clear != 0 resets the word.
+ *   A call that waits for such a pass (sp_cnn_backward and _train_step with
+ *   h_loss, _get_grads, _get_params) returns SP_ETIMEOUT once and resets it;
+ *   there are then no gradients until the next sp_cnn_backward.
+ * Errors: SP_EINVAL, SP_ENOMEM, SP_EWORKSPACE, SP_ECUDA, SP_ETIMEOUT. */
 typedef struct sp_cnn sp_cnn;
 #define SP_CNN_MAX_BATCH 256
 int64_t sp_cnn_num_params(void);
 int sp_cnn_create(int32_t max_batch, uint64_t seed, sp_cnn **out);
 int sp_cnn_destroy(sp_cnn *c);
+int sp_cnn_status(sp_cnn *c, int32_t *h_status, int32_t clear);
 int sp_cnn_get_params(const sp_cnn *c, float *h_params);
 int sp_cnn_set_params(sp_cnn *c, const float *h_params);
 int sp_cnn_get_grads(const sp_cnn *c, float *h_grads);
@@ -670,7 +679,10 @@ int sp_cnn_extract(const sp_plan *plan, const uint8_t *d_staged, int64_t pitch, 
  *   without a classifier).
  * Every batch has its own status word: if a bounded wait of its
  *   dedispersion ran out, each gulp of that batch is returned with status
- *   SP_ETIMEOUT, count 0 and no candidates (its outputs are void). */
+ *   SP_ETIMEOUT, count 0 and no candidates (its outputs are void).  If one
+ *   of its peaks' classification did, the gulps scored together are returned
+ *   with status SP_ETIMEOUT, their candidates and peaks, scores -1 and
+ *   accepted 0. */
 typedef struct sp_stream sp_stream;
 typedef struct {
     int32_t beam;

@@ -115,6 +115,7 @@ SIGNATURES = {
     "sp_cnn_num_params": (I64, []),
     "sp_cnn_create": (ctypes.c_int, [I32, ctypes.c_uint64, P]),
     "sp_cnn_destroy": (ctypes.c_int, [P]),
+    "sp_cnn_status": (ctypes.c_int, [P, P, I32]),
     "sp_cnn_get_params": (ctypes.c_int, [P, P]),
     "sp_cnn_set_params": (ctypes.c_int, [P, P]),
     "sp_cnn_get_grads": (ctypes.c_int, [P, P]),
@@ -414,9 +415,9 @@ class Searcher:
 
 
 def debug_staging_fault(extra_bytes: int, wait_limit_cycles: int = 1 << 31):
-    """Test hook: make every dedispersion CTA's first staging wait expect
-    extra_bytes more than arrive, with waits bounded at wait_limit_cycles
-    (sp_debug_staging_fault); (0, 1 << 31) restores the defaults."""
+    """Test hook: make every dedispersion (and tensor-core classifier) CTA's
+    first staging wait expect extra_bytes more than arrive, with waits bounded at
+    wait_limit_cycles (sp_debug_staging_fault); (0, 1 << 31) restores the defaults."""
     _check(_lib().sp_debug_staging_fault(int(extra_bytes), int(wait_limit_cycles)), "sp_debug_staging_fault")
 
 
@@ -845,6 +846,12 @@ class Classifier:
                                         float(lr), ctypes.byref(loss) if want_loss else None, _stream(stream)),
                "sp_cnn_train_step")
         return float(loss.value) if want_loss else None
+
+    def status(self, clear: bool = False) -> int:
+        """Status word of the passes (0 = ok; SP_STATUS_STAGING_TIMEOUT: outputs void)."""
+        v = ctypes.c_int32()
+        _check(_lib().sp_cnn_status(self._h, ctypes.byref(v), int(clear)), "sp_cnn_status")
+        return int(v.value)
 
     def close(self):
         if getattr(self, "_h", None) is not None and self._h.value:

@@ -58,6 +58,7 @@ struct sp_cnn {
     float *wpart = nullptr;  // partial weight gradients of a layer
     float *flat = nullptr;  // parameters or gradients in the external order, on their way out
     std::mutex flat_lock;   // held while `flat` is filled and copied
+    int32_t *status = nullptr;  // page-locked, set by the tensor-core kernels (a bounded wait ran out)
     int64_t step = 0;
     bool have_grads = false;
 };
@@ -128,6 +129,7 @@ void free_cnn(sp_cnn *c) {
     cudaFree(c->wpart);
     cudaFree(c->prob);
     cudaFree(c->loss);
+    cudaFreeHost(c->status);
 }
 
 bool on_cnn_device(const sp_cnn *c) {
@@ -148,7 +150,7 @@ int upload_params(sp_cnn *c, int br, const std::vector<float> &h) {
 }
 
 int forward(sp_cnn *c, const __nv_bfloat16 *ft, const __nv_bfloat16 *dmt, int B, const float *labels, float *prob,
-            cudaStream_t st) {
+            int32_t *status, cudaStream_t st) {
     // Both branches' layers go in one launch each: with a few candidates a
     // layer is bound by its latency, not by its work.
     int rc = SP_OK;
@@ -162,7 +164,7 @@ int forward(sp_cnn *c, const __nv_bfloat16 *ft, const __nv_bfloat16 *dmt, int B,
             p.bias[bi] = b.params + b.off_b[l];
             p.y[bi] = b.y[l];
         }
-        rc = l == 0 ? cnn_conv0(p, B, kHin[l], kp_of(l), st) : cnn_conv_fwd(p, B, kHin[l], kCin[l], kp_of(l), st);
+        rc = l == 0 ? cnn_conv0(p, B, kHin[l], kp_of(l), st) : cnn_conv_fwd(p, B, kHin[l], kCin[l], kp_of(l), status, st);
         p.x[0] = p.y[0];
         p.x[1] = p.y[1];
     }
@@ -223,8 +225,8 @@ int backward(sp_cnn *c, const __nv_bfloat16 *ft, const __nv_bfloat16 *dmt, int B
         }
         rc = cnn_bias_part(p, (int64_t)B * ho_of(l) * ho_of(l), kCout[l], const_cast<float *>(sums.part[l]),
                            &sums.rows[l], st);
-        if (!rc) rc = cnn_conv_wgrad(p, B, H, C, Kp, c->wpart, st);
-        if (!rc) rc = cnn_conv_dgrad(p, B, H, C, Kp, st);
+        if (!rc) rc = cnn_conv_wgrad(p, B, H, C, Kp, c->wpart, c->status, st);
+        if (!rc) rc = cnn_conv_dgrad(p, B, H, C, Kp, c->status, st);
     }
     return rc ? rc : cnn_column_sums(sums, st);
 }
@@ -233,6 +235,16 @@ int check_batch(const sp_cnn *c, const void *ft, const void *dmt, int32_t B) {
     if (!c || !ft || !dmt || B < 1 || B > c->max_batch) return SP_EINVAL;
     if ((reinterpret_cast<uintptr_t>(ft) & 15) || (reinterpret_cast<uintptr_t>(dmt) & 15)) return SP_EINVAL;
     return on_cnn_device(c) ? SP_OK : SP_EINVAL;
+}
+
+// SP_ETIMEOUT, once, when a pass that the caller has waited for gave up a wait: its
+// gradients are void.
+int take_status(sp_cnn *c) {
+    volatile int32_t *s = c->status;
+    if (!*s) return SP_OK;
+    *s = 0;
+    c->have_grads = false;
+    return SP_ETIMEOUT;
 }
 
 }  // namespace
@@ -279,6 +291,12 @@ extern "C" int sp_cnn_create(int32_t max_batch, uint64_t seed, sp_cnn **out) {
     if (!rc) rc = dalloc((void **)&c->flat, 2 * flat_count() * 4);
     if (!rc) rc = dalloc((void **)&c->prob, B * 4);
     if (!rc) rc = dalloc((void **)&c->loss, 4);
+    if (!rc && cudaHostAlloc((void **)&c->status, sizeof(int32_t), cudaHostAllocPortable | cudaHostAllocMapped) !=
+                   cudaSuccess) {
+        cudaGetLastError();
+        rc = SP_ENOMEM;
+    }
+    if (!rc) *c->status = 0;
     // He-normal convolution weights, zero biases, small head weights.
     std::mt19937_64 gen(seed);
     for (int bi = 0; bi < 2 && !rc; ++bi) {
@@ -316,7 +334,7 @@ extern "C" int sp_cnn_destroy(sp_cnn *c) {
 static int get_flat(const sp_cnn *c, const float *b0, const float *b1, float *h) {
     sp_cnn *m = const_cast<sp_cnn *>(c);
     std::lock_guard<std::mutex> guard(m->flat_lock);
-    const int rc = cudaDeviceSynchronize() == cudaSuccess ? SP_OK : SP_ECUDA;
+    const int rc = cudaDeviceSynchronize() == cudaSuccess ? take_status(m) : SP_ECUDA;
     if (rc) return rc;
     FlatLayout f;
     f.segments = 0;
@@ -368,7 +386,15 @@ extern "C" int sp_cnn_forward(sp_cnn *c, const void *d_ft, const void *d_dmt, in
     if (rc) return rc;
     if (!d_prob) return SP_EINVAL;
     return forward(c, static_cast<const __nv_bfloat16 *>(d_ft), static_cast<const __nv_bfloat16 *>(d_dmt), batch,
-                   nullptr, d_prob, reinterpret_cast<cudaStream_t>(stream));
+                   nullptr, d_prob, c->status, reinterpret_cast<cudaStream_t>(stream));
+}
+
+extern "C" int sp_cnn_status(sp_cnn *c, int32_t *h_status, int32_t clear) {
+    if (!c || !h_status || !on_cnn_device(c)) return SP_EINVAL;
+    if (cudaDeviceSynchronize() != cudaSuccess) return SP_ECUDA;
+    *h_status = *(volatile int32_t *)c->status;
+    if (clear) take_status(c);
+    return SP_OK;
 }
 
 extern "C" int sp_cnn_backward(sp_cnn *c, const void *d_ft, const void *d_dmt, const float *d_labels, int32_t batch,
@@ -378,15 +404,16 @@ extern "C" int sp_cnn_backward(sp_cnn *c, const void *d_ft, const void *d_dmt, c
     if (!d_labels) return SP_EINVAL;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     rc = forward(c, static_cast<const __nv_bfloat16 *>(d_ft), static_cast<const __nv_bfloat16 *>(d_dmt), batch,
-                 d_labels, c->prob, st);
+                 d_labels, c->prob, c->status, st);
     if (!rc)
         rc = backward(c, static_cast<const __nv_bfloat16 *>(d_ft), static_cast<const __nv_bfloat16 *>(d_dmt), batch, st);
     if (rc) return rc;
     c->have_grads = true;
-    if (h_loss && (cudaMemcpyAsync(h_loss, c->loss, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-                   cudaStreamSynchronize(st) != cudaSuccess))
+    if (!h_loss) return SP_OK;
+    if (cudaMemcpyAsync(h_loss, c->loss, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaStreamSynchronize(st) != cudaSuccess)
         return SP_ECUDA;
-    return SP_OK;
+    return take_status(c);
 }
 
 extern "C" int sp_cnn_adam_step(sp_cnn *c, float lr, void *stream) {
@@ -474,4 +501,11 @@ extern "C" int sp_cnn_extract(const sp_plan *plan, const uint8_t *d_staged, int6
 namespace sp {
 int32_t cnn_max_batch(const sp_cnn *c) { return c ? c->max_batch : 0; }
 int cnn_device(const sp_cnn *c) { return c ? c->device : -1; }
+int cnn_forward(sp_cnn *c, const void *d_ft, const void *d_dmt, int32_t batch, float *d_prob, int32_t *status,
+                cudaStream_t st) {
+    const int rc = check_batch(c, d_ft, d_dmt, batch);
+    if (rc) return rc;
+    return forward(c, static_cast<const __nv_bfloat16 *>(d_ft), static_cast<const __nv_bfloat16 *>(d_dmt), batch,
+                   nullptr, d_prob, status, st);
+}
 }  // namespace sp

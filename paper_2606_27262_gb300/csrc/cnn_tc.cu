@@ -10,12 +10,14 @@
 // the last MMA all four warps read the accumulator from tensor memory
 // (tcgen05.ld) and apply the epilogue.  blockIdx.y is the branch: both
 // networks' layers run in one launch.  Every wait is bounded; a wait that runs
-// out skips the epilogue and sets the status word.
+// out skips the epilogue, waits (bounded) for the copies and MMAs in flight and sets
+// the caller's status word.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <atomic>
 #include <climits>
 #include <initializer_list>
 #include <mutex>
@@ -26,10 +28,17 @@ namespace sp {
 namespace {
 
 constexpr int kTcBM = 128;
-constexpr long long kTcWaitLimit = 1LL << 31;
 
-// Bit 0: a tensor-core kernel's wait ran out (its output is void).
-__device__ int g_tc_status = 0;
+// What bounds a kernel's waits, and the word it sets when one runs out (its output
+// is void then).  extra: bytes the first stage expects and nothing brings (test hook).
+struct Waits {
+    int32_t *status;
+    uint32_t extra;
+    long long limit;
+};
+std::atomic<uint32_t> g_extra{0};
+std::atomic<long long> g_limit{1LL << 31};
+Waits waits(int32_t *status) { return {status, g_extra.load(), g_limit.load()}; }
 
 __device__ __forceinline__ uint32_t s_addr32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -112,11 +121,11 @@ __device__ __forceinline__ bool mbar_try_tc(uint32_t bar, uint32_t parity) {
                  : "memory");
     return done != 0;
 }
-__device__ __forceinline__ bool mbar_wait_tc(uint32_t bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_wait_tc(uint32_t bar, uint32_t parity, long long limit) {
     if (mbar_try_tc(bar, parity)) return true;
     const long long t0 = clock64();
     while (!mbar_try_tc(bar, parity))
-        if (clock64() - t0 > kTcWaitLimit) return false;
+        if (clock64() - t0 > limit) return false;
     return true;
 }
 
@@ -158,32 +167,38 @@ struct Pipeline {
         tmem = *tmem_slot;
     }
     // copy(i, stage, full barrier) issues step i's copies (and its expect);
-    // multiply(i, stage address) its MMAs.  Returns whether the accumulator is complete.
+    // multiply(i, stage address) its MMAs.  Returns whether the accumulator is
+    // complete; if not, nothing is in flight any more (within the bounds of the waits).
     template <class Copy, class Multiply>
-    __device__ __forceinline__ bool run(int steps, Copy copy, Multiply multiply) {
+    __device__ __forceinline__ bool run(const Waits &w, int steps, Copy copy, Multiply multiply) {
         bool ok = true;
+        int copied = 0;  // steps
         if (warp == 0 && lane == 0) {
-            for (int i = 0; i < steps && ok; ++i) {
-                const int s = i % NS;
-                if (i >= NS) ok = mbar_wait_tc(empty0 + 8 * s, ((i / NS) - 1) & 1);
-                if (ok) copy(i, smem + s * STAGE, full0 + 8 * s);
+            for (; copied < steps; ++copied) {
+                const int s = copied % NS;
+                if (copied >= NS) ok = mbar_wait_tc(empty0 + 8 * s, ((copied / NS) - 1) & 1, w.limit);
+                if (!ok) break;
+                copy(copied, smem + s * STAGE, full0 + 8 * s);
             }
         } else if (warp == 1 && lane == 0) {
-            for (int i = 0; i < steps && ok; ++i) {
+            for (int i = 0; i < steps; ++i) {
                 const int s = i % NS;
-                ok = mbar_wait_tc(full0 + 8 * s, (i / NS) & 1);
+                ok = mbar_wait_tc(full0 + 8 * s, (i / NS) & 1, w.limit);
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 multiply(i, s_addr32(smem + s * STAGE));
                 mma_commit(empty0 + 8 * s);
             }
-            if (ok) mma_commit(done);
+            mma_commit(done);  // of the MMAs that were issued
         }
-        // Everyone waits for the last MMA (a role that gave up lets the wait run out).
-        ok = mbar_wait_tc(done, 0) && ok;
+        ok = mbar_wait_tc(done, 0, w.limit) && ok;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         ok = !__syncthreads_or(!ok);
-        if (!ok && threadIdx.x == 0) atomicOr(&g_tc_status, 1);
+        if (!ok && threadIdx.x == 0) {
+            // Copies that no MMA waited for may still be landing.
+            for (int i = max(0, copied - NS); i < copied; ++i) mbar_wait_tc(full0 + 8 * (i % NS), (i / NS) & 1, w.limit);
+            *(volatile int32_t *)w.status = SP_STATUS_STAGING_TIMEOUT;
+        }
         return ok;
     }
     __device__ __forceinline__ void finish() {
@@ -222,17 +237,17 @@ struct FwdShape {
 };
 template <int C, int NB>
 __global__ void __launch_bounds__(128) conv_fwd_kernel(const __grid_constant__ ConvMaps maps, const ConvOut out, int M,
-                                                       int lwo) {
+                                                       int lwo, const Waits w) {
     using S = FwdShape<C, NB>;
     extern __shared__ uint8_t smem_raw[];
     typename S::Pipe pipe(smem_raw);
     const bool branch = blockIdx.y;
     const int m0 = blockIdx.x * kTcBM, n0 = blockIdx.z * S::N;
     const bool ok = pipe.run(
-        S::STEPS,
+        w, S::STEPS,
         [&](int i, uint8_t *stage, uint32_t full) {
             const int tap = i / (C / S::KC), c0 = (i % (C / S::KC)) * S::KC;
-            expect(full, S::A_BYTES + S::B_BYTES);
+            expect(full, S::A_BYTES + S::B_BYTES + (i == 0 ? w.extra : 0u));
             load_box4(stage, &maps.a[branch], c0, tap % 3 - 1, 2 * tile_row(m0, lwo) + tap / 3 - 1, tile_image(m0, lwo), full);
             load_box2(stage + S::A_BYTES, &maps.b[branch], tap * C + c0, n0, full);
         },
@@ -302,7 +317,8 @@ struct WgradShape {
 };
 template <int C>
 __global__ void __launch_bounds__(128) conv_wgrad_kernel(const __grid_constant__ ConvMaps maps, int chunks,
-                                                         int chunks_per_split, int lwo, int Kp, float *__restrict__ part) {
+                                                         int chunks_per_split, int lwo, int Kp, float *__restrict__ part,
+                                                         const Waits w) {
     using S = WgradShape<C>;
     extern __shared__ uint8_t smem_raw[];
     typename S::Pipe pipe(smem_raw);
@@ -310,10 +326,10 @@ __global__ void __launch_bounds__(128) conv_wgrad_kernel(const __grid_constant__
     const int tile = blockIdx.x, first = blockIdx.z * chunks_per_split, n = min(chunks, first + chunks_per_split) - first;
     const int ntap = min(S::TAPS, 9 - tile * S::TAPS);
     const bool ok = pipe.run(
-        n,
+        w, n,
         [&](int i, uint8_t *stage, uint32_t full) {
             const int m0 = (first + i) * kTcBM;
-            expect(full, (uint32_t)(ntap * C / S::AC * S::A_BOX + S::B_BYTES));
+            expect(full, (uint32_t)(ntap * C / S::AC * S::A_BOX + S::B_BYTES) + (i == 0 ? w.extra : 0u));
             for (int t = 0; t < ntap; ++t) {
                 const int tap = tile * S::TAPS + t;
                 for (int c = 0; c < C / S::AC; ++c)
@@ -366,7 +382,8 @@ struct DgradShape {
 template <int C>
 __global__ void __launch_bounds__(128) conv_dgrad_kernel(const __grid_constant__ ConvMaps maps, const ConvOut out,
                                                          const __nv_bfloat16 *__restrict__ x0,
-                                                         const __nv_bfloat16 *__restrict__ x1, int M, int lwo) {
+                                                         const __nv_bfloat16 *__restrict__ x1, int M, int lwo,
+                                                         const Waits w) {
     using S = DgradShape<C>;
     extern __shared__ uint8_t smem_raw[];
     typename S::Pipe pipe(smem_raw);
@@ -389,11 +406,11 @@ __global__ void __launch_bounds__(128) conv_dgrad_kernel(const __grid_constant__
     fetch(0);
     // tap row (or column) u of shift d: d = 0: 1 (even pixels), 2 (odd); d = 1: 0 (odd)
     const bool ok = pipe.run(
-        4 * (S::CO / S::KC),
+        w, 4 * (S::CO / S::KC),
         [&](int i, uint8_t *stage, uint32_t full) {
             const int di = (i >> 1) & 1, dj = i & 1, k0 = (i >> 2) * S::KC;
             const int nu = di ? 1 : 2, nv = dj ? 1 : 2;
-            expect(full, (uint32_t)(S::A_BYTES + nu * nv * S::B_BYTES));
+            expect(full, (uint32_t)(S::A_BYTES + nu * nv * S::B_BYTES) + (i == 0 ? w.extra : 0u));
             load_box4(stage, &maps.a[branch], k0, dj, tile_row(m0, lwo) + di, tile_image(m0, lwo), full);
             uint8_t *b = stage + S::A_BYTES;
             for (int u = 0; u < nu; ++u)
@@ -544,7 +561,7 @@ int launched() {
 }
 
 template <int C, int NB>
-int fwd(const ConvPair &p, int Nb, int H, int Kp, cudaStream_t st) {
+int fwd(const ConvPair &p, int Nb, int H, int Kp, const Waits &w, cudaStream_t st) {
     using S = FwdShape<C, NB>;
     ConvMaps maps;
     ConvOut out;
@@ -559,12 +576,12 @@ int fwd(const ConvPair &p, int Nb, int H, int Kp, cudaStream_t st) {
     if (rc) return rc;
     const int M = Nb * (H / 2) * (H / 2);
     conv_fwd_kernel<C, NB><<<dim3((unsigned)((M + kTcBM - 1) / kTcBM), 2, NB), 128, S::Pipe::SMEM, st>>>(maps, out, M,
-                                                                                                       lwo_of(H / 2));
+                                                                                                       lwo_of(H / 2), w);
     return launched();
 }
 
 template <int C>
-int wgrad(const GradPair &p, int Nb, int H, int Kp, float *part, cudaStream_t st) {
+int wgrad(const GradPair &p, int Nb, int H, int Kp, float *part, const Waits &w, cudaStream_t st) {
     using S = WgradShape<C>;
     const int Ho = H / 2, M = Nb * Ho * Ho, chunks = (M + kTcBM - 1) / kTcBM;
     ConvMaps maps;
@@ -576,7 +593,8 @@ int wgrad(const GradPair &p, int Nb, int H, int Kp, float *part, cudaStream_t st
     if (rc) return rc;
     const int want = S::splits(chunks);
     const int per = (chunks + want - 1) / want, nz = (chunks + per - 1) / per;
-    conv_wgrad_kernel<C><<<dim3(S::MT, 2, (unsigned)nz), 128, S::Pipe::SMEM, st>>>(maps, chunks, per, lwo_of(Ho), Kp, part);
+    conv_wgrad_kernel<C><<<dim3(S::MT, 2, (unsigned)nz), 128, S::Pipe::SMEM, st>>>(maps, chunks, per, lwo_of(Ho), Kp, part,
+                                                                                                w);
     rc = launched();
     if (rc) return rc;
     // Many ranges of few values (layers 1, 2) need the lanes: 18 and 14 us without; few of many are slower with them
@@ -587,7 +605,7 @@ int wgrad(const GradPair &p, int Nb, int H, int Kp, float *part, cudaStream_t st
 }
 
 template <int C>
-int dgrad(const GradPair &p, int Nb, int H, int Kp, cudaStream_t st) {
+int dgrad(const GradPair &p, int Nb, int H, int Kp, const Waits &w, cudaStream_t st) {
     using S = DgradShape<C>;
     const int Ho = H / 2, M = Nb * Ho * Ho;
     ConvMaps maps;
@@ -601,7 +619,7 @@ int dgrad(const GradPair &p, int Nb, int H, int Kp, cudaStream_t st) {
     const int rc = limit.set(reinterpret_cast<const void *>(conv_dgrad_kernel<C>), S::Pipe::SMEM);
     if (rc) return rc;
     conv_dgrad_kernel<C><<<dim3((unsigned)((M + kTcBM - 1) / kTcBM), 2), 128, S::Pipe::SMEM, st>>>(maps, out, p.x[0], p.x[1], M,
-                                                                                                 lwo_of(Ho));
+                                                                                                 lwo_of(Ho), w);
     return launched();
 }
 
@@ -617,16 +635,17 @@ bool aligned(std::initializer_list<const void *> ps, uintptr_t to = 16) {
 
 }  // namespace
 
-int cnn_conv_fwd(const ConvPair &p, int Nb, int H, int C, int Kp, cudaStream_t st) {
+int cnn_conv_fwd(const ConvPair &p, int Nb, int H, int C, int Kp, int32_t *status, cudaStream_t st) {
     if (!shape_ok(Nb, H, C, Kp) || !aligned({p.x[0], p.x[1], p.w[0], p.w[1], p.y[0], p.y[1]})) return SP_EINVAL;
     // A few tiles leave SMs idle while each streams all of a layer's weights: where four times the CTAs still fit two
     // an SM, four share a tile's output channels (layers 3, 4 at batch 5: 11, 19 -> 7, 11 us; layer 4 at batch 64: 19 -> 13).
     const bool few = ((int64_t)Nb * (H / 2) * (H / 2) + kTcBM - 1) / kTcBM * 2 * 4 <= 2 * 152;
+    const Waits w = waits(status);
     switch (C) {
-        case 16: return fwd<16, 1>(p, Nb, H, Kp, st);
-        case 32: return fwd<32, 1>(p, Nb, H, Kp, st);
-        case 64: return few ? fwd<64, 4>(p, Nb, H, Kp, st) : fwd<64, 1>(p, Nb, H, Kp, st);
-        default: return few ? fwd<128, 4>(p, Nb, H, Kp, st) : fwd<128, 1>(p, Nb, H, Kp, st);
+        case 16: return fwd<16, 1>(p, Nb, H, Kp, w, st);
+        case 32: return fwd<32, 1>(p, Nb, H, Kp, w, st);
+        case 64: return few ? fwd<64, 4>(p, Nb, H, Kp, w, st) : fwd<64, 1>(p, Nb, H, Kp, w, st);
+        default: return few ? fwd<128, 4>(p, Nb, H, Kp, w, st) : fwd<128, 1>(p, Nb, H, Kp, w, st);
     }
 }
 
@@ -639,39 +658,33 @@ int64_t cnn_wgrad_part_floats(int Nb, int H, int C, int Kp) {
     return (int64_t)nz * 2 * 2 * C * Kp;
 }
 
-int cnn_conv_wgrad(const GradPair &p, int Nb, int H, int C, int Kp, float *part, cudaStream_t st) {
+int cnn_conv_wgrad(const GradPair &p, int Nb, int H, int C, int Kp, float *part, int32_t *status, cudaStream_t st) {
     if (!shape_ok(Nb, H, C, Kp) || !aligned({p.x[0], p.x[1], p.dz[0], p.dz[1]})) return SP_EINVAL;
+    const Waits w = waits(status);
     switch (C) {
-        case 16: return wgrad<16>(p, Nb, H, Kp, part, st);
-        case 32: return wgrad<32>(p, Nb, H, Kp, part, st);
-        case 64: return wgrad<64>(p, Nb, H, Kp, part, st);
-        default: return wgrad<128>(p, Nb, H, Kp, part, st);
+        case 16: return wgrad<16>(p, Nb, H, Kp, part, w, st);
+        case 32: return wgrad<32>(p, Nb, H, Kp, part, w, st);
+        case 64: return wgrad<64>(p, Nb, H, Kp, part, w, st);
+        default: return wgrad<128>(p, Nb, H, Kp, part, w, st);
     }
 }
 
-int cnn_conv_dgrad(const GradPair &p, int Nb, int H, int C, int Kp, cudaStream_t st) {
+int cnn_conv_dgrad(const GradPair &p, int Nb, int H, int C, int Kp, int32_t *status, cudaStream_t st) {
     if (!shape_ok(Nb, H, C, Kp) || !aligned({p.dz[0], p.dz[1], p.w[0], p.w[1]}) ||
         !aligned({p.x[0], p.x[1], p.dx[0], p.dx[1]}, 32))
         return SP_EINVAL;
+    const Waits w = waits(status);
     switch (C) {
-        case 16: return dgrad<16>(p, Nb, H, Kp, st);
-        case 32: return dgrad<32>(p, Nb, H, Kp, st);
-        case 64: return dgrad<64>(p, Nb, H, Kp, st);
-        default: return dgrad<128>(p, Nb, H, Kp, st);
+        case 16: return dgrad<16>(p, Nb, H, Kp, w, st);
+        case 32: return dgrad<32>(p, Nb, H, Kp, w, st);
+        case 64: return dgrad<64>(p, Nb, H, Kp, w, st);
+        default: return dgrad<128>(p, Nb, H, Kp, w, st);
     }
 }
 
-int cnn_tc_status(int *h_status, bool clear) {
-    if (cudaMemcpyFromSymbol(h_status, g_tc_status, sizeof(int)) != cudaSuccess) {
-        cudaGetLastError();
-        return SP_ECUDA;
-    }
-    const int zero = 0;
-    if (clear && cudaMemcpyToSymbol(g_tc_status, &zero, sizeof(int)) != cudaSuccess) {
-        cudaGetLastError();
-        return SP_ECUDA;
-    }
-    return SP_OK;
+void set_tc_fault(uint32_t extra_bytes, long long wait_limit) {
+    g_extra = std::min(extra_bytes, 1u << 16);  // with a stage's own bytes inside a barrier's 20 bits
+    g_limit = wait_limit;
 }
 
 }  // namespace sp

@@ -22,7 +22,8 @@ struct ConvPair {
 // [2 C][Kp] bf16 (k = tap*C + c; Kp >= 9 C, a multiple of 8), y and dz
 // [Nb*(H/2)^2][2 C] bf16, all 16-byte aligned; C 16..128, H 128..16, powers of two.
 // y = relu(conv(x) + bias).
-int cnn_conv_fwd(const ConvPair &p, int Nb, int H, int C, int Kp, cudaStream_t st);
+// A wait of theirs that runs out sets *status (host-visible) to SP_STATUS_STAGING_TIMEOUT.
+int cnn_conv_fwd(const ConvPair &p, int Nb, int H, int C, int Kp, int32_t *status, cudaStream_t st);
 // Operands of a layer's gradients: input x, dz (of the layer's output before its
 // ReLU), weights; dx is the dz of the layer below, dw fp32 [2 C][Kp].
 struct GradPair {
@@ -33,11 +34,9 @@ struct GradPair {
 // dw += dz^T x (part: cnn_wgrad_part_floats of at least Nb, workspace; the split
 // over pixels and the order of its sums depend on the shape only).
 int64_t cnn_wgrad_part_floats(int Nb, int H, int C, int Kp);
-int cnn_conv_wgrad(const GradPair &p, int Nb, int H, int C, int Kp, float *part, cudaStream_t st);
+int cnn_conv_wgrad(const GradPair &p, int Nb, int H, int C, int Kp, float *part, int32_t *status, cudaStream_t st);
 // dx = (transposed convolution of dz) where x > 0, else 0 (x and dx 32-byte aligned).
-int cnn_conv_dgrad(const GradPair &p, int Nb, int H, int C, int Kp, cudaStream_t st);
-// Device status of these kernels (bit 0: a wait ran out).
-int cnn_tc_status(int *h_status, bool clear);
+int cnn_conv_dgrad(const GradPair &p, int Nb, int H, int C, int Kp, int32_t *status, cudaStream_t st);
 // Layer 0 of both branches (one input channel, 16 outputs, 3x3, stride 2,
 // padding 1) as a direct convolution with bias and ReLU: x [Nb][H][H] (H a
 // multiple of 8), y [Nb*(H/2)^2][16] bf16, both 16-byte aligned, weights w

@@ -287,5 +287,10 @@ uint64_t capture_end();
 // Facts about a classifier that the streaming search needs (cnn.cpp).
 int32_t cnn_max_batch(const sp_cnn *c);
 int cnn_device(const sp_cnn *c);
+// sp_cnn_forward that reports a wait that ran out in *status (page-locked) instead of the handle's word.
+int cnn_forward(sp_cnn *c, const void *d_ft, const void *d_dmt, int32_t batch, float *d_prob, int32_t *status,
+                cudaStream_t st);
+// Test hook of the classifier's bounded waits.
+void set_tc_fault(uint32_t extra_bytes, long long wait_limit);
 
 }  // namespace sp

@@ -106,6 +106,7 @@ struct JobRec {  // a classification job (FIFO on the classifier stream)
     cudaEvent_t done = nullptr;
     sp_cand *h_kept = nullptr;     // pinned [kClsCap]
     float *h_prob = nullptr;       // pinned [kClsCap]
+    int32_t *h_status = nullptr;   // pinned, set by the classifier's kernels (a bounded wait ran out)
     std::vector<Result> rs;        // the gulps it scores, their slots and first peaks
     std::vector<int> slots;
     std::vector<int32_t> first;
@@ -206,6 +207,7 @@ void cls_free(sp_stream *s) {
         JobRec &j = s->recs[i];
         cudaFreeHost(j.h_kept);
         cudaFreeHost(j.h_prob);
+        cudaFreeHost(j.h_status);
         if (j.done) cudaEventDestroy(j.done);
     }
     s->recs.reset();
@@ -420,6 +422,7 @@ int dispatch_job(sp_stream *s) {
     const sp_plan *p = s->plan;
     cudaStream_t st = s->cls_stream;
     j.finished.store(0, std::memory_order_relaxed);
+    *j.h_status = 0;  // the record's last job has been collected
     int rc = SP_OK;
     if (cudaMemcpyAsync(s->d_kept, j.h_kept, (size_t)j.total * sizeof(sp_cand), cudaMemcpyHostToDevice, st) !=
         cudaSuccess)
@@ -434,9 +437,8 @@ int dispatch_job(sp_stream *s) {
     const int32_t bmax = cnn_max_batch(s->clf);
     const int64_t img = (int64_t)256 * 256 * 2;  // bytes of one bf16 image
     for (int32_t i = 0; i < j.total && !rc; i += bmax)
-        rc = sp_cnn_forward(s->clf, static_cast<uint8_t *>(s->d_ft) + i * img,
-                            static_cast<uint8_t *>(s->d_img) + i * img, std::min(bmax, j.total - i), s->d_prob + i,
-                            st);
+        rc = cnn_forward(s->clf, static_cast<uint8_t *>(s->d_ft) + i * img, static_cast<uint8_t *>(s->d_img) + i * img,
+                         std::min(bmax, j.total - i), s->d_prob + i, j.h_status, st);
     if (!rc &&
         (cudaMemcpyAsync(j.h_prob, s->d_prob, (size_t)j.total * 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
          cudaLaunchHostFunc(st, mark_classified, &j) != cudaSuccess || cudaEventRecord(j.done, st) != cudaSuccess))
@@ -520,10 +522,15 @@ int progress(sp_stream *s) {
         for (long spins = 0; !j.finished.load(std::memory_order_acquire) && spins < (1L << 26); ++spins) {
         }
         const double t_done = j.finished.load(std::memory_order_acquire) ? j.t_done : now_s();
+        const bool timeout = *(volatile int32_t *)j.h_status != 0;  // the job's scores are void
         for (size_t g = 0; g < j.rs.size(); ++g) {
             Result &r = j.rs[g];
             r.prob.assign(j.h_prob + j.first[g], j.h_prob + j.first[g] + r.kept.size());
             r.info.accepted = 0;
+            if (timeout) {
+                r.info.status = SP_ETIMEOUT;
+                r.prob.assign(r.kept.size(), -1.0f);
+            }
             for (float v : r.prob) r.info.accepted += v >= 0.5f;
             r.info.t_done = t_done;
             s->results.push_back(std::move(r));
@@ -858,6 +865,7 @@ extern "C" int sp_stream_attach(sp_stream *s, const sp_sift_params *params, sp_c
             JobRec &j = s->recs[i];
             rc = alloc_host((void **)&j.h_kept, (int64_t)kClsCap * (int64_t)sizeof(sp_cand));
             if (!rc) rc = alloc_host((void **)&j.h_prob, (int64_t)kClsCap * 4);
+            if (!rc) rc = alloc_host((void **)&j.h_status, sizeof(int32_t));
             if (!rc && cudaEventCreateWithFlags(&j.done, cudaEventDisableTiming) != cudaSuccess) {
                 cudaGetLastError();
                 rc = SP_ECUDA;
