@@ -70,6 +70,9 @@ const char *sp_strerror(int code);
  * at capture.  (A graph the caller captures around library calls counts its
  * kernels once, when they are recorded.)  Never fails. */
 uint64_t sp_launch_count(void);
+/* Of these, the launches of the shared-sum dedispersion kernel: which of the
+ * two dedispersion kernels a call ran. */
+uint64_t sp_sums_launch_count(void);
 
 /* ------------------------------------------------------------------ plan --
  * Dedispersion plan (Sec. 3.1.1).  For trial DM d and channel c the delay is

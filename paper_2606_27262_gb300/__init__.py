@@ -20,7 +20,7 @@ Names mirror the C entry points:
 * ``sift``                       sp_sift (DBSCAN clustering + thresholds, host)
 * ``inject_quantised``           sp_inject_quantised (Appendix B injection)
 * ``Classifier``, ``cnn_features``, ``dmt_shifts``  sp_cnn_* (two-image CNN)
-* ``launch_count``               sp_launch_count (kernels issued, for measurement)
+* ``launch_count``, ``sums_launch_count``  sp_launch_count, sp_sums_launch_count (kernels issued, for measurement)
 """
 from __future__ import annotations
 
@@ -108,6 +108,7 @@ SIGNATURES = {
     "sp_stream_now": (F64, []),
     "sp_stream_attach": (ctypes.c_int, [P, P, P, I32, I32]),
     "sp_launch_count": (ctypes.c_uint64, []),
+    "sp_sums_launch_count": (ctypes.c_uint64, []),
     "sp_plan_check_tables": (ctypes.c_int, [P, I32, F64, P, I32, I32, I64, P]),
     "sp_stream_poll_sifted": (ctypes.c_int, [P, I32, P, P, P, P, I32, P]),
     "sp_sift": (ctypes.c_int, [P, I64, P, I32, P, I32, F64, P, P, I64, P, P]),
@@ -598,6 +599,12 @@ def launch_count() -> int:
     """Kernel launches the library has issued in this process
     (sp_launch_count; graph kernels count once per replay)."""
     return int(_lib().sp_launch_count())
+
+
+def sums_launch_count() -> int:
+    """Of these, the launches of the shared-sum dedispersion kernel
+    (sp_sums_launch_count)."""
+    return int(_lib().sp_sums_launch_count())
 
 
 def stream_now() -> float:

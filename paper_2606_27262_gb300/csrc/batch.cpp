@@ -185,7 +185,7 @@ struct sp_batch {
     std::vector<cudaEvent_t> ev_t0, ev_t1;     // per group, around its persistent launch (timed runs)
     bool timed_valid = false;
     cudaGraphExec_t graph = nullptr;
-    uint64_t graph_kernels = 0;  // kernels recorded in the graph
+    Launches graph_kernels;      // kernels recorded in the graph
     int last_mode = -1;
 };
 
@@ -534,7 +534,7 @@ extern "C" int sp_batch_capture(sp_batch *b, int32_t mode, void *stream) {
     }
     capture_begin();
     const int rc = run_mode(b, mode, s0);
-    const uint64_t kernels = capture_end();
+    const Launches kernels = capture_end();
     cudaGraph_t graph = nullptr;
     const cudaError_t e = cudaStreamEndCapture(s0, &graph);
     if (rc || e != cudaSuccess || !graph) {
@@ -558,7 +558,7 @@ extern "C" int sp_batch_capture(sp_batch *b, int32_t mode, void *stream) {
 extern "C" int sp_batch_launch(sp_batch *b, void *stream) {
     if (!b || !b->graph || !on_device(b)) return SP_EINVAL;
     if (cudaGraphLaunch(b->graph, reinterpret_cast<cudaStream_t>(stream)) != cudaSuccess) return SP_ECUDA;
-    note_launch(b->graph_kernels);
+    note_launch(b->graph_kernels.all, b->graph_kernels.sums);
     return SP_OK;
 }
 

@@ -59,27 +59,32 @@ int sps_common(const int32_t *d_dmt, int32_t ndm, int64_t n_out, const int32_t *
 
 namespace sp {
 namespace {
-std::atomic<uint64_t> g_launches{0};
+std::atomic<uint64_t> g_launches{0}, g_sums_launches{0};
 thread_local bool t_capturing = false;  // launches go into a graph, not to the GPU
-thread_local uint64_t t_captured = 0;
+thread_local Launches t_captured;
 }  // namespace
-void note_launch(uint64_t n) {
-    if (t_capturing)
-        t_captured += n;
-    else
+void note_launch(uint64_t n, uint64_t sums) {
+    if (t_capturing) {
+        t_captured.all += n;
+        t_captured.sums += sums;
+    } else {
         g_launches.fetch_add(n, std::memory_order_relaxed);
+        if (sums) g_sums_launches.fetch_add(sums, std::memory_order_relaxed);
+    }
 }
 void capture_begin() {
     t_capturing = true;
-    t_captured = 0;
+    t_captured = Launches();
 }
-uint64_t capture_end() {
+Launches capture_end() {
     t_capturing = false;
     return t_captured;
 }
 }  // namespace sp
 
 extern "C" uint64_t sp_launch_count(void) { return sp::g_launches.load(std::memory_order_relaxed); }
+
+extern "C" uint64_t sp_sums_launch_count(void) { return sp::g_sums_launches.load(std::memory_order_relaxed); }
 
 extern "C" const char *sp_strerror(int code) {
     switch (code) {

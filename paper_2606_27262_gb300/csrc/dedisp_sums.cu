@@ -536,7 +536,7 @@ int launch_dedisperse_sums(const sp_plan *plan, const uint8_t *d_xt, int64_t pit
     const int64_t ntime = (n_out + kSumTime - 1) / kSumTime;
     dedisp_sums_kernel<<<(unsigned)(ntime * plan->sums_ntiles), kThreads, kSumSmem, stream>>>(
         d_xt, pitch, n_out, d_out, plan->d_sums, ntime, status ? status : plan->d_status);
-    note_launch();
+    note_launch(1, 1);
     return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
 }
 
@@ -546,7 +546,7 @@ int launch_dedisperse_sums_batch(const BatchLaunch &b, cudaStream_t stream) {
     if (rc) return rc;
     dedisp_sums_items_kernel<<<(unsigned)b.nitems, kThreads, kSumSmem, stream>>>(b.d_beams, b.d_item_begin, b.nbeams,
                                                                                b.d_status);
-    note_launch();
+    note_launch(1, 1);
     return cudaGetLastError() == cudaSuccess ? SP_OK : SP_ECUDA;
 }
 

@@ -280,9 +280,12 @@ int check_widths(const int32_t *w, int32_t nw);
 // Between capture_begin and capture_end the calling thread's launches are
 // recorded into a graph: they are counted for the graph (capture_end
 // returns how many) instead of as launches.
-void note_launch(uint64_t n = 1);
+void note_launch(uint64_t n = 1, uint64_t sums = 0);  // sums: of them, shared-sum dedispersion kernels
 void capture_begin();
-uint64_t capture_end();
+struct Launches {
+    uint64_t all = 0, sums = 0;
+};
+Launches capture_end();
 
 // Facts about a classifier that the streaming search needs (cnn.cpp).
 int32_t cnn_max_batch(const sp_cnn *c);
