@@ -178,7 +178,6 @@ static int upload_sums(sp_plan *p, const SumTables &t) {
     if (cudaMemcpy(d, h.data(), h.size(), cudaMemcpyHostToDevice) != cudaSuccess) return SP_ECUDA;
     p->d_sums = reinterpret_cast<SumTablesDev *>(d);
     p->sums_ntiles = v.ntiles;
-    p->sums_tile_clocks = t.tile_clocks;
     return SP_OK;
 }
 
@@ -256,7 +255,8 @@ static int create_plan(const double *freqs_mhz, int32_t nchan, double tsamp_s, c
 
     int smem_optin = 0;
     if (cudaGetDevice(&p->device) != cudaSuccess ||
-        cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device) != cudaSuccess) {
+        cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess) {
         cudaGetLastError();
         delete p;
         return SP_ECUDA;
@@ -276,9 +276,12 @@ static int create_plan(const double *freqs_mhz, int32_t nchan, double tsamp_s, c
         // Without room for these tables, here or on the device, the plan is the direct kernel's as well.
         try {
             SumTables t;
-            if (build_sum_tables(*p, t) == SP_OK && sum_tables_pay(*p, t)) {
-                rc = upload_sums(p, t);
-                if (!rc) rc = sums_configure();
+            if (build_sum_tables(*p, t) == SP_OK) {
+                model_items(*p, t);
+                if (sum_tables_pay(*p, t)) {
+                    rc = upload_sums(p, t);
+                    if (!rc) rc = sums_configure();
+                }
             }
         } catch (const std::bad_alloc &) {
             rc = SP_ENOMEM;

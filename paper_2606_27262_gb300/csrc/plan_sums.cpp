@@ -342,6 +342,15 @@ void build_tile(const sp_plan &p, int32_t d0, int cnt, Tile &t) {
 
 }  // namespace
 
+// SM clocks of a work item of a tile: a fixed part (set-up, first copies, output), its
+// groups' modelled clocks, what a job costs besides, and the producers' time
+// that consumers without trials do not cover.  Fitted to 32 plans (64 to 16384 channels,
+// steps of 0.02 to 4, 9 to 64 trials a tile) with an item an SM.
+static double item_clocks(const Tile &t, int32_t cnt) {
+    return 38000.0 + 0.81 * t.clocks + 26.0 * (double)(t.jobs.size() / 2) +
+           550.0 * t.ngroups * (kSumDms - cnt) / kSumDms;
+}
+
 // Tiles of up to kSumDms consecutive DMs, halved where a tile's delay spread
 // leaves no group that fits a row slot.  SP_ELIMIT: the plan has no tables
 // (too many channels for the 16-bit carries, or a table beyond int32).
@@ -385,6 +394,7 @@ static int build_tables(const sp_plan &p, SumTables &t) {
     run_on_cores(work, (int64_t)spans.size());
     if (bad) return no_memory ? SP_ENOMEM : SP_ELIMIT;
     double clocks = 0.0;
+    t.tile_most = 0.0;
     t.tile_chunk.push_back(0);
     t.tile_group.push_back(0);
     t.tile_job.push_back(0);
@@ -412,7 +422,9 @@ static int build_tables(const sp_plan &p, SumTables &t) {
             t.tile_job.push_back((int32_t)(t.jobs.size() / 2));
             t.tile_chunk.push_back(t.tile_chunk.back() + x.nchunks);
             t.tile_group.push_back(t.tile_group.back() + x.ngroups);
-            clocks += x.clocks;
+            const double item = item_clocks(x, s.counts[k]);
+            clocks += item;
+            t.tile_most = std::max(t.tile_most, item);
         }
     }
     t.tile_clocks = clocks / (double)t.tile_first.size();
@@ -428,44 +440,84 @@ int build_sum_tables(const sp_plan &p, SumTables &t) {
 }
 
 namespace {
-// The direct kernel (dedisperse.cu) adds 74 channel x DM x sample sums per SM
-// and clock: 133 ms for the 5751-trial, 4096-channel, 131072-sample transform
-// on 152 SMs at 2.07 GHz.  The shared-sum kernel takes 0.97 to 1.14 of its
-// modelled clocks over that plan's four DM steps (48.5 ms in all).
-constexpr double kDirectAddsPerClock = 74.0;
-constexpr double kModelRatio = 1.05;
-constexpr double kSms = 152.0;
-double direct_tile_clocks(const sp_plan &p) {
-    return (double)p.ndm / p.ntiles * p.time_tile * p.nchan / kDirectAddsPerClock;
+// Direct kernel: 74 sums per SM and clock on full tiles with two items on an SM; a
+// tile of few trials costs more than its share (it loads the same samples, and
+// half its threads or more have no trials).  alone: an item that has its SM to itself.
+constexpr double kDirectFixedClocks = 4000.0, kDirectAddsPerClock = 74.0;
+constexpr double kDirectAlone = 1.32, kDirectWaves = 0.97;
+double direct_item_clocks(const sp_plan &p, int32_t tile, bool alone) {
+    const double full = (double)p.tile_count[(size_t)tile] / p.dm_tile;
+    const double part = full > 0.5 ? 0.6 + 0.4 * full : alone ? 0.54 + 0.34 * full : 0.4 + 0.44 * full;
+    return kDirectFixedClocks + part * p.dm_tile * p.time_tile * p.nchan / kDirectAddsPerClock;
 }
 }  // namespace
+
+// The plan's modelled clocks of its items: shared sums and direct, average and largest.
+void model_items(sp_plan &p, const SumTables &t) {
+    p.sums_clocks = t.tile_clocks;
+    p.sums_most = t.tile_most;
+    p.direct_clocks = p.direct_most = p.direct_alone = 0.0;
+    for (int32_t j = 0; j < p.ntiles; ++j) {
+        const double item = direct_item_clocks(p, j, false);
+        p.direct_clocks += item / p.ntiles;
+        p.direct_most = std::max(p.direct_most, item);
+        p.direct_alone = std::max(p.direct_alone, direct_item_clocks(p, j, true));
+    }
+}
 
 // Whether a plan keeps shared-sum tables: on long inputs they beat the direct
 // kernel.  DM lists whose trials share too little (coarse steps on few
 // channels, random lists) stay with the direct kernel.
 bool sum_tables_pay(const sp_plan &p, const SumTables &t) {
-    return t.tile_clocks * kModelRatio * (double)t.tile_first.size() / kSumTime <
-           direct_tile_clocks(p) * p.ntiles / p.time_tile;
+    return p.sums_clocks * (double)t.tile_first.size() / kSumTime <
+           kDirectWaves * p.direct_clocks * p.ntiles / p.time_tile;
+}
+
+// Modelled clocks of one launch over these beams with either kernel.  Shared
+// sums run in whole waves of an item an SM; the direct kernel's items share an
+// SM as soon as they are more than the SMs.  A launch takes at least its largest item.
+// Measured on 642 launches, from one item to twenty waves, of the plans that item_clocks
+// was fitted to and of 45 others (trial lists of 100 to 900 pc cm^-3, 256 to 4096
+// channels): nine in ten shared-sum launches take 0.97 to 1.12 of this, nine in ten
+// direct launches 0.97 to 1.17.  None goes to shared sums that take longer than the
+// direct kernel; 16 stay with the direct kernel and are 2 to 12 % slower.  Among them, us
+// with the direct kernel and with shared sums: 4096 channels, 129 trials 1.0 apart,
+// 700 samples 843, 917, 16384 samples 1101, 924; 64 channels, 512 trials 0.1 apart,
+// 2048 samples 26, 41; 1024 channels, 512 trials 0.1 apart, 2048 samples 293, 172.
+DedispClocks dedisp_clocks(const sp_plan *const *plans, const int64_t *n_out, int32_t nbeams) {
+    DedispClocks c;
+    double sums = 0.0, direct = 0.0, direct_items = 0.0, sms = 1.0, sums_most = 0.0, direct_most = 0.0, alone = 0.0;
+    for (int32_t b = 0; b < nbeams; ++b) {
+        const sp_plan &p = *plans[b];
+        const double si = (double)sums_items(&p, n_out[b]), di = (double)p.ntiles * (double)dedisp_time_tiles(&p, n_out[b]);
+        c.sum_items += si;
+        direct_items += di;
+        sums += si * p.sums_clocks;
+        direct += di * p.direct_clocks;
+        sums_most = std::max(sums_most, p.sums_most);
+        direct_most = std::max(direct_most, p.direct_most);
+        alone = std::max(alone, p.direct_alone);
+        sms = p.sms;
+    }
+    c.sums = std::max(sums_most, std::ceil(c.sum_items / sms) * sums / c.sum_items);
+    const double half_waves = std::ceil(direct_items / sms);
+    if (half_waves <= 1.0) {
+        c.direct = kDirectAlone * alone;
+        return c;
+    }
+    c.direct = kDirectWaves * std::max(2.0 * direct_most, half_waves * direct / direct_items);
+    if (half_waves == 3.0 || half_waves == 5.0)  // full waves, then items alone
+        c.direct = std::max(c.direct, kDirectWaves * (half_waves - 1.0) * direct / direct_items + 0.9 * kDirectAlone * alone);
+    return c;
 }
 
 // Whether one launch over these beams goes to the shared-sum kernel: all plans
-// have tables, and the modelled clocks are fewer.  Its items are larger (one
-// CTA of 1024 samples per SM; two CTAs of 512 for the direct kernel), so a
-// short input can fill fewer, longer waves: full waves are compared.
+// have tables, and the modelled clocks are fewer.
 bool sums_pay(const sp_plan *const *plans, const int64_t *n_out, int32_t nbeams) {
-    double sums = 0.0, direct = 0.0, sum_items = 0.0, direct_items = 0.0;
-    for (int32_t b = 0; b < nbeams; ++b) {
-        const sp_plan &p = *plans[b];
-        if (!p.d_sums) return false;
-        const double si = (double)sums_items(&p, n_out[b]), di = (double)p.ntiles * (double)dedisp_time_tiles(&p, n_out[b]);
-        sums += si * p.sums_tile_clocks * kModelRatio;
-        direct += di * direct_tile_clocks(p);
-        sum_items += si;
-        direct_items += di;
-    }
-    if (sum_items > INT32_MAX) return false;
-    auto waves = [](double items, double at_once) { return std::ceil(items / at_once) * at_once / items; };
-    return sums * waves(sum_items, kSms) < direct * waves(direct_items, 2.0 * kSms);
+    for (int32_t b = 0; b < nbeams; ++b)
+        if (!plans[b]->d_sums) return false;
+    const DedispClocks c = dedisp_clocks(plans, n_out, nbeams);
+    return c.sum_items <= INT32_MAX && c.sums < c.direct;
 }
 
 int64_t sums_items(const sp_plan *p, int64_t n_out) {

@@ -103,7 +103,7 @@ constexpr int kSumMinJobs = kSumHalf / 128;  // of a chunk: a row has at least k
 struct SumTables {
     std::vector<int32_t> tile_first, tile_count, tile_chunk, tile_group, tile_job, chunks, prog_bytes, geo, off;
     std::vector<uint32_t> prog, jobs;
-    double tile_clocks = 0.0;  // modelled SM clocks of an average work item
+    double tile_clocks = 0.0, tile_most = 0.0;  // modelled SM clocks of a work item: average, largest
 };
 
 }  // namespace sp
@@ -142,7 +142,10 @@ struct sp_plan {
     sp::SumTablesDev *d_sums = nullptr;
     void *d_sums_mem = nullptr;
     int32_t sums_ntiles = 0;
-    double sums_tile_clocks = 0.0;
+    // For the choice between the two kernels: SMs of the device, modelled clocks of
+    // a work item (average, largest).
+    int32_t sms = 1;
+    double sums_clocks = 0.0, sums_most = 0.0, direct_clocks = 0.0, direct_most = 0.0, direct_alone = 0.0;
 };
 
 namespace sp {
@@ -196,6 +199,11 @@ int64_t dedisp_time_tiles(const sp_plan *plan, int64_t n_out);
 // Shared-sum kernel: whether a launch over these beams goes to it
 // (plan_sums.cpp), its tables, its launches.
 bool sums_pay(const sp_plan *const *plans, const int64_t *n_out, int32_t nbeams);
+struct DedispClocks {
+    double sums = 0.0, direct = 0.0, sum_items = 0.0;
+};
+DedispClocks dedisp_clocks(const sp_plan *const *plans, const int64_t *n_out, int32_t nbeams);
+void model_items(sp_plan &p, const SumTables &t);
 int build_sum_tables(const sp_plan &p, SumTables &t);
 bool sum_tables_pay(const sp_plan &p, const SumTables &t);
 int64_t check_sum_tables(const sp_plan &p, const SumTables &t, int64_t n_out);

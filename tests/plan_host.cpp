@@ -113,10 +113,31 @@ static int late_band(bool apart) {
     return rc || report[5] || report[6] < 800000000 || seconds > 2.0;
 }
 
+// Which kernel launches of a plan go to (1: shared sums), and their modelled clocks: channels, first
+// trial, step, trials, then lengths.
+static int clocks(int argc, char **argv) {
+    const int nchan = std::atoi(argv[2]), ndm = std::atoi(argv[5]);
+    const double first = std::atof(argv[3]), step = std::atof(argv[4]);
+    const std::vector<double> f = band(nchan);
+    std::vector<double> dms;
+    for (int d = 0; d < ndm; ++d) dms.push_back(first + step * d);
+    sp_plan *p = nullptr;
+    if (sp_plan_create(f.data(), nchan, 1.31072e-3, dms.data(), ndm, &p)) return 1;
+    for (int i = 6; i < argc; ++i) {
+        const int64_t n_out = std::atoll(argv[i]);
+        const sp::DedispClocks c = sp::dedisp_clocks(&p, &n_out, 1);
+        std::printf("%lld %d %d %.0f %.0f\n", (long long)n_out, p->d_sums != nullptr, sp::sums_pay(&p, &n_out, 1),
+                    c.sums, c.direct);
+    }
+    sp_plan_destroy(p);
+    return 0;
+}
+
 int main(int argc, char **argv) {
     const std::string what = argc > 1 ? argv[1] : "";
     if (what == "blocks") return blocks();
     if (what == "no_room") return no_room();
     if (what == "late_band") return late_band(argc > 2);
+    if (what == "clocks" && argc > 6) return clocks(argc, argv);
     return 2;
 }

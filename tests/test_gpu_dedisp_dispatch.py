@@ -31,11 +31,12 @@ def _sums_launches(call):
     return sp.sums_launch_count() - before, out
 
 
-# Direct and shared-sum time of each on one GB300, us: 290 and 172; 294 and 226; 1134 and 347; 1109 and 924; 210 and 333.
-# The last has no tables.
+# Direct and shared-sum time of each on one GB300, us: 290 and 172; 294 and 226; 1134 and 347; 1109 and 924; 1109 and
+# 923; 843 and 917; 210 and 333; 26 and 41 (no tables).  The last has no tables either.
 @pytest.mark.parametrize("nchan,kind,ndm,n_out,sums", [
     (1024, "fine", 512, 1025, 1), (1024, "mid", 512, 1500, 1), (4096, "fine", 64, 513, 1),
-    (4096, "coarse", 129, 20001, 1), (1024, "coarse", 256, 1500, 0), (64, "coarse", 96, 2048, 0),
+    (4096, "coarse", 129, 20001, 1), (4096, "coarse", 256, 12288, 1), (4096, "coarse", 129, 700, 0),
+    (1024, "coarse", 256, 1500, 0), (64, "fine", 512, 2048, 0), (64, "coarse", 96, 2048, 0),
 ])
 def test_kernel_of_a_call(nchan, kind, ndm, n_out, sums):
     f, dms = synth.band_freqs(nchan), _dms(kind, ndm)
