@@ -484,12 +484,13 @@ bool sum_tables_pay(const sp_plan &p, const SumTables &t) {
 // with the direct kernel and with shared sums: 4096 channels, 129 trials 1.0 apart,
 // 700 samples 843, 917, 16384 samples 1101, 924; 64 channels, 512 trials 0.1 apart,
 // 2048 samples 26, 41; 1024 channels, 512 trials 0.1 apart, 2048 samples 293, 172.
-DedispClocks dedisp_clocks(const sp_plan *const *plans, const int64_t *n_out, int32_t nbeams) {
+DedispClocks dedisp_clocks(const sp_plan *const *plans, const int64_t *n_out, int32_t nbeams, bool alike) {
     DedispClocks c;
     double sums = 0.0, direct = 0.0, direct_items = 0.0, sms = 1.0, sums_most = 0.0, direct_most = 0.0, alone = 0.0;
     for (int32_t b = 0; b < nbeams; ++b) {
-        const sp_plan &p = *plans[b];
-        const double si = (double)sums_items(&p, n_out[b]), di = (double)p.ntiles * (double)dedisp_time_tiles(&p, n_out[b]);
+        const sp_plan &p = *plans[alike ? 0 : b];
+        const int64_t n = n_out[alike ? 0 : b];
+        const double si = (double)sums_items(&p, n), di = (double)p.ntiles * (double)dedisp_time_tiles(&p, n);
         c.sum_items += si;
         direct_items += di;
         sums += si * p.sums_clocks;
@@ -513,10 +514,10 @@ DedispClocks dedisp_clocks(const sp_plan *const *plans, const int64_t *n_out, in
 
 // Whether one launch over these beams goes to the shared-sum kernel: all plans
 // have tables, and the modelled clocks are fewer.
-bool sums_pay(const sp_plan *const *plans, const int64_t *n_out, int32_t nbeams) {
-    for (int32_t b = 0; b < nbeams; ++b)
+bool sums_pay(const sp_plan *const *plans, const int64_t *n_out, int32_t nbeams, bool alike) {
+    for (int32_t b = 0; b < (alike ? 1 : nbeams); ++b)
         if (!plans[b]->d_sums) return false;
-    const DedispClocks c = dedisp_clocks(plans, n_out, nbeams);
+    const DedispClocks c = dedisp_clocks(plans, n_out, nbeams, alike);
     return c.sum_items <= INT32_MAX && c.sums < c.direct;
 }
 

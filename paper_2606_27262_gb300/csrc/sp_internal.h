@@ -198,11 +198,12 @@ int launch_dedisperse_batch(const BatchLaunch &b, cudaStream_t stream, bool pers
 int64_t dedisp_time_tiles(const sp_plan *plan, int64_t n_out);
 // Shared-sum kernel: whether a launch over these beams goes to it
 // (plan_sums.cpp), its tables, its launches.
-bool sums_pay(const sp_plan *const *plans, const int64_t *n_out, int32_t nbeams);
+// (alike: every beam has the first one's plan and length, and only those are read).
+bool sums_pay(const sp_plan *const *plans, const int64_t *n_out, int32_t nbeams, bool alike = false);
 struct DedispClocks {
     double sums = 0.0, direct = 0.0, sum_items = 0.0;
 };
-DedispClocks dedisp_clocks(const sp_plan *const *plans, const int64_t *n_out, int32_t nbeams);
+DedispClocks dedisp_clocks(const sp_plan *const *plans, const int64_t *n_out, int32_t nbeams, bool alike = false);
 void model_items(sp_plan &p, const SumTables &t);
 int build_sum_tables(const sp_plan &p, SumTables &t);
 bool sum_tables_pay(const sp_plan &p, const SumTables &t);

@@ -151,7 +151,6 @@ struct sp_stream {
     // SP_STREAM_ONE_STREAM keeps all of a batch on its launch stream.
     cudaStream_t search_stream = nullptr;
     BatchLaunch geometry{};
-    bool sums = false;  // the batched launches go to the shared-sum kernel
     std::deque<Gulp> pending;
     std::deque<Searched> searched;
     std::deque<Result> results;
@@ -330,7 +329,7 @@ int launch_batch(sp_stream *s, int li) {
             rc = launch_dedisperse(p, sl.d_staged, s->pitch, s->gulp, sl.d_dmt, st, L.d_status);
         }
     } else if (!rc) {
-        const bool sums = s->sums;
+        const bool sums = sums_pay(&p, &s->gulp, n, true);
         const int64_t items = sums ? sums_items(p, s->gulp) : (int64_t)p->ntiles * dedisp_time_tiles(p, s->gulp);
         L.h_begin[0] = 0;
         for (int i = 0; i < n; ++i) {
@@ -701,12 +700,6 @@ extern "C" int sp_stream_create(const sp_plan *plan, int32_t nbeams, int64_t gul
         G.raw_max = plan->raw_max;
         G.smem_bytes = plan->smem_bytes;
         rc = batch_grid(G);
-    }
-    if (!rc) {  // a full batch decides: every batch then runs the same kernel
-        const std::vector<const sp_plan *> plans((size_t)max_batch, plan);
-        const std::vector<int64_t> n_outs((size_t)max_batch, gulp);
-        s->sums = sums_pay(plans.data(), n_outs.data(), max_batch);
-        if (s->sums) rc = sums_configure();
     }
     if (!rc) rc = dedisp_configure(plan);
     if (!rc) rc = sps_configure(h_widths[nw - 1]);
