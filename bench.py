@@ -79,7 +79,8 @@ METRIC = "real-time beams per GB300; dedispersion G(chan·DM·samp)/s vs rooflin
 MAX_SM_MHZ = 2070.0  # GB300 maximum SM clock
 DIRECT_ADDS = "adds of the direct sum; sums that trial DMs share are formed once, so fewer are performed"
 PROFILE_JSON = os.path.join(ROOT, "profiles", "dedisperse_config2_traffic.json")
-DEDISP_SRC = os.path.join(ROOT, "paper_2606_27262_gb300", "csrc", "dedisp_sums.cu")
+DEDISP_SRC = [os.path.join(ROOT, "paper_2606_27262_gb300", "csrc", f)
+              for f in ("dedisp_sums.cu", "plan_sums.cpp", "sp_internal.h")]  # the kernel, its tables, its sizes
 
 
 def parse_args(argv=None):
@@ -211,12 +212,12 @@ def workload(n_out=None):
 
 
 def kernel_source_hash() -> str:
-    return hashlib.sha256(open(DEDISP_SRC, "rb").read()).hexdigest()[:16]
+    return hashlib.sha256(b"".join(open(f, "rb").read() for f in DEDISP_SRC)).hexdigest()[:16]
 
 
 def profiled_traffic(n_out: int):
-    """DRAM bytes per launch of the dedispersion kernel from the committed ncu
-    summary of the full single-beam workload, or None when the kernel source
+    """DRAM bytes per launch of the shared-sum kernel from the committed ncu
+    summary of the full single-beam workload, or None when the kernel's sources
     changed since the capture or another length is being measured."""
     try:
         prof = json.load(open(PROFILE_JSON))
@@ -228,9 +229,9 @@ def profiled_traffic(n_out: int):
 
 
 def profiled_instructions_per_add():
-    """Lane instructions the dedispersion kernel issues per channel x DM x
+    """Lane instructions the shared-sum kernel issues per channel x DM x
     sample add (smsp__inst_executed x 32 / adds of one ncu capture, committed
-    with the traffic summary), or None when the kernel source changed since."""
+    with the traffic summary), or None when the kernel's sources changed since."""
     try:
         prof = json.load(open(PROFILE_JSON))
     except (OSError, ValueError):
@@ -241,7 +242,7 @@ def profiled_instructions_per_add():
 
 
 def issue_roofline(adds_tps: float, nsm: int):
-    """The dedispersion kernel against the SMs' instruction-issue rate (four
+    """The shared-sum kernel against the SMs' instruction-issue rate (four
     schedulers x 32 lanes per SM per clock at the maximum SM clock): lane
     instructions per add (from the committed ncu capture) x adds per second."""
     ipa = profiled_instructions_per_add()
@@ -251,6 +252,18 @@ def issue_roofline(adds_tps: float, nsm: int):
     return {"lane_instructions_per_add": ipa, "achieved": adds_tps * ipa, "peak": peak,
             "unit": "T lane-instructions/s", "frac": adds_tps * ipa / peak,
             "peak_basis": f"{nsm} SMs x 4 schedulers x 32 lanes x {MAX_SM_MHZ:.0f} MHz"}
+
+
+def ran_kernel(sums: bool, plan, achieved: float, nsm: int, n_out: int):
+    """The roofline fields that belong to the dedispersion kernel that ran: the
+    committed captures are the shared-sum kernel's, the tile shape the direct one's."""
+    import paper_2606_27262_gb300 as sp
+    if sums:
+        return {"kernel": "dedisp_sums_kernel", "counts": DIRECT_ADDS, "traffic": profiled_traffic(n_out),
+                "issue": issue_roofline(achieved, nsm)}
+    return {"kernel": "dedisperse_kernel", "traffic": None, "issue": None,
+            "kernel_shape": dict(zip(("dm_tile", "time_tile", "chan_chunk"), sp.shape_info(plan.shape)))
+            | {"shape": plan.shape, "dm_tiles": plan.ntiles}}
 
 
 def cpu_oracle_sample(wl, plan_delays, x, stride: int):
@@ -337,12 +350,12 @@ def run_ours(args):
     clocks.start()
     barrier(world)
     torch.cuda.synchronize(dev)
-    lc0 = sp.launch_count()
+    lc0, sc0 = sp.launch_count(), sp.sums_launch_count()
     t_start.record(stream)
     for k in range(args.steps):
         step(evs[k])
     t_end.record(stream)
-    launches = sp.launch_count() - lc0
+    launches, sums = sp.launch_count() - lc0, sp.sums_launch_count() - sc0
     torch.cuda.synchronize(dev)
     barrier(world)
     clk = clocks.stop()
@@ -407,13 +420,9 @@ def run_ours(args):
         "stage_ms": {"stage_input": tr_ms, "dedisperse": dd_ms, "single_pulse_search": sps_ms},
         "candidates_per_beam": ncand,
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tadd/s",
-                     "frac": achieved / peak, "traffic": profiled_traffic(wl.n_out),
-                     "counts": DIRECT_ADDS, "kernel": "dedisp_sums_kernel",
-                     "kernel_shape": dict(zip(("dm_tile", "time_tile", "chan_chunk"), sp.shape_info(plan.shape)))
-                     | {"shape": plan.shape, "dm_tiles": plan.ntiles},
-                     "issue": issue_roofline(achieved, nsm),
+                     "frac": achieved / peak,
                      "peak_basis": f"{nsm} SMs x {lanes:.1f} measured 32-bit add lanes/SM/clk x "
-                                   f"{MAX_SM_MHZ:.0f} MHz"},
+                                   f"{MAX_SM_MHZ:.0f} MHz"} | ran_kernel(sums > 0, plan, achieved, nsm, wl.n_out),
         "e2e": e2e, "cpu_baseline": cpu, "clocks": clk, "gpu_launches": launches,
         # staging, dedispersion, block sums, block coefficients, streamed
         # boxcar/peaks, tile kernel over the listed tiles, 64-bit pass
@@ -524,13 +533,13 @@ def run_batched(args):
         ev = [torch.cuda.Event(enable_timing=True) for _ in range(steps + 1)]
         barrier(world)
         torch.cuda.synchronize(dev)
-        lc0 = sp.launch_count()
+        lc0, sc0 = sp.launch_count(), sp.sums_launch_count()
         ev[0].record(stream)
         for k in range(steps):
             batch.launch(stream)
             ev[k + 1].record(stream)
         torch.cuda.synchronize(dev)
-        timed_graph.launches = sp.launch_count() - lc0
+        timed_graph.launches, timed_graph.sums = sp.launch_count() - lc0, sp.sums_launch_count() - sc0
         barrier(world)
         return reduce_max(ev[0].elapsed_time(ev[-1]), world, dev) / steps
 
@@ -548,7 +557,7 @@ def run_batched(args):
     clocks = ClockSampler(torch.cuda.current_device())
     clocks.start()
     ms_step = timed_graph(main_mode, args.steps, args.warmup)
-    launches = timed_graph.launches
+    launches, sums = timed_graph.launches, timed_graph.sums // args.steps
     clk = clocks.stop()
     counts = [batch.count(b, stream) for b in range(bw.nbeams)]
     value = world * data_s / (ms_step / 1e3)
@@ -598,8 +607,9 @@ def run_batched(args):
         "candidates": int(sum(counts)),
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tadd/s", "frac": achieved / peak,
                      "traffic": None, "counts": DIRECT_ADDS,
-                     "kernel": "dedisp_sums_items_kernel, or the direct kernel (%s) where sharing does not pay"
-                     % ("dedisperse_items_kernel" if args.batch_mode == "grid" else "dedisperse_batch_kernel"),
+                     "kernel": "dedisp_sums_items_kernel in %d of a step's %d group launches, %s in the others"
+                     % (sums, ngroups,
+                        "dedisperse_items_kernel" if args.batch_mode == "grid" else "dedisperse_batch_kernel"),
                      "kernel_ms_per_step": dd_ms,
                      "peak_basis": f"{nsm} SMs x {lanes:.1f} measured 32-bit add lanes/SM/clk x "
                                    f"{MAX_SM_MHZ:.0f} MHz"},
