@@ -106,7 +106,8 @@ int sp_plan_info(const sp_plan *plan, int32_t *max_delay, int32_t *nchan, int32_
 int sp_plan_status(const sp_plan *plan, int32_t *h_status, int32_t clear);
 /* Test hook of the failure path above (the paper has no counterpart): on
  * the current device, every later dedispersion CTA's first chunk expects
- * extra_bytes (a multiple of 16, <= 1 MiB) more than its bulk copies bring,
+ * extra_bytes (a multiple of 16, <= 1 MiB; 64 KiB at most are used, a barrier
+ * counts 2^20 - 1 pending bytes) more than its bulk copies bring,
  * and every staging wait gives up after wait_limit_cycles SM cycles (>=
  * 1024).  With extra_bytes > 0 the first wait of every CTA runs out, the CTA
  * waits once more (bounded) and leaves, and the status word gets

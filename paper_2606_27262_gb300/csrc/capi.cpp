@@ -105,8 +105,10 @@ extern "C" int sp_debug_staging_fault(int32_t extra_bytes, int64_t wait_limit_cy
     if (extra_bytes < 0 || (extra_bytes & 15) || extra_bytes > (1 << 20) || wait_limit_cycles < 1024 ||
         wait_limit_cycles > (1LL << 40))
         return SP_EINVAL;
-    const int rc = set_staging_fault((uint32_t)extra_bytes, (long long)wait_limit_cycles);
-    if (!rc) set_tc_fault((uint32_t)extra_bytes, (long long)wait_limit_cycles);
+    // With a stage's own bytes inside a barrier's 20 bits of pending transactions.
+    const uint32_t extra = (uint32_t)std::min(extra_bytes, 1 << 16);
+    const int rc = set_staging_fault(extra, (long long)wait_limit_cycles);
+    if (!rc) set_tc_fault(extra, (long long)wait_limit_cycles);
     return rc;
 }
 

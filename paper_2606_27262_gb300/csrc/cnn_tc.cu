@@ -683,7 +683,7 @@ int cnn_conv_dgrad(const GradPair &p, int Nb, int H, int C, int Kp, int32_t *sta
 }
 
 void set_tc_fault(uint32_t extra_bytes, long long wait_limit) {
-    g_extra = std::min(extra_bytes, 1u << 16);  // with a stage's own bytes inside a barrier's 20 bits
+    g_extra = extra_bytes;
     g_limit = wait_limit;
 }
 
