@@ -644,13 +644,62 @@ __global__ void __launch_bounds__(kImg) normalise_kernel(const float *__restrict
 // and, for bins of many samples, by loads whose lanes lie far apart: a window that
 // lies inside the beam in every channel of the subband is read without checks
 // from one address and offsets the CTA shares, and bins of eight samples or more four
-// samples at a time (the ends of a bin masked) where rows are 4-byte aligned.
-// Five candidates of a gulp, 4096 channels, 512 bins: 40 -> 31 us.
-constexpr int kExtractPer = 64;  // channels of a subband that share offsets
+// samples at a time (the ends of a bin masked) where rows are 4-byte aligned.  Windows
+// that leave the beam (all of a wide candidate's in a short gulp) clamp each bin and
+// are read the same way.  4096 channels, 512 bins, one load, check and add per sample
+// against this: 60 candidates of width 1 inside the beam 200 -> 43 us, at its edge
+// 194 -> 151; five of width 64 at the edge 76 -> 42, of width 256 644 -> 265.
+// The widths are read in the parameters' own memory: a copy of them on the stack, which
+// an index makes, costs 25 us of launches of 15360 CTAs.
+constexpr int kExtractPer = 256;  // channels of a subband that share offsets
+
+// A subband of a window that leaves the beam, or of too many channels to share
+// offsets: every channel's samples inside the beam.
+__device__ __forceinline__ void extract_edge(const uint8_t *__restrict__ rows, int64_t pitch, int64_t n_in,
+                                          const int32_t *__restrict__ dl, int per, int64_t first, int dec, int t_in,
+                                          bool words, float *__restrict__ out) {
+    for (int u = threadIdx.x; u < t_in; u += 256) {
+        const int64_t tb = first + (int64_t)u * dec;
+        uint32_t acc = 0;
+        if (dec < 4) {
+#pragma unroll 4
+            for (int k = 0; k < per; ++k) {
+                const int64_t t = tb + __ldg(dl + k);
+#pragma unroll
+                for (int i = 0; i < 3; ++i)
+                    if (i < dec && t + i >= 0 && t + i < n_in) acc += __ldg(rows + k * pitch + t + i);
+            }
+        } else if (dec < 8 || !words) {
+            for (int k = 0; k < per; ++k) {
+                const int64_t t = tb + __ldg(dl + k), lo = max(t, (int64_t)0), hi = min(t + dec, n_in);
+                const uint8_t *r = rows + k * pitch;
+#pragma unroll 4
+                for (int64_t i = lo; i < hi; ++i) acc += __ldg(r + i);
+            }
+        } else {
+#pragma unroll 2
+            for (int k = 0; k < per; ++k) {
+                const int64_t t = tb + __ldg(dl + k), lo = max(t, (int64_t)0), hi = min(t + dec, n_in);
+                if (lo >= hi) continue;
+                const uint8_t *r = rows + k * pitch + lo;
+                const int skip = (int)(reinterpret_cast<uintptr_t>(r) & 3), end = skip + (int)(hi - lo) - 1;
+                const uint32_t *w = reinterpret_cast<const uint32_t *>(r - skip);
+                const int last = end >> 2;
+                const uint32_t tail = 0xFFFFFFFFu >> (8 * (3 - (end & 3)));
+                acc = __dp4a((__ldg(w) & (last ? 0xFFFFFFFFu : tail)) >> (8 * skip), 0x01010101u, acc);
+#pragma unroll 4
+                for (int i = 1; i < last; ++i) acc = __dp4a(__ldg(w + i), 0x01010101u, acc);
+                if (last) acc = __dp4a(__ldg(w + last) & tail, 0x01010101u, acc);
+            }
+        }
+        out[u] = (float)acc;
+    }
+}
 
 __global__ void __launch_bounds__(256) extract_kernel(const uint8_t *__restrict__ xt, int64_t pitch, int64_t n_in,
                                                       int32_t nchan, const int32_t *__restrict__ delays,
-                                                      const sp_cand *__restrict__ cands, ExtractWidths wt, int32_t nsub,
+                                                      const sp_cand *__restrict__ cands,
+                                                      const __grid_constant__ ExtractWidths wt, int32_t nsub,
                                                       int32_t t_in, bool words, float *__restrict__ sub) {
     __shared__ int64_t off_s[kExtractPer];
     const int q = blockIdx.y, s = blockIdx.x;
@@ -699,16 +748,7 @@ __global__ void __launch_bounds__(256) extract_kernel(const uint8_t *__restrict_
         }
         return;
     }
-    for (int u = threadIdx.x; u < t_in; u += 256) {
-        const int64_t tb = first + (int64_t)u * dec;
-        uint32_t acc = 0;
-        for (int k = 0; k < per; ++k) {
-            const uint8_t *row = rows + (int64_t)k * pitch;
-            const int64_t base = tb + __ldg(dl + k), lo = max(base, (int64_t)0), hi = min(base + dec, n_in);
-            for (int64_t t = lo; t < hi; ++t) acc += __ldg(row + t);
-        }
-        out[u] = (float)acc;
-    }
+    extract_edge(rows, pitch, n_in, dl, per, first, dec, t_in, words, out);
 }
 
 int grid_for(int64_t n, int threads = 256) {
