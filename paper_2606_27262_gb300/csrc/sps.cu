@@ -1083,9 +1083,11 @@ __global__ void __launch_bounds__(256, 4) sps_stream_kernel(BoxcarArgs a) {
 // full S/N where the points of such a group lie in several blocks, or one lies
 // outside the beam or has a width that leaves it: those points are scored
 // again that way here.  Used for widths up to 256 and blocks of a multiple of
-// 256 samples (or one), any row alignment; there it is the faster one at every
-// size (501 x 20011, ten widths, odd rows: 111 -> 61 us; 1751 x 16384, nine
-// widths: 225 -> 155 us).
+// 256 samples (or one), any row alignment; there it is the faster one (501 x 20011,
+// ten widths, odd rows: 111 -> 61 us; 1751 x 16384, nine widths: 225 -> 155 us) but for
+// small planes, where the second launch costs more than the streaming saves
+// (map_as_tiles; the whole map of 64 x 300, one to six widths: 25 to 31 us as tiles, 29 to
+// 33 so).
 constexpr int kMapSeg = 16;  // chunks per CTA at most (a segment loads and scans one chunk more)
 constexpr int kMapMaxWidth = 256;
 
@@ -1519,6 +1521,15 @@ int sps_configure(int32_t maxw) {
     return rc;
 }
 
+// Planes whose map the tile kernel computes sooner than the streamed one: up to a tile
+// an SM, with one normalisation block or one width (two to 128 tiles, one to nine
+// widths: by 4 us to -1; several blocks and widths: later, by up to 12 us), and twice
+// as many tiles with both (240 tiles: 2 us; 440: 2 to -2, by the width).
+static bool map_as_tiles(int64_t tiles, int64_t nblk, int nw, int nsm) {
+    if (tiles <= nsm) return nblk == 1 || nw == 1;
+    return tiles <= 2 * (int64_t)nsm && nblk == 1 && nw == 1;
+}
+
 int launch_sps(const SpsArgs &a, cudaStream_t stream) {
     WidthList wl;
     for (int k = 0; k < SP_MAX_WIDTHS; ++k) wl.w[k] = k < a.nw ? a.widths[k] : 0;
@@ -1588,7 +1599,8 @@ int launch_sps(const SpsArgs &a, cudaStream_t stream) {
         return SP_ECUDA;
     }
     if (map) {
-        if (maxw <= kMapMaxWidth && (a.nblk == 1 || a.norm_block % kBxT == 0) && ntx <= INT32_MAX) {
+        if (maxw <= kMapMaxWidth && (a.nblk == 1 || a.norm_block % kBxT == 0) && ntx <= INT32_MAX &&
+            !map_as_tiles(ntx * ngroups, a.nblk, a.nw, nsm)) {
             // The segment length of the least time: whole waves of two CTAs per SM, each as long as its chunks and
             // about 3/4 of one more to load and scan the first (501 x 20011: 2 chunks 72 us, 10 chunks 62 us).
             int64_t seg = 1, least = INT64_MAX;
