@@ -135,9 +135,9 @@ int sp_compute_delays(const double *freqs_mhz, int32_t nchan, double tsamp_s,
  * counterpart in the paper (whose kernels come from its dedispersion
  * library); it exists because the best tile shape depends on the channel
  * count, the DM list and the GPU.  A plan of shape 0 also holds the tables of
- * the shared-sum kernel where its trials share enough of their sums (and memory
- * allows), and its
- * launches then run that kernel (the same transform, bit for bit).
+ * the shared-sum kernel where its trials share enough of their sums and memory
+ * allows, and its launches run that kernel where it is modelled to be the faster
+ * one (the same transform, bit for bit).
  * sp_dedisp_shape_info: the triple of a shape (out pointers may be NULL).
  * sp_plan_create_shaped: sp_plan_create for a given shape, or for
  *   SP_SHAPE_AUTO: the shape sp_autotune_dedisperse picks with

@@ -227,7 +227,7 @@ struct ConvOut {
 // map's element strides); the padding is the zero fill.  Bound by latency and
 // L2 (the layers read 9/4 of their input).  Both branches at batch 256, layers
 // 1-4: 305, 149, 104, 67 us with patches gathered by two warps (the last by
-// im2col) -> 140, 61, 52, 35; at batch 5: 21, 30, 49, 38 -> 8, 9, 10, 19.
+// im2col) -> 140, 61, 52, 35; at batch 5: 21, 30, 49, 38 -> 8, 9, 7, 11.
 // NB: CTAs that share a tile's output channels, 2 C / NB each.
 template <int C, int NB>
 struct FwdShape {

@@ -10,10 +10,10 @@
 // sample; here a DM reads two bytes per GROUP and sample, and the rows cost
 // about a channel's loads each.
 //
-// What bounds it: the SM's shared-memory data pipe (82 % busy on the 0.1 steps
-// of the 5751-trial, 4096-channel plan: 43 % of its wavefronts are the DMs'
+// What bounds it: the SM's shared-memory data pipe (78 % busy over the
+// 5751-trial, 4096-channel plan: 43 % of its wavefronts are the DMs'
 // reads of the rows, the rest makes the rows) and instruction issue (67 %).
-// That plan over 131072 samples: 133 ms with the direct kernel, 46 ms here;
+// That plan over 131072 samples: 133 ms with the direct kernel, 45.5 ms here;
 // 64 x 1024 because a tile's 65536 packed sums take half the registers, and
 // rows serve more DMs, and waste less on the spread of their delays, the larger
 // the tile is (modelled: 128 x 512 18 % slower, 32 x 2048 12 %, two CTAs of
@@ -472,7 +472,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 dedisp_sums_kernel(const uint8_t *__restrict__ xt, int64_t pitch, int64_t n_out, int32_t *__restrict__ out,
                    const SumTablesDev *__restrict__ tables, int64_t ntime, int32_t *__restrict__ status) {
     extern __shared__ __align__(128) uint8_t smem[];
-        int tile;
+    int tile;
     int64_t tq;
     raster((int64_t)blockIdx.x, tables->ntiles, ntime, tile, tq);
     sums_tile(smem, tables, xt, pitch, n_out, out, tile, tq * kSumTime, status);
@@ -492,7 +492,7 @@ dedisp_sums_items_kernel(const BatchBeamDev *__restrict__ beams, const int64_t *
         else hi = mid - 1;
     }
     const BatchBeamDev bm = beams[lo];
-        int tile;
+    int tile;
     int64_t tq;
     raster(item - __ldg(item_begin + lo), bm.sums->ntiles, (int64_t)bm.ntime, tile, tq);
     sums_tile(smem, bm.sums, bm.xt, bm.pitch, bm.n_out, bm.out, tile, tq * kSumTime, status);
