@@ -1,4 +1,4 @@
-// Host checks of plan.cpp and plan_sums.cpp without a GPU: the driver links
+// Host checks of plan.cpp and plan_sums.cpp without a GPU: the program links
 // them with a CUDA runtime of its own (host memory; allocation number g_refuse
 // fails) and is built with the undefined-behaviour sanitizer.
 #include <cstdio>
